@@ -238,6 +238,16 @@ int check_system(const md_surface& s, const md_params& p, SysDev& S, std::string
   }
   S.gconst_df = df_split(S.gconst);
   S.R_df = df_split(s.kind == MD_SURF_TORUS ? s.p[0] : 0.0);
+  if (s.kind == MD_SURF_GAUSSIAN_BUMP) {
+    S.bumpA_df = df_split(s.p[0]);
+    S.half_iw2_df = df_split(0.5 / (s.p[1] * s.p[1]));
+  }
+  if (s.kind == MD_SURF_THYLAKOID) {
+    const double Rb = s.p[0], Lx = s.p[1], Rc = s.p[2], Lb = s.p[3], xf = 0.5 * Lb + Rc;
+    S.thyl_df = {df_split(0.5 * Lb), df_split(xf), df_split(xf + Rc), df_split(xf + Rc + Lx),
+                 df_split(xf + 2.0 * Rc + Lx), df_split(0.5 * Lx), df_split(0.5 * Lx + Rc), df_split(Rb + Rc),
+                 df_split((Rb + Rc) * (Rb + Rc)), df_split(-Rc * Rc), df_split(-Rb * Rb)};
+  }
   S.dt_df = df_split(S.dt);
   S.half_dt_df = df_split(S.half_dt);
   for (int t = 0; t < kMaxTypes; ++t) {
@@ -248,6 +258,7 @@ int check_system(const md_surface& s, const md_params& p, SysDev& S, std::string
     S.box_lo[d] = p.box_lo[d];
     S.box_len[d] = p.box_hi[d] - p.box_lo[d];
     S.inv_box_len[d] = S.box_len[d] > 0.0 ? 1.0 / S.box_len[d] : 0.0;
+    S.box_len_df[d] = df_split(S.box_len[d]);
     S.periodic[d] = p.periodic[d] ? 1 : 0;
   }
   S.bpm = p.beads_per_mol;
@@ -839,6 +850,8 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
   A.pair_queue = 1;
   A.list_warp = 32;
   A.store_noise = 1;
+  for (const SysDev& S : h->sys)
+    if (S.kind == kBump || S.kind == kThylakoid) A.composed = 1;
   A.ntypes = prms[0].ntypes;
   A.spin_limit = kDefaultSpinLimit;
   A.rec_cell = (!h->excl && cell_total < (uint64_t(1) << 29)) ? 1 : 0;

@@ -408,6 +408,12 @@ __device__ __forceinline__ bool finite3(double a, double b, double c) {
   return isfinite(a) && isfinite(b) && isfinite(c);
 }
 
+}  // namespace surfmd
+
+#include "position.cuh"
+
+namespace surfmd {
+
 // ---------------------------------------------------------------------------
 // meta / set state / restore
 // ---------------------------------------------------------------------------
@@ -2508,28 +2514,6 @@ __device__ __forceinline__ void surf_n(const SysDev& S, const GEval& e, double& 
   }
 }
 
-// Float32 gradient from the pieces surf_g kept (offsets in float64).
-__device__ __forceinline__ void surf_n_f(const SysDev& S, const GEval& e, float& nx, float& ny, float& nz) {
-  switch (S.kind) {
-    case kThylakoid: nx = d2f_rn(e.ux); ny = d2f_rn(e.uy); nz = d2f_rn(e.uz); break;
-    case kPlane: nx = S.p_f[0]; ny = S.p_f[1]; nz = S.p_f[2]; break;
-    case kTorus: {
-      const float q = d2f_rn(e.q);
-      nx = q * d2f_rn(e.ux); ny = q * d2f_rn(e.uy); nz = 2.f * d2f_rn(e.uz);
-      break;
-    }
-    case kBump: {
-      const float q = d2f_rn(e.q);
-      nx = q * d2f_rn(e.ux); ny = q * d2f_rn(e.uy); nz = 1.f;
-      break;
-    }
-    case kSphere:
-    case kEllipsoid:
-    case kCylinder: nx = 2.f * d2f_rn(e.ux); ny = 2.f * d2f_rn(e.uy); nz = 2.f * d2f_rn(e.uz); break;
-    default: nx = ny = nz = 0.f;
-  }
-}
-
 template <typename R> struct Force3 { R x, y, z; };
 
 template <typename R> __device__ __forceinline__ Force3<R> load_f3(const void* f, int64_t i);
@@ -2787,211 +2771,10 @@ __device__ __forceinline__ void integrate_particle_fp64(const DevArrays& A, int6
 // float32 pipe) from the float64 masters, which are read and written as
 // float64.
 //
-// Algorithm 1 in multiplier form. The momentum half at x^k and the kick of the
-// position half give q = p^{k-1/2} + dt F^k - s n0, s = n0.(p^{k-1/2} + h F^k)
-// / |n0|^2, n0 = grad g(x^k); the position half then subtracts h lambda n0.
-// Both corrections lie along n0, so with q0 = p^{k-1/2} + dt F^k,
-// y = x^k + (dt/m) q0 and mu = (dt/m)(s + h lambda):
-//   x^{k+1} = y - mu n0,   p^{k+1/2} = q0 - (m/dt) mu n0,   g(y - mu n0) = 0.
-// The projection s only sets where the Newton iteration starts (mu_0 =
-// (dt/m) s, formed in float32), not its root. On the first step after a state
-// is set there is no momentum half: q0 = p^k + h F^k, mu_0 = 0.
-//
-// The position-half Newton update lambda += g / (a n1.n0) of Algorithm 1 reads
-// mu += g(x(mu)) / (n1.n0) on the line x(mu) = y - mu n0 (mu = a lambda,
-// n1 = grad g(x(mu)); n1 = n0 in the frozen-normal variant). g along the line
-// is evaluated in double-float: for the quadrics (plane, sphere, ellipsoid,
-// cylinder) by its exact line form g(y) - b mu + c mu^2 (b = grad g(y).n0,
-// c = n0.H n0 / 2, H the constant Hessian), for the torus at the point
-// itself; the Newton denominator n1.n0 is float32 (it scales the step, not
-// the root). The other surfaces (Gaussian bump, thylakoid) take the float64
-// form below. The full-step momentum p^k is not needed by the step and is
-// formed only on read-out, with the float64 normal.
+// The position half of a constrained particle is position.cuh; a free particle
+// drifts in float64.
 // ---------------------------------------------------------------------------
-
-// Any surface by re-evaluation of g at x(mu) in float64 (Gaussian bump,
-// thylakoid composite).
-struct LineGeneric {
-  const SysDev* S;
-  double yx, yy, yz, n0x, n0y, n0z;
-  float n0xf, n0yf, n0zf;
-  Piece q;  // the held piece of a composite surface
-  GEval e;
-  __device__ __forceinline__ double g(double mu) {
-    const double px = fma(-mu, n0x, yx), py = fma(-mu, n0y, yy), pz = fma(-mu, n0z, yz);
-    e = S->kind == kThylakoid ? thyl_geval(*S, q, px, py, pz) : surf_g(*S, px, py, pz);
-    return e.g;
-  }
-  __device__ __forceinline__ float n1n0(float) const {
-    float n1x, n1y, n1z;
-    surf_n_f(*S, e, n1x, n1y, n1z);
-    return fmaf(n1x, n0xf, fmaf(n1y, n0yf, n1z * n0zf));
-  }
-};
-
-// Newton on the line from mu_0: stop when |g| < tol_n (tolerance times |n0|,
-// with a 1% margin for |n(x^{k+1})| != |n0|) or when an update falls under the
-// round-off floor (4 ulp of the position).
-template <class L>
-__device__ __forceinline__ bool newton_line(L& line, int max_newton, bool frozen, float nnf, float tol_n,
-                                            float floor_mu, float mu0f, double& mu) {
-  mu = f2d(mu0f);
-  double g = line.g(mu);
-  for (int it = 0; it <= max_newton; ++it) {
-    const float gf = d2f_rn(g);
-    if (fabsf(gf) < tol_n) return true;
-    if (it == max_newton) break;
-    const float rden = __frcp_rn(frozen ? nnf : line.n1n0(d2f_rn(mu)));
-    mu = fma(g, f2d(rden), mu);
-    if (it > 0 && fabsf(gf * rden) <= floor_mu) return true;
-    g = line.g(mu);
-  }
-  return false;
-}
-
-__device__ __forceinline__ bool df_surface(int32_t kind) {
-  return kind == kPlane || kind == kSphere || kind == kEllipsoid || kind == kCylinder || kind == kTorus;
-}
-
-// g on the line x(mu) = y - mu n0 in double-float, D = y - c, N = n0.
-// Quadrics: the line form g(y) - b mu + c mu^2. Torus: g at the point, with
-// rho - R, rho and x(mu) - c kept in float32 for the Newton denominator.
-struct DFTorusEval {
-  float ttf, rhof, e0, e1, e2;
-  __device__ __forceinline__ DF g(const SysDev& S, const DF D[3], const DF N[3], DF mu) {
-    DF E[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) E[d] = df_sub(D[d], df_mul(N[d], mu));
-    const DF rho = df_sqrt(df_add(df_mul(E[0], E[0]), df_mul(E[1], E[1])));
-    const DF t = df_sub(rho, S.R_df);
-    ttf = t.h;
-    rhof = rho.h;
-    e0 = E[0].h; e1 = E[1].h; e2 = E[2].h;
-    return df_add(df_add(df_mul(t, t), df_mul(E[2], E[2])), S.gconst_df);
-  }
-  // n1.n0 = 2 (rho - R)/rho (e_xy . n0_xy) + 2 e_z n0_z
-  __device__ __forceinline__ float n1n0(const DF N[3]) const {
-    return 2.f * ttf / rhof * fmaf(e0, N[0].h, e1 * N[1].h) + 2.f * e2 * N[2].h;
-  }
-};
-
-// Position half of a constrained particle on a plane, sphere, ellipsoid,
-// cylinder or torus (multiplier form above): reads x^k, p^{k-1/2} (or p^k on
-// the first step) and the combined force F, returns x^{k+1} and p^{k+1/2}.
-// y - c, n0 = grad g(x^k) and g in double-float. For the quadrics the Newton
-// iteration runs on the line form first in float32, which brings mu to
-// float32 resolution (about 1e-7 of mu n0, itself about 1e-4 sigma), then
-// continues in double-float until g, evaluated in double-float, meets the
-// tolerance; the torus iterates in double-float throughout. x^{k+1} =
-// c + (y - c) - mu n0 is rounded once to float64; p^{k+1/2} = p + (kick F -
-// (m/dt) mu n0) adds a float32 increment to the float64 momentum.
-__device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, int mode, const double xv[3],
-                                                 const double pv[3], const float pf[3], const float F[3],
-                                                 uint32_t* status, double xo[3], double qo[3]) {
-  DF D[3], N[3];
-  const DF kick = mode ? S.dt_df : S.half_dt_df;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const DF q0 = df_add(df_from(pv[d]), df_mul_f(kick, F[d]));  // q0 = p + kick F
-    const DF X = df_from(xv[d]);
-    N[d] = S.c_zero ? X : df_sub(X, S.c_df[d]);                   // x - c (n0 below)
-    D[d] = df_add(N[d], df_mul(S.dtm_df[ty], q0));               // y - c = x - c + (dt/m) q0
-  }
-  DF gy{0.f, 0.f}, b{0.f, 0.f};
-  float c = 0.f;
-  switch (S.kind) {
-    case kPlane:
-#pragma unroll
-      for (int d = 0; d < 3; ++d) N[d] = S.pn_df[d];
-      gy = df_dot3(S.pn_df, D);
-      b = df_dot3(S.pn_df, N);
-      break;
-    case kEllipsoid: {
-      DF U[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        N[d] = df_scale2(df_mul(N[d], S.inv_a2_df[d]), 2.f);
-        U[d] = df_mul(D[d], S.inv_a2_df[d]);
-        c = fmaf(N[d].h * N[d].h, S.inv_a2_df[d].h, c);
-      }
-      gy = df_add_f(df_dot3(U, D), -1.f);
-      b = df_scale2(df_dot3(U, N), 2.f);
-      break;
-    }
-    case kTorus: {
-      const DF rho = df_sqrt(df_add(df_mul(N[0], N[0]), df_mul(N[1], N[1])));
-      const DF q = df_scale2(df_div(df_sub(rho, S.R_df), rho), 2.f);  // 2 (rho - R) / rho
-      N[0] = df_mul(q, N[0]);
-      N[1] = df_mul(q, N[1]);
-      N[2] = df_scale2(N[2], 2.f);
-      break;
-    }
-    default: {  // sphere; cylinder without the axis component (n0 has none)
-      DF M[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const bool off = S.kind == kCylinder && d == S.axis;
-        M[d] = off ? DF{0.f, 0.f} : D[d];
-        N[d] = off ? DF{0.f, 0.f} : df_scale2(N[d], 2.f);
-      }
-      gy = df_add(df_dot3(M, M), S.gconst_df);
-      b = df_scale2(df_dot3(M, N), 2.f);
-      break;
-    }
-  }
-  const float nnf = fmaf(N[0].h, N[0].h, fmaf(N[1].h, N[1].h, N[2].h * N[2].h));
-  if (S.kind == kSphere || S.kind == kCylinder) c = nnf;
-  float mu0 = 0.f;
-  if (mode) {  // mu_0 = (dt/m) n0.(p + h F) / |n0|^2
-    float sp = 0.f;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) sp = fmaf(N[d].h, fmaf(S.half_dt_f, F[d], pf[d]), sp);
-    mu0 = S.dtm_f[ty] * sp / nnf;
-  }
-  const float tol_n = 0.99f * S.tol_f * sqrtf(nnf);
-  // round-off floor: an update below 4 units of the double-float resolution of the position
-  const float dmax = fmaxf(fabsf(D[0].h), fmaxf(fabsf(D[1].h), fabsf(D[2].h)));
-  const float floor_mu = 4.f * 0x1p-47f * dmax / fmaxf(fabsf(N[0].h), fmaxf(fabsf(N[1].h), fabsf(N[2].h)));
-  const bool torus = S.kind == kTorus;
-  int it = 0;
-  if (!torus) {  // float32 Newton on the line form g(y) - b mu + c mu^2
-    for (; it < S.max_newton; ++it) {
-      const float gf = fmaf(fmaf(c, mu0, -b.h), mu0, gy.h);
-      if (fabsf(gf) < 0.5f * tol_n) break;
-      const float dmu = gf * __frcp_rn(S.frozen ? nnf : fmaf(-2.f * mu0, c, b.h));
-      mu0 += dmu;
-      if (fabsf(dmu) <= 0x1p-22f * fabsf(mu0)) {
-        ++it;
-        break;
-      }
-    }
-  }
-  DFTorusEval T;
-  DF mu = {mu0, 0.f};
-  DF g = torus ? T.g(S, D, N, mu) : df_add_f(df_sub(gy, df_mul(b, mu)), c * mu.h * mu.h);
-  bool ok = false;
-  for (;; ++it) {
-    if (fabsf(g.h) < tol_n) { ok = true; break; }
-    if (it >= S.max_newton) break;
-    const float den = S.frozen ? nnf : (torus ? T.n1n0(N) : fmaf(-2.f * mu.h, c, b.h));
-    const float dmu = g.h * __frcp_rn(den);
-    mu = df_add_f(mu, dmu);
-    if (it > 0 && fabsf(dmu) <= floor_mu) { ok = true; break; }
-    g = torus ? T.g(S, D, N, mu) : df_add_f(df_sub(gy, df_mul(b, mu)), c * mu.h * mu.h);
-  }
-  if (!ok) flag(status, kFlagRattle);
-  const float kickf = mode ? S.dt_df.h : S.half_dt_df.h;
-  const float cm = mu.h * S.inv_dtm_df[ty].h;  // (m/dt) mu
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    DF e = df_sub(D[d], df_mul(N[d], mu));  // (y - c) - mu n0
-    if (!S.c_zero) e = df_add(e, S.c_df[d]);
-    xo[d] = df_to(e);
-    qo[d] = pv[d] + f2d(fmaf(kickf, F[d], -cm * N[d].h));  // p + kick F - (m/dt) mu n0
-  }
-}
-
-template <class Bin>
+template <bool COMPOSED, class Bin>
 __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int64_t i, Force3<float> fr_in,
                                                          unsigned long long k, int mode, const Bin& bin,
                                                          float4* xi = nullptr, bool xi_prev = false) {
@@ -3001,59 +2784,23 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
   const uint32_t ty = meta_type(m);
   const double x = A.x[i], y = A.x[n + i], z = A.x[2 * n + i];
   const double px = A.ph[i], py = A.ph[n + i], pz = A.ph[2 * n + i];
-  const float pxf = d2f_rn(px), pyf = d2f_rn(py), pzf = d2f_rn(pz);
+  const DF P[3] = {df_from(px), df_from(py), df_from(pz)};  // the high parts are p rounded to float32
   Force3<float> F =
-      combine<float>(S, A.types, ty, (uint32_t)(i - S.first), k, mode, fr_in, pxf, pyf, pzf, xi, xi_prev);
+      combine<float>(S, A.types, ty, (uint32_t)(i - S.first), k, mode, fr_in, P[0].h, P[1].h, P[2].h, xi, xi_prev);
   if (S.kind == kXY2D) F.z = 0.f;  // 2D plane: no z update
   double xn, yn, zn, qx, qy, qz;
-  if (meta_con(m) && df_surface(S.kind)) {
+  if (meta_con(m)) {
     const double xv[3] = {x, y, z}, pv[3] = {px, py, pz};
-    const float pf[3] = {pxf, pyf, pzf}, Fv[3] = {F.x, F.y, F.z};
+    const float Fv[3] = {F.x, F.y, F.z};
     double xo[3], qo[3];
-    position_half_df(S, ty, mode, xv, pv, pf, Fv, A.status, xo, qo);
+    position_half_df<COMPOSED>(S, ty, mode, xv, pv, P, Fv, A.status, xo, qo);
     xn = xo[0]; yn = xo[1]; zn = xo[2];
     qx = qo[0]; qy = qo[1]; qz = qo[2];
   } else {
     const double kick = mode ? S.dt : S.half_dt;
     qx = fma(kick, f2d(F.x), px); qy = fma(kick, f2d(F.y), py); qz = fma(kick, f2d(F.z), pz);
     const double dtm = S.dtm[ty];
-    const double yx = fma(dtm, qx, x), yy = fma(dtm, qy, y), yz = fma(dtm, qz, z);
-    xn = yx; yn = yy; zn = yz;
-    if (meta_con(m)) {  // Gaussian bump, thylakoid: float64 line
-      const float xf = d2f_rn(x), yf = d2f_rn(y), zf = d2f_rn(z);
-      float n0xf, n0yf, n0zf;
-      Piece q0{};
-      if (S.kind == kThylakoid) {  // composite surface: the piece at x^k, held for the solve
-        q0 = thyl_select(S, x, y, z);
-        double gx, gy, gz;
-        thyl_eval(S, q0, x, y, z, gx, gy, gz);
-        n0xf = d2f_rn(gx); n0yf = d2f_rn(gy); n0zf = d2f_rn(gz);
-      } else {
-        surf_grad_f(S, xf - S.c_f[0], yf - S.c_f[1], zf - S.c_f[2], n0xf, n0yf, n0zf);
-      }
-      const float nnf = fmaf(n0xf, n0xf, fmaf(n0yf, n0yf, n0zf * n0zf));
-      float mu0f = 0.f;
-      if (mode) {  // mu_0 = (dt/m) n0.(p + h F) / |n0|^2
-        const float hf = S.half_dt_f;
-        const float sp =
-            fmaf(n0xf, fmaf(hf, F.x, pxf), fmaf(n0yf, fmaf(hf, F.y, pyf), n0zf * fmaf(hf, F.z, pzf)));
-        mu0f = S.dtm_f[ty] * sp / nnf;
-      }
-      const float tol_n = 0.99f * S.tol_f * sqrtf(nnf);
-      const float floor_mu = 4.f * (float)DBL_EPSILON * fmaxf(fabsf(xf), fmaxf(fabsf(yf), fabsf(zf))) /
-                             fmaxf(fabsf(n0xf), fmaxf(fabsf(n0yf), fabsf(n0zf)));
-      LineGeneric L;
-      L.S = &S;
-      L.yx = yx; L.yy = yy; L.yz = yz;
-      L.n0x = f2d(n0xf); L.n0y = f2d(n0yf); L.n0z = f2d(n0zf);
-      L.n0xf = n0xf; L.n0yf = n0yf; L.n0zf = n0zf;
-      L.q = q0;
-      double mu;
-      if (!newton_line(L, S.max_newton, S.frozen, nnf, tol_n, floor_mu, mu0f, mu)) flag(A.status, kFlagRattle);
-      xn = fma(-mu, L.n0x, yx); yn = fma(-mu, L.n0y, yy); zn = fma(-mu, L.n0z, yz);
-      const double c = mu * S.inv_dtm[ty];
-      qx = fma(-c, L.n0x, qx); qy = fma(-c, L.n0y, qy); qz = fma(-c, L.n0z, qz);
-    }
+    xn = fma(dtm, qx, x); yn = fma(dtm, qy, y); zn = fma(dtm, qz, z);
   }
   if (!(finite_bits(xn) && finite_bits(yn) && finite_bits(zn) && finite_bits(qx) && finite_bits(qy) &&
         finite_bits(qz)))
@@ -3069,7 +2816,9 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
   }
 }
 
-template <typename R>
+// COMPOSED (mixed path): some system's surface is a Gaussian bump or a
+// thylakoid composite (DevArrays::composed).
+template <typename R, bool COMPOSED>
 __global__ void __launch_bounds__(256, 4) k_integrate_nl(DevArrays A) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
@@ -3080,13 +2829,13 @@ __global__ void __launch_bounds__(256, 4) k_integrate_nl(DevArrays A) {
     const bool store = A.noise && A.store_noise;
     float4* xi = store ? A.noise + i : nullptr;
     const bool xi_prev = store && k > 0ull && *A.noise_k == k - 1ull;  // ~0: none stored
-    integrate_particle_mixed(A, i, load_f3<float>(A.f, i), k, mode, bin, xi, xi_prev);
+    integrate_particle_mixed<COMPOSED>(A, i, load_f3<float>(A.f, i), k, mode, bin, xi, xi_prev);
   } else {
     integrate_particle_fp64(A, i, load_f3<double>(A.f, i), k, mode, bin);
   }
 }
 
-template <typename R, bool BIN>
+template <typename R, bool BIN, bool COMPOSED>
 __global__ void __launch_bounds__(256, 4) k_integrate(DevArrays A) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
@@ -3094,7 +2843,7 @@ __global__ void __launch_bounds__(256, 4) k_integrate(DevArrays A) {
   const int mode = *A.mode;
   using Bin = typename std::conditional<BIN, GlobalBin, NoBin>::type;
   const Bin bin(A);
-  if constexpr (sizeof(R) == 4) integrate_particle_mixed(A, i, load_f3<float>(A.f, i), k, mode, bin);
+  if constexpr (sizeof(R) == 4) integrate_particle_mixed<COMPOSED>(A, i, load_f3<float>(A.f, i), k, mode, bin);
   else integrate_particle_fp64(A, i, load_f3<double>(A.f, i), k, mode, bin);
 }
 
@@ -3278,7 +3027,7 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 2) k_resident(DevArrays A
       const int mode = j == 0 ? mode0 : 1;
       for (uint32_t li = tid; li < n; li += bd) {
         const Force3<R> f{s_fx[li], s_fy[li], s_fz[li]};
-        if constexpr (sizeof(R) == 4) integrate_particle_mixed(A, first + li, f, k, mode, bin);
+        if constexpr (sizeof(R) == 4) integrate_particle_mixed<true>(A, first + li, f, k, mode, bin);
         else integrate_particle_fp64(A, first + li, f, k, mode, bin);
       }
       __syncthreads();
@@ -3804,14 +3553,18 @@ cudaError_t launch_integrate(const DevArrays& A, int precision, int has_pairs, c
   const int b = block_for(A.n);
   const unsigned g = grid_for(A.n, b);
   if (A.nl_dirty && has_pairs) {
-    if (precision == 0) k_integrate_nl<double><<<g, b, 0, st>>>(A);
-    else k_integrate_nl<float><<<g, b, 0, st>>>(A);
+    if (precision == 0) k_integrate_nl<double, false><<<g, b, 0, st>>>(A);
+    else if (A.composed) k_integrate_nl<float, true><<<g, b, 0, st>>>(A);
+    else k_integrate_nl<float, false><<<g, b, 0, st>>>(A);
   } else if (precision == 0) {
-    if (has_pairs) k_integrate<double, true><<<g, b, 0, st>>>(A);
-    else k_integrate<double, false><<<g, b, 0, st>>>(A);
+    if (has_pairs) k_integrate<double, true, false><<<g, b, 0, st>>>(A);
+    else k_integrate<double, false, false><<<g, b, 0, st>>>(A);
+  } else if (has_pairs) {
+    if (A.composed) k_integrate<float, true, true><<<g, b, 0, st>>>(A);
+    else k_integrate<float, true, false><<<g, b, 0, st>>>(A);
   } else {
-    if (has_pairs) k_integrate<float, true><<<g, b, 0, st>>>(A);
-    else k_integrate<float, false><<<g, b, 0, st>>>(A);
+    if (A.composed) k_integrate<float, false, true><<<g, b, 0, st>>>(A);
+    else k_integrate<float, false, false><<<g, b, 0, st>>>(A);
   }
   return cudaGetLastError();
 }

@@ -35,6 +35,15 @@ struct DF {
   float h, l;
 };
 
+// Lengths of the thylakoid composite about its centre, in the quadrant x, y >=
+// 0 (double-float): the bridge's half length, the faces towards the bridge
+// (xf) and away from it (face_hi), the inner square's x range and half side,
+// the side planes, the connector's ring radius R_b + R_c and its square, -R_c^2
+// and -R_b^2.
+struct ThylDF {
+  DF half_lb, xf, inner, inner_hi, face_hi, half_lx, side_y, rout, rout2, m_rc2, m_rb2;
+};
+
 // One system's constants as the kernels read them.
 struct SysDev {
   // surface g(x) = 0
@@ -59,6 +68,9 @@ struct SysDev {
   // double-float copies for the mixed path's position half
   DF c_df[3], inv_a2_df[3], pn_df[3];  // centre, ellipsoid 1/a_d^2, plane normal
   DF gconst_df, R_df;                  // constant term of g; torus R
+  DF bumpA_df, half_iw2_df;            // Gaussian bump: A and 1 / (2 w^2)
+  DF box_len_df[3];
+  ThylDF thyl_df;
   DF dt_df, half_dt_df;
   DF dtm_df[kMaxTypes], inv_dtm_df[kMaxTypes];  // dt/m and m/dt per type
   int32_t c_zero;            // 1: the centre is the origin
@@ -162,6 +174,7 @@ struct DevArrays {
   int32_t pair_lanes;   // lanes per particle in the pair kernel (1, 2, 4 or 8)
   int32_t pair_tile;    // 0, or particles per warp (8, 16, 32) of the cell-tiled pair kernel (needs hashed == 0)
   int32_t pair_queue;   // mixed path with the Verlet list: 1 = warp-queued list walk (k_pair_nlq), 0 = per-lane walk
+  int32_t composed;     // 1: some system's surface is a Gaussian bump or a thylakoid composite
   int32_t list_warp;    // particles per warp of the warp-queued list walk (8, 16 or 32)
   // Verlet neighbour list (nl_dirty == null: off). Built from the cell list
   // with every pair within r_c + skin; between builds the integrator moves
