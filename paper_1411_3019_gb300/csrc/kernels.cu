@@ -966,8 +966,8 @@ __device__ __forceinline__ void lj_term(const PairTab<R>& tab, uint32_t qt, R r2
 // double-float product. The Lennard-Jones factor of Eq. S1 is written as
 //   f(r)/r = 24 eps s6 (2 s6 - 1) / r^2 = 24 eps sigma^6 (2 sigma^6 - r^6) / (r^6 r^6 r^2),
 // with 2 sigma^6 - r^6 formed from the double-float r^6 (exact cancellation
-// near the WCA cutoff) and 1/r^6, 1/r^2 from a float32 reciprocal corrected
-// by the low part. Only float32 products of well-conditioned factors remain,
+// near the WCA cutoff) and 1/r^6, 1/r^2 as float32 reciprocals of the
+// double-floats (df_rcp_f). Only float32 products of well-conditioned factors remain,
 // so the pair force carries a few float32 roundings relative to itself,
 // while a float32 r^2 (relative error 2^-24) would move it by up to 22 of
 // them near contact (d ln f / d ln r = -22 at r = 1.03 sigma) and by up to
@@ -1001,16 +1001,14 @@ __device__ __forceinline__ bool acc_pair(const PairTab<float>& tab, uint32_t qt,
   const DF r2 = df_fast_sum(s2.h, lo);
   const DF rc2 = tab.acc.rc2[qt];
   if (!(__fadd_rn(__fsub_rn(r2.h, rc2.h), __fsub_rn(r2.l, rc2.l)) < 0.f)) return false;  // r >= r_c
-  const float iR0 = __frcp_rn(r2.h);
-  const float iR = __fmaf_rn(-__fmul_rn(r2.l, iR0), iR0, iR0);  // 1 / r^2
+  const float iR = df_rcp_f(r2);  // 1 / r^2
   DF r4 = df_two_prod(r2.h, r2.h);
   r4.l = __fmaf_rn(2.f * r2.h, r2.l, r4.l);
   DF r6 = df_two_prod(r4.h, r2.h);
   r6.l = __fmaf_rn(r4.h, r2.l, __fmaf_rn(r4.l, r2.h, r6.l));
   const DF s = tab.acc.s6x2[qt];
   const float num = __fadd_rn(__fsub_rn(s.h, r6.h), __fsub_rn(s.l, r6.l));  // 2 sigma^6 - r^6
-  const float iq0 = __frcp_rn(r6.h);
-  const float iq = __fmaf_rn(-__fmul_rn(r6.l, iq0), iq0, iq0);  // 1 / r^6
+  const float iq = df_rcp_f(r6);  // 1 / r^6
   t.fr = tab.acc.c24[qt] * num * (iq * iq) * iR;
   const float s6 = tab.acc.s6[qt] * iq;
   t.v = tab.acc.c4[qt] * iq * (s6 - 1.f) - tab.shift[qt];
