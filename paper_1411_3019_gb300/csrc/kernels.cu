@@ -936,20 +936,26 @@ template <> __device__ __forceinline__ double rsq<double>(double v) { return nr_
 // force -phi'(r) + phi'(r_c) vanishes at r_c. Adds the force on i (along the
 // displacement d = x_i - x_j) and half the pair energy.
 template <typename R>
-__device__ __forceinline__ void lj_term(const PairTab<R>& tab, uint32_t qt, R r2, R ddx, R ddy, R ddz, R& fx,
-                                        R& fy, R& fz, R& u) {
+__device__ __forceinline__ void lj_factor(const PairTab<R>& tab, uint32_t qt, R r2, R& fr, R& v) {
   const R inv_r2 = rcp<R>(r2);
   const R s2 = tab.sig2[qt] * inv_r2;
   const R s6 = s2 * s2 * s2;
   const R e = tab.eps[qt];
-  R fr = (R)24 * e * s6 * ((R)2 * s6 - (R)1) * inv_r2;
-  R v = (R)4 * e * s6 * (s6 - (R)1) - tab.shift[qt];
+  fr = (R)24 * e * s6 * ((R)2 * s6 - (R)1) * inv_r2;
+  v = (R)4 * e * s6 * (s6 - (R)1) - tab.shift[qt];
   const R lin = tab.lin[qt];
   if (lin != (R)0) {
     const R inv_r = rsq<R>(r2);
     fr += lin * inv_r;
     v -= (r2 * inv_r - tab.rc[qt]) * lin;
   }
+}
+
+template <typename R>
+__device__ __forceinline__ void lj_term(const PairTab<R>& tab, uint32_t qt, R r2, R ddx, R ddy, R ddz, R& fx,
+                                        R& fy, R& fz, R& u) {
+  R fr, v;
+  lj_factor<R>(tab, qt, r2, fr, v);
   fx += fr * ddx; fy += fr * ddy; fz += fr * ddz;
   u += (R)0.5 * v;
 }
@@ -1375,6 +1381,38 @@ template <typename R> struct GlobalCells {
   __device__ __forceinline__ uint32_t bucket(uint32_t cell) const { return bucket_of(cell, hashed, log_t); }
 };
 
+// Tangent-slab pruning of a surface-bound particle's stencil (no free particle
+// in its system): a cell farther from the tangent plane than a neighbour can
+// be holds none.
+struct SlabPrune {
+  float nx, ny, nz, reach, on;
+  bool active;
+  __device__ __forceinline__ SlabPrune(const DevArrays& A, const SysDev& S, uint32_t sid, uint32_t m, const int c[3],
+                                       float ox, float oy, float oz) {
+    nx = ny = nz = reach = on = 0.f;
+    active = S.slab > 0.f && meta_con(m) && A.sys_free[sid] == 0;
+    if (!active) return;
+    const float rx = S.grid_lo_f[0] + ((float)c[0] + 0.5f) * S.cs_f[0] + ox - S.c_f[0];
+    const float ry = S.grid_lo_f[1] + ((float)c[1] + 0.5f) * S.cs_f[1] + oy - S.c_f[1];
+    const float rz = S.grid_lo_f[2] + ((float)c[2] + 0.5f) * S.cs_f[2] + oz - S.c_f[2];
+    surf_grad_f(S, rx, ry, rz, nx, ny, nz);
+    const float nn = fmaf(nx, nx, fmaf(ny, ny, nz * nz));
+    if (nn > 0.f) {
+      const float inv = rsqrtf(nn);
+      nx *= inv; ny *= inv; nz *= inv;
+      reach = 0.5f * (S.cs_f[0] * fabsf(nx) + S.cs_f[1] * fabsf(ny) + S.cs_f[2] * fabsf(nz)) + S.slab;
+      on = nx * ox + ny * oy + nz * oz;
+    } else {
+      active = false;
+    }
+  }
+  __device__ __forceinline__ bool skips(const SysDev& S, int dx, int dy, int dz) const {
+    if (!active) return false;
+    const float dist = nx * (float)dx * S.cs_f[0] + ny * (float)dy * S.cs_f[1] + nz * (float)dz * S.cs_f[2] - on;
+    return fabsf(dist) > reach;
+  }
+};
+
 template <typename R, bool BONDS, bool WALLS, bool EXCL, class Cells>
 __device__ __forceinline__ uint32_t pair_slot(const DevArrays& A, const Cells& C, const PairTab<R>& tab, uint32_t s,
                                               R& fx, R& fy, R& fz, R& u) {
@@ -1394,25 +1432,7 @@ __device__ __forceinline__ uint32_t pair_slot(const DevArrays& A, const Cells& C
   const R csx = sizeof(R) == 4 ? (R)S.cs_f[0] : (R)S.cs[0];
   const R csy = sizeof(R) == 4 ? (R)S.cs_f[1] : (R)S.cs[1];
   const R csz = sizeof(R) == 4 ? (R)S.cs_f[2] : (R)S.cs[2];
-  // tangent-slab pruning
-  bool prune = S.slab > 0.f && meta_con(m) && A.sys_free[sid] == 0;
-  float nhx = 0.f, nhy = 0.f, nhz = 0.f, reach = 0.f, on = 0.f;
-  if (prune) {
-    const float ox = (float)ri.x, oy = (float)ri.y, oz = (float)ri.z;
-    const float rx = S.grid_lo_f[0] + ((float)c[0] + 0.5f) * S.cs_f[0] + ox - S.c_f[0];
-    const float ry = S.grid_lo_f[1] + ((float)c[1] + 0.5f) * S.cs_f[1] + oy - S.c_f[1];
-    const float rz = S.grid_lo_f[2] + ((float)c[2] + 0.5f) * S.cs_f[2] + oz - S.c_f[2];
-    surf_grad_f(S, rx, ry, rz, nhx, nhy, nhz);
-    const float nn = fmaf(nhx, nhx, fmaf(nhy, nhy, nhz * nhz));
-    if (nn > 0.f) {
-      const float inv = rsqrtf(nn);
-      nhx *= inv; nhy *= inv; nhz *= inv;
-      reach = 0.5f * (S.cs_f[0] * fabsf(nhx) + S.cs_f[1] * fabsf(nhy) + S.cs_f[2] * fabsf(nhz)) + S.slab;
-      on = nhx * ox + nhy * oy + nhz * oz;
-    } else {
-      prune = false;
-    }
-  }
+  const SlabPrune P(A, S, sid, m, c, (float)ri.x, (float)ri.y, (float)ri.z);
   fx = 0; fy = 0; fz = 0; u = 0;
   for (int dz = -1; dz <= 1; ++dz) {
     int z = c[2] + dz;
@@ -1438,11 +1458,7 @@ __device__ __forceinline__ uint32_t pair_slot(const DevArrays& A, const Cells& C
           if (!S.periodic[0]) continue;
           x = (x + S.nc[0]) % S.nc[0];
         }
-        if (prune) {
-          const float dist = nhx * (float)dx * S.cs_f[0] + nhy * (float)dy * S.cs_f[1] +
-                             nhz * (float)dz * S.cs_f[2] - on;
-          if (fabsf(dist) > reach) continue;
-        }
+        if (P.skips(S, dx, dy, dz)) continue;
         nb[q] = cell_id(S, x, y, z);
         const uint32_t b = C.bucket(nb[q]);
         t0[q] = C.start(b);
@@ -1481,6 +1497,187 @@ __global__ void __launch_bounds__(256) k_pair_row(DevArrays A) {
   R fx, fy, fz, u;
   const uint32_t tag = pair_slot<R, BONDS, WALLS, EXCL>(A, GlobalCells<R>(A), tab, s, fx, fy, fz, u);
   store_f<R>(A.f, tag, fx, fy, fz, u);
+}
+
+// Cell list every step, one warp per particle: the same pairs, terms and order
+// of sums as k_pair_row (pair_slot), with 32 lanes over the particle's
+// candidates in place of one. Lane q < 27 reads the bounds of stencil cell q, a
+// prefix sum over the lanes makes the candidates one sequence in stencil order,
+// and 32 of them at a time are loaded and screened. Those that pass are queued
+// in order (ballot); 32 queued ones are evaluated on all lanes, and lanes 0..3
+// then add the force components and the energy of the terms in queue order:
+// every sum has k_pair_row's terms in k_pair_row's order (a candidate outside
+// the cutoff adds exact zeros), so the bits are the same.
+// What bounds k_pair_row on a small system is latency: one lane's serial walk
+// of 27 cells, 23 to 30 us however few the particles (float64: 43 to 124). Pair
+// kernel time, row -> warp: 1,000 particles on a sphere 29.6 -> 9.2 us (float64
+// 64.9 -> 12.5), four surfaces of 500 with r_c = 2.5 in float64 123.9 -> 17.5,
+// a liquid of 4,096 with r_c = 2.5 250.9 -> 21.4.
+constexpr int kPairWarps = 4;
+
+template <typename R> struct PairWarp {
+  static constexpr bool kLow = sizeof(R) == 4;  // the displacement's low part (double-float terms)
+  R fr[32];
+  R d[4][32];               // displacement x, y, z and the pair energy
+  R dl[kLow ? 4 : 1][32];   // low parts (0 for the energy)
+  uint32_t qt[64];          // queue: candidate slot
+  uint8_t qc[64];           // queue: its stencil cell
+};
+
+template <typename R, bool BONDS, bool WALLS, bool EXCL>
+__global__ void __launch_bounds__(kPairWarps * 32) k_pair_warp(DevArrays A) {
+  using Rec = typename RecT<R>::T;
+  constexpr unsigned kAll = 0xffffffffu;
+  __shared__ PairTab<R> tab;
+  __shared__ __align__(16) PairWarp<R> buf[kPairWarps];
+  load_tab<R>(tab, A.types);
+  __syncthreads();
+  const int lane = (int)(threadIdx.x & 31u);
+  PairWarp<R>& W = buf[threadIdx.x >> 5];
+  const Rec* __restrict__ rec = reinterpret_cast<const Rec*>(A.rec);
+  const float4* __restrict__ lo = A.rec_lo;
+  const uint32_t s = blockIdx.x * (uint32_t)kPairWarps + (threadIdx.x >> 5);
+  if (s >= (uint32_t)A.n) return;
+  const uint32_t tag = A.stag[s];
+  const uint32_t cell = A.scell[s];
+  const Rec ri = rec[s];
+  const float4 li = rec_lo_at<R>(lo, s);
+  const uint32_t bi = RecT<R>::bits(ri);
+  const uint32_t ti = bi & 7u, moli = bi >> 3;
+  const uint32_t m = A.meta[tag];
+  const uint32_t sid = meta_sys(m);
+  const SysDev& S = A.sys[sid];
+  int c[3];
+  cell_decode(S, cell, c[0], c[1], c[2]);
+  const R csx = sizeof(R) == 4 ? (R)S.cs_f[0] : (R)S.cs[0];
+  const R csy = sizeof(R) == 4 ? (R)S.cs_f[1] : (R)S.cs[1];
+  const R csz = sizeof(R) == 4 ? (R)S.cs_f[2] : (R)S.cs[2];
+  // bounds of stencil cell q = lane < 27
+  uint32_t nb = 0u, t0 = 0u, cl = 0u;
+  if (lane < 27) {
+    const int dx = lane % 3 - 1, dy = lane / 3 % 3 - 1, dz = lane / 9 - 1;
+    int x = c[0] + dx, y = c[1] + dy, z = c[2] + dz;
+    bool have = true;
+    if (x < 0 || x >= S.nc[0]) { have = have && S.periodic[0]; x = (x + S.nc[0]) % S.nc[0]; }
+    if (y < 0 || y >= S.nc[1]) { have = have && S.periodic[1]; y = (y + S.nc[1]) % S.nc[1]; }
+    if (z < 0 || z >= S.nc[2]) { have = have && S.periodic[2]; z = (z + S.nc[2]) % S.nc[2]; }
+    const SlabPrune P(A, S, sid, m, c, (float)ri.x, (float)ri.y, (float)ri.z);
+    if (have && !P.skips(S, dx, dy, dz)) {
+      nb = cell_id(S, x, y, z);
+      const uint32_t b = bucket_of(nb, A.hashed, A.log_t);
+      t0 = A.start[b];
+      cl = A.start[b + 1] - t0;
+    }
+  }
+  __syncwarp();
+  uint32_t pre = cl;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(kAll, pre, o);
+    if (lane >= o) pre += v;
+  }
+  const uint32_t total = __shfl_sync(kAll, pre, 31);
+  pre -= cl;
+  const uint32_t base = t0 - pre;  // candidate j of this cell is slot base + j
+  uint32_t qn = 0u;
+  R acc = (R)0;  // lanes 0..3: force x, y, z and energy
+  // evaluates the first k <= 32 queued candidates, then adds their terms
+  auto drain = [&](uint32_t k) {
+    __syncwarp();
+    R fr = (R)0, v = (R)0, d[3] = {(R)0, (R)0, (R)0}, dl[3] = {(R)0, (R)0, (R)0};
+    if ((uint32_t)lane < k) {
+      const uint32_t t = W.qt[lane], code = W.qc[lane];
+      const Rec rj = rec[t];
+      const int dz = (int)(code / 9u) - 1, dy = (int)(code / 3u % 3u) - 1, dx = (int)(code % 3u) - 1;
+      const R shx = (R)dx * csx, shy = (R)dy * csy, shz = (R)dz * csz;
+      const uint32_t qt = ti * kMaxTypes + (RecT<R>::bits(rj) & 7u);
+      if constexpr (sizeof(R) == 4) {
+        AccTerm T;
+        if (acc_pair(tab, qt, ri, li, rj, lo[t], shx, shy, shz, T)) {
+          fr = T.fr; v = T.v;
+          d[0] = T.dx.h; d[1] = T.dy.h; d[2] = T.dz.h;
+          dl[0] = T.dx.l; dl[1] = T.dy.l; dl[2] = T.dz.l;
+        }
+      } else {
+        const R ddx = ri.x - rj.x - shx, ddy = ri.y - rj.y - shy, ddz = ri.z - rj.z - shz;
+        const R r2 = ddx * ddx + ddy * ddy + ddz * ddz;
+        if (r2 < tab.rc2[qt]) {
+          lj_factor<R>(tab, qt, r2, fr, v);
+          d[0] = ddx; d[1] = ddy; d[2] = ddz;
+        }
+      }
+    }
+    W.fr[lane] = fr;
+    W.d[3][lane] = v;
+    if (sizeof(R) == 4) W.dl[sizeof(R) == 4 ? 3 : 0][lane] = (R)0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      W.d[a][lane] = d[a];
+      if (sizeof(R) == 4) W.dl[sizeof(R) == 4 ? a : 0][lane] = dl[a];
+    }
+    __syncwarp();
+    if (lane < 4) {
+      for (uint32_t j = 0; j < k; j += 4) {  // padded by the zeros of idle lanes
+#pragma unroll
+        for (uint32_t i = j; i < j + 4; ++i) {
+          const R f = lane == 3 ? (R)0.5 : W.fr[i];
+          if constexpr (sizeof(R) == 4) acc = __fmaf_rn(f, W.d[lane][i], __fmaf_rn(f, W.dl[lane][i], acc));
+          else acc = fma(f, W.d[lane][i], acc);
+        }
+      }
+    }
+    __syncwarp();
+  };
+  for (uint32_t c0 = 0; c0 < total; c0 += 32u) {
+    const uint32_t j = c0 + (uint32_t)lane;
+    // stencil cell of candidate j: the last lane whose prefix is <= j (lanes 27.. hold the total)
+    uint32_t q = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1) {
+      const uint32_t cand = q + (uint32_t)step;
+      const uint32_t pc = __shfl_sync(kAll, pre, (int)cand);
+      if (pc <= j) q = cand;
+    }
+    const uint32_t t = __shfl_sync(kAll, base, (int)q) + j;
+    const uint32_t nbq = __shfl_sync(kAll, nb, (int)q);
+    bool hit = j < total && t != s;
+    if (hit) {
+      const Rec rj = rec[t];
+      const uint32_t bj = RecT<R>::bits(rj);
+      const uint32_t cj = A.rec_cell ? bj >> 3 : (A.hashed ? A.scell[t] : nbq);
+      const int dz = (int)(q / 9u) - 1, dy = (int)(q / 3u % 3u) - 1, dx = (int)(q % 3u) - 1;
+      const R ddx = ri.x - rj.x - (R)dx * csx, ddy = ri.y - rj.y - (R)dy * csy, ddz = ri.z - rj.z - (R)dz * csz;
+      const R r2 = ddx * ddx + ddy * ddy + ddz * ddz;
+      const uint32_t qt = ti * kMaxTypes + (bj & 7u);
+      // (another cell of the same hash bucket drops out; a superset of the pairs inside the cutoff passes)
+      hit = cj == nbq && !(EXCL && (bj >> 3) == moli);
+      if constexpr (sizeof(R) == 4) hit = hit && r2 < tab.acc.rc2m[qt];
+      else hit = hit && r2 <= tab.rc2[qt] * (1.0 + 0x1p-40);
+    }
+    const uint32_t mask = __ballot_sync(kAll, hit);
+    if (hit) {
+      const uint32_t at = qn + (uint32_t)__popc(mask & ((1u << lane) - 1u));
+      W.qt[at] = t;
+      W.qc[at] = (uint8_t)q;
+    }
+    qn += (uint32_t)__popc(mask);
+    if (qn >= 32u) {
+      drain(32u);
+      qn -= 32u;
+      if ((uint32_t)lane < qn) {  // the rest moves to the front
+        W.qt[lane] = W.qt[32 + lane];
+        W.qc[lane] = W.qc[32 + lane];
+      }
+    }
+  }
+  if (qn) drain(qn);
+  const R fx = __shfl_sync(kAll, acc, 0), fy = __shfl_sync(kAll, acc, 1), fz = __shfl_sync(kAll, acc, 2),
+          u = __shfl_sync(kAll, acc, 3);
+  if (lane == 0) {
+    R f[4] = {fx, fy, fz, u};
+    if (BONDS || WALLS) bonded_terms<R>(A, S, tag, m, BONDS, WALLS, f[0], f[1], f[2], f[3]);
+    store_f<R>(A.f, tag, f[0], f[1], f[2], f[3]);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -3432,6 +3629,31 @@ static void pair_dispatch_row(const DevArrays& A, int bonds, int walls, int excl
   }
 }
 
+// A system of at most this many particles takes k_pair_warp instead of
+// k_pair_row (same bits). Above, a warp per particle is more work than the row
+// kernel's latency hides: on the sparsest workload (a 2D plane, 9 cells of one
+// particle each) the two cross near 12,000 particles on the mixed path (20,000:
+// row 15.7, warp 21.1 us) and 8,000 in float64 (20,000: 29.3 and 47.3 us); on
+// the others later (sphere, 16,000: 29.3 and 19.1 us; float64 57.6 and 42.2).
+template <typename R> constexpr int64_t warp_pair_max() { return sizeof(R) == 4 ? 12288 : 8192; }
+
+template <typename R>
+static void pair_dispatch_warp(const DevArrays& A, int bonds, int walls, int excl, cudaStream_t st) {
+  const int b = kPairWarps * 32;
+  const unsigned g = grid_for(A.n, kPairWarps);
+  const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
+  switch (key) {
+    case 0: k_pair_warp<R, false, false, false><<<g, b, 0, st>>>(A); break;
+    case 1: k_pair_warp<R, false, false, true><<<g, b, 0, st>>>(A); break;
+    case 2: k_pair_warp<R, false, true, false><<<g, b, 0, st>>>(A); break;
+    case 3: k_pair_warp<R, false, true, true><<<g, b, 0, st>>>(A); break;
+    case 4: k_pair_warp<R, true, false, false><<<g, b, 0, st>>>(A); break;
+    case 5: k_pair_warp<R, true, false, true><<<g, b, 0, st>>>(A); break;
+    case 6: k_pair_warp<R, true, true, false><<<g, b, 0, st>>>(A); break;
+    default: k_pair_warp<R, true, true, true><<<g, b, 0, st>>>(A); break;
+  }
+}
+
 template <typename R, int L>
 static void pair_dispatch_l(const DevArrays& A, int bonds, int walls, int excl, cudaStream_t st) {
   const int b = block_for((int64_t)A.n * L);
@@ -3477,7 +3699,9 @@ static void pair_dispatch(const DevArrays& A, int bonds, int walls, int excl, in
     case 2: pair_dispatch_l<R, 2>(A, bonds, walls, excl, st); break;
     case 4: pair_dispatch_l<R, 4>(A, bonds, walls, excl, st); break;
     case 8: pair_dispatch_l<R, 8>(A, bonds, walls, excl, st); break;
-    default: pair_dispatch_row<R>(A, bonds, walls, excl, st); break;
+    default:
+      if (A.n <= warp_pair_max<R>()) pair_dispatch_warp<R>(A, bonds, walls, excl, st);
+      else pair_dispatch_row<R>(A, bonds, walls, excl, st);
   }
 }
 
