@@ -279,6 +279,13 @@ int check_system(const md_surface& s, const md_params& p, SysDev& S, std::string
   for (int d = 0; d < 3; ++d) S.wall_center[d] = p.wall_center[d];
   S.wall_sigma = p.wall_sigma;
   S.wall_rc = std::pow(2.0, 1.0 / 6.0) * p.wall_sigma;
+  S.bond_r02_df = df_split(S.bond_r0 * S.bond_r0);
+  S.angle_sin0_df = df_split(S.angle_sin0);
+  S.angle_cos0_df = df_split(S.angle_cos0);
+  S.wall_lo_df = df_split(S.wall_lo);
+  S.wall_hi_df = df_split(S.wall_hi);
+  for (int d = 0; d < 3; ++d) S.wall_center_df[d] = df_split(S.wall_center[d]);
+  S.wall_r2_df = df_split(S.wall_radius * S.wall_radius);
   S.seed_lo = (uint32_t)(p.seed & 0xffffffffu);
   S.replica = p.replica;
   return MD_OK;
@@ -356,6 +363,7 @@ void fill_types(const md_params& p, TypeTable& T) {
       T.lin[a][b] = lin;
       T.rc[a][b] = rc;
       T.bond_r0_mix[a][b] = std::pow(2.0, 1.0 / 6.0) * sg / 2.0;
+      T.bond_r02_mix_df[a][b] = df_split(T.bond_r0_mix[a][b] * T.bond_r0_mix[a][b]);
       T.eps_f[a][b] = (float)ep;
       T.sig2_f[a][b] = (float)(sg * sg);
       T.rc2_f[a][b] = (float)(rc * rc);

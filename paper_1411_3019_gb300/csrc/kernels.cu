@@ -147,27 +147,43 @@ __device__ __forceinline__ double f2d(float v) {
 }
 
 // float64 -> double-float on the integer pipe: h = v rounded to float32 (as
-// d2f_rn), l = the remainder v - h. The remainder is an integer number rem of
-// units 2^(E-1075) of v's binade (E = v's biased exponent; rem is the low
-// bits of the fraction field minus the rounding, |rem| <= 2^28); l keeps its
-// leading bits, rem >> 6 (<= 2^22 in magnitude, so converted exactly by the
-// 1.5 * 2^23 bias), times 2^(E-1069). h + l = v within 2^-46 |v|. Outside
-// 2^-80 <= |v| < 2^128 (zero, tiny or huge values) the split takes one
-// float64 subtraction instead.
-__device__ __forceinline__ DF df_from(double v) {
+// d2f_rn) and l = the rest, for v = 0 or 2^-80 <= |v| < 2^128 (ok says so).
+// The fraction is cut after 23 bits (t) and the cut bits, an integer of units
+// 2^(E-1075) of v's binade (E = v's biased exponent), keep their leading 23:
+// rest >> 6 < 2^23, exact in float32 by the 2^23 bias, times 2^(E-1069); one
+// fast_two_sum then moves the rounding of h into place. h + l = v within
+// 2^-46 |v|.
+__device__ __forceinline__ DF df_from_fast(double v, bool& ok) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-  const uint32_t e = (hi >> 20) & 0x7ffu;
-  if (e - 943u < 208u) {  // biased exponent in [943, 1150]
-    uint32_t up, rest;
-    const uint32_t q = d2f_bits_rn(hi, lo, up, rest);
-    const int32_t rem = (int32_t)rest - (int32_t)(up << 29);  // dropped bits, less 2^29 if rounded up
-    const float k = __fsub_rn(__int_as_float(0x4B400000 + (rem >> 6)), 12582912.0f);
-    const float l = __fmul_rn(k, __uint_as_float((e - 942u) << 23));
-    const uint32_t sign = hi & 0x80000000u;
-    return {__uint_as_float(sign | q), sign ? -l : l};
-  }
+  const uint32_t e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+  const bool zero = ((hi << 1) | lo) == 0u;
+  ok = ok && (e - 943u < 208u || zero);
+  const uint32_t t = __funnelshift_l(lo, hi & 0x7fffffffu, 3) - 0xC0000000u;  // 896 << 23 modulo 2^32
+  const float k = __fsub_rn(__uint_as_float(0x4B000000u | ((lo >> 6) & 0x7fffffu)), 8388608.0f);
+  const DF r = df_fast_sum(__uint_as_float(sign | t), __fmul_rn(k, __uint_as_float(sign | ((e - 942u) << 23))));
+  return zero ? DF{__uint_as_float(hi), 0.f} : r;
+}
+// The same for any v: one float64 subtraction for tiny or huge values.
+__device__ __forceinline__ DF df_from_slow(double v) {
   const float h = d2f_rn(v);
   return {h, d2f_rn(v - f2d(h))};
+}
+__device__ __forceinline__ DF df_from(double v) {
+  bool ok = true;
+  DF r = df_from_fast(v, ok);
+  if (!ok) r = df_from_slow(v);
+  return r;
+}
+// Three values at once, with one branch for the rare ones (a branch for each
+// value keeps the three splits from overlapping).
+__device__ __forceinline__ void df_from3(const double v[3], DF o[3]) {
+  bool ok = true;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) o[d] = df_from_fast(v[d], ok);
+  if (!ok) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) o[d] = df_from_slow(v[d]);
+  }
 }
 __device__ __forceinline__ double df_to(DF a) { return f2d(a.h) + f2d(a.l); }
 
@@ -1135,31 +1151,54 @@ __device__ __forceinline__ double bend_term(const SysDev& S, const double* xa, c
   return S.angle_k * dth * dth;
 }
 
-// The bend term on the mixed path. Float64 forms what cancels: u, w, the
+// Position of particle i as double-floats, and the minimum-image difference of
+// two positions of one system.
+struct DF3 {
+  DF v[3];
+};
+__device__ __forceinline__ DF3 load_df3(const DevArrays& A, int64_t i) {
+  const double x[3] = {A.x[i], A.x[A.n + i], A.x[2 * A.n + i]};
+  DF3 r;
+  df_from3(x, r.v);
+  return r;
+}
+__device__ __forceinline__ DF3 df_image_diff(const SysDev& S, const DF3& a, const DF3& b) {
+  DF3 d;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    d.v[k] = df_sub(a.v[k], b.v[k]);
+    if (S.periodic[k]) {
+      const float q = rintf(d.v[k].h / S.box_len_df[k].h);
+      if (q != 0.f) d.v[k] = df_sub(d.v[k], df_mul_f(S.box_len_df[k], q));
+    }
+  }
+  return d;
+}
+
+// The bend term on the mixed path. Double-float forms what cancels: u, w, the
 // cross product C = u x w, u.w, |C| and the two arguments of
 // dth = atan2(sin(theta - theta0), cos(theta - theta0)) (both scaled by
 // |u||w|), so dth keeps float32's relative precision even near theta0 and near
 // a straight chain. Float32 does the rest, with the brackets written without
 // cancellation: w - (u.w / |u|^2) u = (C x u) / |u|^2 and
-// u - (u.w / |w|^2) w = (w x C) / |w|^2.
-__device__ __forceinline__ float bend_term_f(const SysDev& S, const double* xa, const double* xm, const double* xb,
-                                             int which, float f[3]) {
-  double u[3], w[3];
-  min_image_diff(S, xa, xm, u);
-  min_image_diff(S, xb, xm, w);
-  const double C[3] = {u[1] * w[2] - u[2] * w[1], u[2] * w[0] - u[0] * w[2], u[0] * w[1] - u[1] * w[0]};
-  const double uw = fma(u[0], w[0], fma(u[1], w[1], u[2] * w[2]));
-  const double CC = fma(C[0], C[0], fma(C[1], C[1], C[2] * C[2]));
-  const double sn = CC > 0.0 ? CC * nr_rsqrt(CC) : 0.0;  // |u||w| sin(theta)
-  const float dth = atan2f(d2f_rn(fma(sn, S.angle_cos0, -uw * S.angle_sin0)),
-                           d2f_rn(fma(uw, S.angle_cos0, sn * S.angle_sin0)));  // theta - theta0
-  const float uf[3] = {d2f_rn(u[0]), d2f_rn(u[1]), d2f_rn(u[2])};
-  const float wf[3] = {d2f_rn(w[0]), d2f_rn(w[1]), d2f_rn(w[2])};
-  const float Cf[3] = {d2f_rn(C[0]), d2f_rn(C[1]), d2f_rn(C[2])};
+// u - (u.w / |w|^2) w = (w x C) / |w|^2. (In float64, at two operations per SM
+// and clock, the bend pass of 1,024 capsids of 240 beads took 54 us.)
+__device__ __forceinline__ float bend_term_f(const SysDev& S, const DF3& xa, const DF3& xm, const DF3& xb, int which,
+                                             float f[3]) {
+  const DF3 u = df_image_diff(S, xa, xm), w = df_image_diff(S, xb, xm);
+  const DF C[3] = {df_det2(u.v[1], w.v[2], u.v[2], w.v[1]), df_det2(u.v[2], w.v[0], u.v[0], w.v[2]),
+                   df_det2(u.v[0], w.v[1], u.v[1], w.v[0])};
+  const DF uw = df_dot3(u.v, w.v), CC = df_dot3(C, C);
+  const DF sn = CC.h > 0.f ? df_sqrt(CC) : DF{0.f, 0.f};  // |u||w| sin(theta)
+  const float dth = atan2f(df_det2(sn, S.angle_cos0_df, uw, S.angle_sin0_df).h,
+                           df_add(df_mul(uw, S.angle_cos0_df), df_mul(sn, S.angle_sin0_df)).h);  // theta - theta0
+  const float uf[3] = {u.v[0].h, u.v[1].h, u.v[2].h};
+  const float wf[3] = {w.v[0].h, w.v[1].h, w.v[2].h};
+  const float Cf[3] = {C[0].h, C[1].h, C[2].h};
   const float uu = fmaf(uf[0], uf[0], fmaf(uf[1], uf[1], uf[2] * uf[2]));
   const float ww = fmaf(wf[0], wf[0], fmaf(wf[1], wf[1], wf[2] * wf[2]));
   const float inv_norm = rsqrtf(uu * ww);
-  const float sth = d2f_rn(sn) * inv_norm;
+  const float sth = sn.h * inv_norm;
   const float k = (float)S.angle_k;
   const float ratio = sth > 0.f ? __fdividef(2.f * k * dth, sth) : 0.f;
   const float ga = __fdividef(ratio * inv_norm, uu), gb = __fdividef(ratio * inv_norm, ww);
@@ -1173,7 +1212,7 @@ __device__ __forceinline__ float bend_term_f(const SysDev& S, const double* xa, 
 }
 
 // Bend angles of particle `tag` (float64 on the float64 path, float32 after
-// float64 bond vectors on the mixed path): the force on it from every angle
+// double-float bond vectors on the mixed path): the force on it from every angle
 // of three consecutive beads of its chain that contains it, and its energy
 // share (a third of each angle). Kept out of the pair kernels (its registers
 // would lower their occupancy): k_bend and a phase of the resident engine add
@@ -1188,12 +1227,16 @@ __device__ __forceinline__ void bend_on(const DevArrays& A, const SysDev& S, int
   for (int64_t mid = pid - 1; mid <= pid + 1; ++mid) {  // middle bead of each angle containing the particle
     if (mid < 1 || mid + 1 >= S.n || mid % B == 0 || mid % B == B - 1) continue;
     const int64_t gm = S.first + mid;
-    const double xa[3] = {A.x[gm - 1], A.x[n + gm - 1], A.x[2 * n + gm - 1]};
-    const double xm[3] = {A.x[gm], A.x[n + gm], A.x[2 * n + gm]};
-    const double xb[3] = {A.x[gm + 1], A.x[n + gm + 1], A.x[2 * n + gm + 1]};
     R fa[3];
-    if constexpr (sizeof(R) == 4) v += bend_term_f(S, xa, xm, xb, (int)(pid - mid + 1), fa) * (1.f / 3.f);
-    else v += bend_term(S, xa, xm, xb, (int)(pid - mid + 1), fa) / 3.0;
+    if constexpr (sizeof(R) == 4) {
+      v += bend_term_f(S, load_df3(A, gm - 1), load_df3(A, gm), load_df3(A, gm + 1), (int)(pid - mid + 1), fa) *
+           (1.f / 3.f);
+    } else {
+      const double xa[3] = {A.x[gm - 1], A.x[n + gm - 1], A.x[2 * n + gm - 1]};
+      const double xm[3] = {A.x[gm], A.x[n + gm], A.x[2 * n + gm]};
+      const double xb[3] = {A.x[gm + 1], A.x[n + gm + 1], A.x[2 * n + gm + 1]};
+      v += bend_term(S, xa, xm, xb, (int)(pid - mid + 1), fa) / 3.0;
+    }
     f[0] += fa[0]; f[1] += fa[1]; f[2] += fa[2];
   }
 }
@@ -1205,17 +1248,16 @@ __device__ __forceinline__ bool has_bends(const SysDev& S) { return S.bpm > 2 &&
 // and the wall V_w (two z planes, or a sphere about wall_center) on
 // unconstrained particles. The particle's energy share is half of each bond
 // and all of its wall term. The float64 path works in float64 throughout.
-// The mixed path forms in float64 only what cancels: the displacement, r^2
+// The mixed path forms in double-float what cancels: the displacement, r^2
 // and r^2 - r0^2 (the stretch r - r0 is small against r), the wall distance,
 // or r^2 - R_w^2 for the spherical wall; then r - r0 = (r^2 - r0^2) / (r + r0)
 // and the rest in float32, where the rounding of r enters denominators only.
 __device__ __forceinline__ void bonded_terms_f(const DevArrays& A, const SysDev& S, uint32_t tag, uint32_t m,
                                                bool bonds, bool walls, float& fx, float& fy, float& fz,
                                                float& u) {
-  const int64_t n = A.n;
-  const double xi[3] = {A.x[tag], A.x[n + tag], A.x[2 * n + tag]};
   float bx = 0.f, by = 0.f, bz = 0.f, bu = 0.f;
   if (bonds && S.bpm > 1) {
+    const DF3 xi = load_df3(A, tag);
     const int64_t pid = (int64_t)tag - S.first;
     const int64_t B = S.bpm;
     const float k = (float)S.bond_k;
@@ -1229,29 +1271,31 @@ __device__ __forceinline__ void bonded_terms_f(const DevArrays& A, const SysDev&
         if (pid % B == B - 1 || pid + 1 >= S.n) continue;
         j = (int64_t)tag + 1;
       }
-      const double xj[3] = {A.x[j], A.x[n + j], A.x[2 * n + j]};
-      double d[3];
-      min_image_diff(S, xi, xj, d);
-      const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
-      const double r0 = S.bond_mix ? A.types->bond_r0_mix[meta_type(m)][meta_type(A.meta[j])] : S.bond_r0;
-      const float q = d2f_rn(fma(-r0, r0, r2));  // r^2 - r0^2
-      const float r2f = d2f_rn(r2);
+      const DF3 d = df_image_diff(S, xi, load_df3(A, j));
+      const DF r2 = df_dot3(d.v, d.v);
+      const uint32_t ti = meta_type(m), tj = S.bond_mix ? meta_type(A.meta[j]) : 0u;
+      const DF r02 = S.bond_mix ? A.types->bond_r02_mix_df[ti][tj] : S.bond_r02_df;
+      const float r0 = S.bond_mix ? (float)A.types->bond_r0_mix[ti][tj] : (float)S.bond_r0;
+      const float q = df_sub(r2, r02).h;  // r^2 - r0^2
+      const float r2f = r2.h;
       const float ir = rsqrtf(r2f);
-      const float dr = __fdividef(q, fmaf(r2f, ir, (float)r0));  // r - r0
+      const float dr = __fdividef(q, fmaf(r2f, ir, r0));  // r - r0
       const float fo = -2.f * k * dr * ir;
-      bx = fmaf(fo, d2f_rn(d[0]), bx);
-      by = fmaf(fo, d2f_rn(d[1]), by);
-      bz = fmaf(fo, d2f_rn(d[2]), bz);
+      bx = fmaf(fo, d.v[0].h, bx);
+      by = fmaf(fo, d.v[1].h, by);
+      bz = fmaf(fo, d.v[2].h, bz);
       bu = fmaf(0.5f * k * dr, dr, bu);
     }
   }
   if (walls && S.wall && !meta_con(m)) {
     const float eps = (float)S.wall_eps, sig2 = (float)(S.wall_sigma * S.wall_sigma);
     if (S.wall_kind == 1) {
-      const double d0 = xi[0] - S.wall_center[0], d1 = xi[1] - S.wall_center[1], d2 = xi[2] - S.wall_center[2];
-      const double r2 = fma(d0, d0, fma(d1, d1, d2 * d2));
-      const float q = d2f_rn(fma(-S.wall_radius, S.wall_radius, r2));  // r^2 - R_w^2
-      const float r2f = d2f_rn(r2);
+      const DF3 xi = load_df3(A, tag);
+      const DF d[3] = {df_sub(xi.v[0], S.wall_center_df[0]), df_sub(xi.v[1], S.wall_center_df[1]),
+                       df_sub(xi.v[2], S.wall_center_df[2])};
+      const DF r2 = df_dot3(d, d);
+      const float q = df_sub(r2, S.wall_r2_df).h;  // r^2 - R_w^2
+      const float r2f = r2.h;
       const float ir = rsqrtf(r2f);
       const float h = __fdividef(q, fmaf(r2f, ir, (float)S.wall_radius));  // r - R_w
       if (!(h > 0.f)) {
@@ -1261,21 +1305,23 @@ __device__ __forceinline__ void bonded_terms_f(const DevArrays& A, const SysDev&
         const float s2 = sig2 * ih * ih;
         const float s6 = s2 * s2 * s2;
         const float fr = 24.f * eps * (2.f * s6 * s6 - s6) * ih * ir;
-        bx = fmaf(fr, d2f_rn(d0), bx);
-        by = fmaf(fr, d2f_rn(d1), by);
-        bz = fmaf(fr, d2f_rn(d2), bz);
+        bx = fmaf(fr, d[0].h, bx);
+        by = fmaf(fr, d[1].h, by);
+        bz = fmaf(fr, d[2].h, bz);
         bu += 4.f * eps * (s6 * s6 - s6 + 0.25f);
       }
     } else {
-      const double dist[2] = {xi[2] - S.wall_lo, S.wall_hi - xi[2]};
+      const float rc = (float)S.wall_rc;
+      const DF z = df_from(A.x[2 * A.n + tag]);
+      const float dist[2] = {df_sub(z, S.wall_lo_df).h, df_sub(S.wall_hi_df, z).h};
 #pragma unroll
       for (int w = 0; w < 2; ++w) {
-        if (!(dist[w] > 0.0)) {
+        if (!(dist[w] > 0.f)) {
           flag(A.status, kFlagOutOfGrid);
           continue;
         }
-        if (dist[w] >= S.wall_rc) continue;
-        const float ir = __fdividef(1.f, d2f_rn(dist[w]));
+        if (dist[w] >= rc) continue;
+        const float ir = __fdividef(1.f, dist[w]);
         const float s2 = sig2 * ir * ir;
         const float s6 = s2 * s2 * s2;
         const float fr = 24.f * eps * (2.f * s6 * s6 - s6) * ir;

@@ -101,6 +101,9 @@ struct SysDev {
   double angle_sin0, angle_cos0;  // sin and cos of theta0
   int32_t bond_mix, wall_kind;
   double wall_radius, wall_center[3];
+  // double-float copies of the mixed path's bonded terms: r0^2, sin and cos of
+  // theta0, the wall planes, the wall sphere's centre and R_w^2
+  DF bond_r02_df, angle_sin0_df, angle_cos0_df, wall_lo_df, wall_hi_df, wall_center_df[3], wall_r2_df;
   // noise key, particle range
   uint32_t seed_lo, replica;
   int64_t first, n;
@@ -121,6 +124,7 @@ struct TypeTable {
   float lin_f[kMaxTypes][kMaxTypes];
   float rc_f[kMaxTypes][kMaxTypes];
   double bond_r0_mix[kMaxTypes][kMaxTypes];  // 2^(1/6) sigma_ij / 2
+  DF bond_r02_mix_df[kMaxTypes][kMaxTypes];  // its square
   double mass[kMaxTypes], inv_mass[kMaxTypes], sqrt_mass[kMaxTypes];
   float sqrt_mass_f[kMaxTypes];
   // mixed path, pair terms from double-float displacements (kernels.cu, lj_term_acc)
