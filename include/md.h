@@ -288,7 +288,9 @@ int md_step(md_handle* h, int64_t nsteps);
  * default 256); longer md_step calls are split into several launches. */
 #define MD_OPT_RESIDENT_STEPS 5
 /* MD_OPT_PAIR_TILE: 0 (default) = the pair kernel runs one particle per
- * thread (or MD_OPT_PAIR_LANES lanes per particle); 8, 16 or 32 = cell-tiled:
+ * thread, one per warp on small systems (same bits), MD_OPT_PAIR_LANES lanes
+ * per particle, or the cell-tiled kernel at 8 where cells are dense and the
+ * systems too large for the resident engine; 8, 16 or 32 = cell-tiled:
  * each warp takes that many consecutive sorted particles, split at cell
  * boundaries; for each piece it copies the records of the home cell's
  * 27-cell stencil into shared memory once and the piece's particles share

@@ -858,6 +858,21 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
   A.pair_queue = 1;
   A.list_warp = 32;
   A.store_noise = 1;
+  // Cell list every step, dense cells: the cell-tiled pair kernel (8 particles
+  // per warp) instead of the row kernel, whose lanes diverge over hundreds of
+  // candidates. The line is the mean number of candidates in the 27 cells,
+  // measured on a periodic liquid of 97,336 particles, row and tiled, us: mixed
+  // 383 candidates 271 and 153, 216: 104 and 91, 108: 114 and 92, 56: 65 and 95;
+  // float64 383: 2661 and 1262, 108: 1040 and 515, 56: 547 and 399, 22: 144 and
+  // 396. The two add a particle's terms in different orders, so a handle whose
+  // systems the resident engine could hold keeps the row kernel's order, which
+  // that engine repeats bit for bit.
+  if (h->has_pairs && !A.hashed && cell_total > 0) {
+    const double mean = 27.0 * (double)total / (double)cell_total;
+    const bool resident_fits =
+        resident_smem_bytes(h->precision, h->res_nmax, res_t_bound(h->res_nmax)) <= 232448;  // 227 KB per CTA
+    if (mean >= (h->precision == MD_PREC_FP64 ? 48.0 : 96.0) && !resident_fits) A.dense_tile = 8;
+  }
   for (const SysDev& S : h->sys)
     if (S.kind == kBump || S.kind == kThylakoid) A.composed = 1;
   A.ntypes = prms[0].ntypes;

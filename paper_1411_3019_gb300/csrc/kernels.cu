@@ -3741,6 +3741,12 @@ static void pair_dispatch(const DevArrays& A, int bonds, int walls, int excl, in
     pair_dispatch_cell<R>(A, bonds, walls, excl, st);
     return;
   }
+  if (A.dense_tile && lanes == 1 && A.n > warp_pair_max<R>()) {
+    DevArrays T = A;
+    T.pair_tile = A.dense_tile;
+    pair_dispatch_cell<R>(T, bonds, walls, excl, st);
+    return;
+  }
   switch (lanes) {
     case 2: pair_dispatch_l<R, 2>(A, bonds, walls, excl, st); break;
     case 4: pair_dispatch_l<R, 4>(A, bonds, walls, excl, st); break;
