@@ -315,9 +315,8 @@ int md_step(md_handle* h, int64_t nsteps);
  * positions before it steps. With 0 the wait gives up without reading, so a
  * scan of more than one tile (more than 8192 buckets) always times out. */
 #define MD_OPT_SPIN_LIMIT 8
-/* MD_OPT_PAIR_QUEUE (mixed precision with the Verlet list): 1 (default) = a
- * warp walks its particles' packed list entries as one sequence (their
- * records staged in shared memory a few chunks of 32 at a time), queues the
+/* MD_OPT_PAIR_QUEUE (with the Verlet list): 1 (default) = a warp walks its
+ * particles' packed list entries as one sequence, 32 at a time, queues the
  * pairs near or inside the cutoff and evaluates 32 queued pairs at a time on
  * all lanes; 0 = each lane walks its particle's list alone. Both add every
  * particle's terms in list order with the same arithmetic: the same bits. */
@@ -331,20 +330,21 @@ int md_step(md_handle* h, int64_t nsteps);
  * run, md_step falls back to the separate launches (md_get_option then
  * reads 0). */
 #define MD_OPT_FUSED_REBUILD 10
-/* MD_OPT_LIST_WARP (mixed precision with the Verlet list, MD_OPT_PAIR_QUEUE =
- * 1): particles per warp of the list walk, 32 (default), 16 or 8. The warp
- * walks its particles' lists as one sequence, 32 entries at a time, so long
- * lists (long cutoffs, dense systems) spread over more warps with fewer
- * particles each. The same bits for every setting. */
+/* MD_OPT_LIST_WARP (with the Verlet list, MD_OPT_PAIR_QUEUE = 1): most
+ * particles per warp of the list walk, 32 (default), 16 or 8 (small systems
+ * take fewer by themselves). The warp walks its particles' lists as one
+ * sequence, 32 entries at a time, so long lists (long cutoffs, dense systems)
+ * spread over more warps with fewer particles each. The same bits for every
+ * setting. */
 #define MD_OPT_LIST_WARP 11
-/* MD_OPT_STORE_NOISE (mixed precision with the Verlet list): 1 (default) =
- * the integrator stores the unit normals xi^k it draws for step k (16 bytes
- * per particle) and the next step's force combination, which needs xi^k
- * again beside xi^(k+1), reads them instead of drawing them a second time;
- * 0 = both steps' normals are drawn every step. The stored values are the
- * ones the generator gives, so trajectories are the same bit for bit either
- * way. After md_set_state or md_restore (and after switching the option) the
- * first step draws both. */
+/* MD_OPT_STORE_NOISE: 1 (default) = the integrator stores the unit normals
+ * xi^k it draws for step k (16 bytes per particle, 24 in float64) and the next
+ * step's force combination, which needs xi^k again beside xi^(k+1), reads them
+ * instead of drawing them a second time; 0 = both steps' normals are drawn
+ * every step (the resident engine always draws both). The stored values are
+ * the ones the generator gives, so trajectories are the same bit for bit
+ * either way. After md_set_state or md_restore (and after switching the
+ * option) the first step draws both. */
 #define MD_OPT_STORE_NOISE 12
 /* Verlet neighbour list (the LAMMPS-style list the paper's simulations
  * ran with; the cell list is how it is built). With skin > 0 every pair

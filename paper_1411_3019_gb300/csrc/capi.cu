@@ -345,8 +345,11 @@ void fill_types(const md_params& p, TypeTable& T) {
     for (int b = 0; b < kMaxTypes; ++b) {
       if (a >= p.ntypes || b >= p.ntypes) continue;
       const double rc = p.rcut[a][b], sg = p.sigma[a][b], ep = p.eps[a][b];
-      T.eps[a][b] = ep;
-      T.sig2[a][b] = sg * sg;
+      const double sg6 = std::pow(sg * sg, 3.0);
+      T.c24[a][b] = 24.0 * ep * sg6;
+      T.c48[a][b] = 48.0 * ep * sg6 * sg6;
+      T.c4[a][b] = 4.0 * ep * sg6;
+      T.c4b[a][b] = 4.0 * ep * sg6 * sg6;
       T.rc2[a][b] = rc * rc;
       double shift = 0.0;
       if (rc > 0.0) {
@@ -364,14 +367,11 @@ void fill_types(const md_params& p, TypeTable& T) {
       T.rc[a][b] = rc;
       T.bond_r0_mix[a][b] = std::pow(2.0, 1.0 / 6.0) * sg / 2.0;
       T.bond_r02_mix_df[a][b] = df_split(T.bond_r0_mix[a][b] * T.bond_r0_mix[a][b]);
-      T.eps_f[a][b] = (float)ep;
-      T.sig2_f[a][b] = (float)(sg * sg);
       T.rc2_f[a][b] = (float)(rc * rc);
       T.shift_f[a][b] = (float)shift;
       T.lin_f[a][b] = (float)lin;
       T.rc_f[a][b] = (float)rc;
       // mixed path, pair terms from double-float displacements
-      const double sg6 = std::pow(sg * sg, 3.0);
       T.rc2m_f[a][b] = (float)(rc * rc * (1.0 + std::ldexp(1.0, -18)));
       T.rc2_df[a][b] = df_split(rc * rc);
       T.s6x2_df[a][b] = df_split(2.0 * sg6);
@@ -442,7 +442,7 @@ struct StepKernel {
 };
 
 cudaError_t k_pair_step(md_handle* h, cudaStream_t st) {
-  return launch_pair(h->A, h->precision, h->has_pairs, h->bonds, h->walls, h->excl, st);
+  return launch_pair(h->A, h->precision, h->has_pairs, h->bonds, h->walls, h->excl, 0, st);
 }
 cudaError_t k_bend_step(md_handle* h, cudaStream_t st) { return launch_bend(h->A, h->precision, st); }
 cudaError_t k_integrate_step(md_handle* h, cudaStream_t st) {
@@ -643,7 +643,7 @@ int resident_steps(md_handle* h, int64_t nsteps) {
 }
 
 int forces_now(md_handle* h) {
-  CK(h, launch_pair(h->A, h->precision, h->has_pairs, h->bonds, h->walls, h->excl, h->stream()));
+  CK(h, launch_pair(h->A, h->precision, h->has_pairs, h->bonds, h->walls, h->excl, 1, h->stream()));
   if (h->bends) CK(h, launch_bend(h->A, h->precision, h->stream()));
   return MD_OK;
 }
@@ -905,6 +905,13 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
     A.rec = r;
     if (h->precision != MD_PREC_FP64) al(dalloc(h, &A.rec_lo, n));
   }
+  {  // unit normals of the last step
+    void* w = nullptr;
+    al(h->precision == MD_PREC_FP64 ? dalloc(h, reinterpret_cast<double**>(&w), 3 * n)
+                                    : dalloc(h, reinterpret_cast<float4**>(&w), n));
+    A.noise = w;
+    al(dalloc(h, &A.noise_k, 1));
+  }
   al(dalloc(h, &A.meta, n));
   if (h->excl) al(dalloc(h, &A.mol, n));
   al(dalloc(h, &A.cell, n));
@@ -991,6 +998,7 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
   if (e == cudaSuccess) e = cudaMemset(A.status, 0, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(A.step, 0, sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMemset(A.mode, 0, sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMemset(A.noise_k, 0xff, sizeof(unsigned long long));  // none stored
   if (e == cudaSuccess) {
     const uint32_t nn = (uint32_t)total;
     e = cudaMemcpy(A.start + A.nbucket, &nn, sizeof(uint32_t), cudaMemcpyHostToDevice);
@@ -1243,11 +1251,7 @@ int md_set_neighbor_list(md_handle* h, double skin, int32_t max_neighbors) {
         e = h->precision == MD_PREC_FP64 ? dalloc(h, reinterpret_cast<double4_32a**>(&A.rec0), n)
                                          : dalloc(h, reinterpret_cast<float4**>(&A.rec0), n);
       if (e == cudaSuccess && h->precision != MD_PREC_FP64) e = dalloc(h, &A.rec0_lo, n);
-      if (e == cudaSuccess && h->precision != MD_PREC_FP64) e = dalloc(h, &A.noise, n);
-      if (e == cudaSuccess && h->precision != MD_PREC_FP64 && !A.noise_k) {
-        e = dalloc(h, &A.noise_k, 1);
-        if (e == cudaSuccess) e = cudaMemsetAsync(A.noise_k, 0xff, sizeof(unsigned long long), h->stream());
-      }
+      if (e == cudaSuccess && h->precision == MD_PREC_FP64) e = dalloc(h, &A.rec_lo, n);
       if (e != cudaSuccess) return cuda_fail(h, e, "neighbour list allocation");
       h->nl_capacity = max_neighbors;
     }
@@ -1823,7 +1827,7 @@ extern "C" int md_forces_noalloc(const md_surface* surf, const md_params* prm, i
     if (e == cudaSuccess) e = launch_cells_after_bin(A, 0, st);
     if (e == cudaSuccess) e = launch_bucket_build(A, prm->precision, st);
   }
-  if (e == cudaSuccess) e = launch_pair(A, prm->precision, has_pairs, bonds, walls, excl, st);
+  if (e == cudaSuccess) e = launch_pair(A, prm->precision, has_pairs, bonds, walls, excl, 1, st);
   if (e == cudaSuccess && prm->beads_per_mol > 2 && prm->angle_k != 0.0) e = launch_bend(A, prm->precision, st);
   if (e == cudaSuccess) e = launch_get_forces(A, prm->precision, d_f, d_u, st);
   uint32_t status = 0;

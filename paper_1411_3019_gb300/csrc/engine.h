@@ -47,8 +47,9 @@ cudaError_t launch_nl_build(const DevArrays& A, int precision, int excl, cudaStr
 // returns at once unless the rebuild flag is up, advances the step counter.
 int rebuild_blocks(int precision, int excl, int64_t n);
 cudaError_t launch_rebuild(const DevArrays& A, int precision, int excl, int blocks, cudaStream_t st);
+// energy = 0 inside a step, which needs no energies.
 cudaError_t launch_pair(const DevArrays& A, int precision, int has_pairs, int bonds, int walls,
-                        int excl, cudaStream_t st);
+                        int excl, int energy, cudaStream_t st);
 
 // Combine + momentum half + position half (+ binning when has_pairs).
 // Bend-angle forces added to the pair kernel's output (systems with angles).

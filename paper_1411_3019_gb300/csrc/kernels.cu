@@ -70,17 +70,17 @@ __device__ __forceinline__ void gauss3(uint32_t seed, uint32_t rep, uint32_t pid
   const float r23 = sqrtf(fmaxf(-2.0f * __logf(u2), 0.0f));
   float sn, cs;
   __sincosf(two_pi * (u1 - 0.5f), &sn, &cs);
-  gx = -r01 * cs;
-  gy = -r01 * sn;
-  gz = -r23 * __cosf(two_pi * (u3 - 0.5f));
+  gx = __fmul_rn(-r01, cs);  // rounded here, also where the next step's sum would take the product into an FMA:
+  gy = __fmul_rn(-r01, sn);  // a normal read back from memory must be the one drawn again
+  gz = __fmul_rn(-r23, __cosf(two_pi * (u3 - 0.5f)));
 #else
   const float r01 = sqrtf(-2.0f * logf(u0));
   const float r23 = sqrtf(-2.0f * logf(u2));
   float sn, cs;
   sincospif(2.0f * u1, &sn, &cs);
-  gx = r01 * cs;
-  gy = r01 * sn;
-  gz = r23 * cospif(2.0f * u3);
+  gx = __fmul_rn(r01, cs);
+  gy = __fmul_rn(r01, sn);
+  gz = __fmul_rn(r23, cospif(2.0f * u3));
 #endif
 }
 
@@ -95,9 +95,9 @@ __device__ __forceinline__ void gauss3(uint32_t seed, uint32_t rep, uint32_t pid
   const double r23 = sqrt(-2.0 * log(u2));
   double sn, cs;
   sincospi(2.0 * u1, &sn, &cs);
-  gx = r01 * cs;
-  gy = r01 * sn;
-  gz = r23 * cospi(2.0 * u3);
+  gx = __dmul_rn(r01, cs);
+  gy = __dmul_rn(r01, sn);
+  gz = __dmul_rn(r23, cospi(2.0 * u3));
 }
 
 // Format conversions on the integer pipe. On this GPU a float64 <-> float32
@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_onepass(DevArrays A, int 
     if (threadIdx.x == 0 && atomicAdd(&ctl->done, 1u) == gridDim.x - 1) {
       ctl->done = 0u;
       if (advance) {
-        if (A.nl_dirty && A.noise_k) *A.noise_k = *A.step;  // list mode: this step's normals are stored
+        if (A.noise_k) *A.noise_k = *A.step;  // this step's normals are stored
         *A.step += 1ull;
         *A.mode = 1;
       }
@@ -684,7 +684,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_onepass(DevArrays A, int 
       ctl->tile = 0u;
       ctl->epoch = epoch + 1u;
       if (advance) {
-        if (A.nl_dirty && A.noise_k) *A.noise_k = *A.step;  // list mode: this step's normals are stored
+        if (A.noise_k) *A.noise_k = *A.step;  // this step's normals are stored
         *A.step += 1ull;
         *A.mode = 1;
       }
@@ -713,10 +713,15 @@ template <> __device__ __forceinline__ void put_rec<float>(void* rec, float4* lo
   reinterpret_cast<float4*>(rec)[s] = make_float4(x.h, y.h, z.h, __uint_as_float(bits));
   lo[s] = make_float4(x.l, y.l, z.l, 0.f);
 }
-template <> __device__ __forceinline__ void put_rec<double>(void* rec, float4*, uint32_t s, double ox, double oy,
+// Float64 path: the record rounded to float32, the list walk's screen copy.
+__device__ __forceinline__ float4 screen_rec(const double4_32a& r) {
+  return make_float4(d2f_rn(r.x), d2f_rn(r.y), d2f_rn(r.z), __uint_as_float((uint32_t)__double_as_longlong(r.w)));
+}
+template <> __device__ __forceinline__ void put_rec<double>(void* rec, float4* lo, uint32_t s, double ox, double oy,
                                                             double oz, uint32_t bits) {
-  reinterpret_cast<double4_32a*>(rec)[s] =
-      make_double4_32a(ox, oy, oz, __longlong_as_double((long long)bits));
+  const double4_32a r = make_double4_32a(ox, oy, oz, __longlong_as_double((long long)bits));
+  reinterpret_cast<double4_32a*>(rec)[s] = r;
+  if (lo) lo[s] = screen_rec(r);
 }
 
 // Offset of a position from the centre of its cell, formed in float64 (the
@@ -776,28 +781,26 @@ __global__ void k_bucket_build(DevArrays A) {
 }
 
 // float64 reciprocal and inverse square root without the long divide/sqrt
-// sequences: a float32 hardware estimate refined by Newton-Raphson steps
-// (Newton's method on 1/e - v = 0 and on 1/e^2 - v = 0), each step doubling
-// the correct bits (2^-22 -> 2^-44 -> full float64). v must be a positive
-// normal number inside the float32 range; otherwise the float64 operator is
-// used.
+// sequences: a float32 hardware estimate y with relative error below 2^-22, its
+// residual e in float64 (1 - v y, or 1 - v y^2), and the series of 1 / (1 - e)
+// or (1 - e)^(-1/2) to second order, whose remainder e^3 is below 2^-63: three
+// and five float64 operations (two each per SM and clock) in place of four and
+// seven for two Newton steps. v must be a positive normal number inside the
+// float32 range; otherwise the float64 operator is used.
 __device__ __forceinline__ double nr_rcp(double v) {
   const float vf = d2f_rn(v);
   if (!(vf > 1.0e-37f && vf < 1.0e37f)) return 1.0 / v;
-  double e = f2d(__frcp_rn(vf));
-  e = fma(e, fma(-v, e, 1.0), e);
-  e = fma(e, fma(-v, e, 1.0), e);
-  return e;
+  const double y = f2d(__frcp_rn(vf));
+  const double e = fma(-v, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 
 __device__ __forceinline__ double nr_rsqrt(double v) {
   const float vf = d2f_rn(v);
   if (!(vf > 1.0e-37f && vf < 1.0e37f)) return 1.0 / sqrt(v);
-  double r = f2d(rsqrtf(vf));
-  const double hv = 0.5 * v;
-  r = r * fma(-hv * r, r, 1.5);
-  r = r * fma(-hv * r, r, 1.5);
-  return r;
+  const double r = f2d(rsqrtf(vf));
+  const double e = fma(-v * r, r, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
 }
 
 // Surface direction in float32 (mixed path): the gradient of g at a point
@@ -902,7 +905,7 @@ struct PairAcc {
 };
 
 template <typename R> struct PairTab {
-  R eps[kMaxTypes * kMaxTypes], sig2[kMaxTypes * kMaxTypes], rc2[kMaxTypes * kMaxTypes],
+  R c24[kMaxTypes * kMaxTypes], c48[kMaxTypes * kMaxTypes], c4[kMaxTypes * kMaxTypes], c4b[kMaxTypes * kMaxTypes], rc2[kMaxTypes * kMaxTypes],
       shift[kMaxTypes * kMaxTypes], lin[kMaxTypes * kMaxTypes], rc[kMaxTypes * kMaxTypes];
   PairAcc acc;
 };
@@ -911,8 +914,6 @@ template <typename R> __device__ __forceinline__ void load_tab(PairTab<R>& t, co
 template <> __device__ __forceinline__ void load_tab<float>(PairTab<float>& t, const TypeTable* T) {
   for (int q = threadIdx.x; q < kMaxTypes * kMaxTypes; q += blockDim.x) {
     const int a = q / kMaxTypes, b = q % kMaxTypes;
-    t.eps[q] = T->eps_f[a][b];
-    t.sig2[q] = T->sig2_f[a][b];
     t.rc2[q] = T->rc2_f[a][b];
     t.shift[q] = T->shift_f[a][b];
     t.lin[q] = T->lin_f[a][b];
@@ -928,18 +929,17 @@ template <> __device__ __forceinline__ void load_tab<float>(PairTab<float>& t, c
 template <> __device__ __forceinline__ void load_tab<double>(PairTab<double>& t, const TypeTable* T) {
   for (int q = threadIdx.x; q < kMaxTypes * kMaxTypes; q += blockDim.x) {
     const int a = q / kMaxTypes, b = q % kMaxTypes;
-    t.eps[q] = T->eps[a][b];
-    t.sig2[q] = T->sig2[a][b];
+    t.c24[q] = T->c24[a][b];
+    t.c48[q] = T->c48[a][b];
+    t.c4[q] = T->c4[a][b];
+    t.c4b[q] = T->c4b[a][b];
     t.rc2[q] = T->rc2[a][b];
     t.shift[q] = T->shift[a][b];
     t.lin[q] = T->lin[a][b];
     t.rc[q] = T->rc[a][b];
+    t.acc.rc2m[q] = T->rc2m_f[a][b];  // the list walk's float32 screen
   }
 }
-
-template <typename R> __device__ __forceinline__ R rcp(R v);
-template <> __device__ __forceinline__ float rcp<float>(float v) { return __frcp_rn(v); }
-template <> __device__ __forceinline__ double rcp<double>(double v) { return 1.0 / v; }
 
 template <typename R> __device__ __forceinline__ R rsq(R v);
 template <> __device__ __forceinline__ float rsq<float>(float v) { return rsqrtf(v); }
@@ -951,14 +951,15 @@ template <> __device__ __forceinline__ double rsq<double>(double v) { return nr_
 // energy-conservation study, V = phi(r) - phi(r_c) - (r - r_c) phi'(r_c), whose
 // force -phi'(r) + phi'(r_c) vanishes at r_c. Adds the force on i (along the
 // displacement d = x_i - x_j) and half the pair energy.
+// With q = r^-6 it reads f/r = r^-2 q (48 eps sigma^12 q - 24 eps sigma^6) and
+// V = q (4 eps sigma^12 q - 4 eps sigma^6) - phi(r_c).
 template <typename R>
 __device__ __forceinline__ void lj_factor(const PairTab<R>& tab, uint32_t qt, R r2, R& fr, R& v) {
-  const R inv_r2 = rcp<R>(r2);
-  const R s2 = tab.sig2[qt] * inv_r2;
-  const R s6 = s2 * s2 * s2;
-  const R e = tab.eps[qt];
-  fr = (R)24 * e * s6 * ((R)2 * s6 - (R)1) * inv_r2;
-  v = (R)4 * e * s6 * (s6 - (R)1) - tab.shift[qt];
+  static_assert(sizeof(R) == 8, "the mixed path's terms are acc_pair's");
+  const R inv_r2 = nr_rcp(r2);
+  const R q = inv_r2 * inv_r2 * inv_r2;
+  fr = inv_r2 * q * fma(tab.c48[qt], q, -tab.c24[qt]);
+  v = fma(q, fma(tab.c4b[qt], q, -tab.c4[qt]), -tab.shift[qt]);
   const R lin = tab.lin[qt];
   if (lin != (R)0) {
     const R inv_r = rsq<R>(r2);
@@ -2297,6 +2298,174 @@ __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(
   store_f<float>(A.f, tag, fx, fy, fz, u);
 }
 
+// Float64 path with the Verlet list: k_pair_nlq's walk with float64 terms. The
+// entries are screened in float32 on the records' rounded copies (A.rec_lo, 16
+// bytes a gather instead of 32 and no float64 operation for the about half of
+// the entries that lie between the cutoff and the skin), and the queued pairs
+// are evaluated 32 at a time on all lanes from the float64 records: the float64
+// pipe retires two lanes per SM and clock whether or not the others are idle, so
+// full warps are what counts. ENERGY = false (inside a step, which only needs
+// forces) leaves the energies out. Terms and order of sums are k_pair_nl's: the
+// same bits.
+struct QueueWarp64 {
+  float4 ri[32];                    // the lanes' own rounded records
+  float csx[32], csy[32], csz[32];  // the lanes' cell edges
+  double fr[32], d[4][32];          // evaluated terms: factor, displacement, energy
+  uint32_t qt[kNlqStage];           // queue: the neighbour's slot
+  uint8_t qc[kNlqStage], qo[kNlqStage];  // queue: its stencil cell and the pair's particle (lane)
+  uint8_t run0[32], runn[32];       // per particle: first position and length of its run in the evaluated 32
+};
+
+template <bool BONDS, bool WALLS, bool ENERGY>
+__global__ void __launch_bounds__(kQueueWarps * 32) k_pair_nlq64(DevArrays A) {
+  __shared__ PairTab<double> tab;
+  __shared__ QueueWarp64 qw_all[kQueueWarps];
+  load_tab<double>(tab, A.types);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *A.nl_dirty = 0u;  // the previous step's rebuild is done
+  const int lane = (int)(threadIdx.x & 31u);
+  QueueWarp64& Q = qw_all[threadIdx.x >> 5];
+  __syncthreads();
+  const uint32_t P = (uint32_t)A.list_warp;
+  const uint32_t s0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * P;  // the warp's first slot
+  const uint32_t s = s0 + (uint32_t)lane;
+  const bool valid = (uint32_t)lane < P && s < (uint32_t)A.n;
+  const double4_32a* __restrict__ rec = reinterpret_cast<const double4_32a*>(A.rec);
+  const float4* __restrict__ recf = A.rec_lo;
+  uint32_t m = 0, cnt = 0, off = 0;
+  float4 rif = make_float4(0.f, 0.f, 0.f, 0.f);
+  float csx = 0.f, csy = 0.f, csz = 0.f;
+  if (valid) {
+    off = A.nl_off[s];
+    m = A.smeta[s];
+    const SysDev& S = A.sys[meta_sys(m)];
+    rif = recf[s];
+    csx = S.cs_f[0]; csy = S.cs_f[1]; csz = S.cs_f[2];
+    cnt = A.nl_cnt[s];
+  }
+  Q.ri[lane] = rif;
+  Q.csx[lane] = csx; Q.csy[lane] = csy; Q.csz[lane] = csz;
+  uint32_t incl = cnt;  // prefix sums of the list lengths over the warp
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const uint32_t pre = incl - cnt;
+  const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+  const uint32_t* __restrict__ list =
+      A.nl_pk + (int64_t)(s0 & ~31u) * (uint32_t)A.nl_max + __shfl_sync(0xffffffffu, off, 0);
+  double fx = 0.0, fy = 0.0, fz = 0.0, u = 0.0;
+  // evaluate the k <= 32 queued pairs from queue position q0; each particle adds its run in order
+  auto drain = [&](uint32_t q0, uint32_t k) {
+    __syncwarp();
+    const bool have = (uint32_t)lane < k;
+    uint32_t ow = 0;
+    double fr = 0.0, v = 0.0, ddx = 0.0, ddy = 0.0, ddz = 0.0;
+    if (have) {
+      ow = Q.qo[q0 + lane];
+      const uint32_t code = Q.qc[q0 + lane];
+      const double4_32a ri = rec[s0 + ow], rj = rec[Q.qt[q0 + lane]];
+      const SysDev& S = A.sys[meta_sys(A.smeta[s0 + ow])];
+      const int dz = (int)(code / 9u) - 1, dy = (int)(code / 3u % 3u) - 1, dx = (int)(code % 3u) - 1;
+      const uint32_t qt = (RecT<double>::bits(ri) & 7u) * kMaxTypes + (RecT<double>::bits(rj) & 7u);
+      // (the shift only where there is one: x - 0 is x)
+      double ax = ri.x - rj.x, ay = ri.y - rj.y, az = ri.z - rj.z;
+      if (dx) ax -= dx < 0 ? -S.cs[0] : S.cs[0];
+      if (dy) ay -= dy < 0 ? -S.cs[1] : S.cs[1];
+      if (dz) az -= dz < 0 ? -S.cs[2] : S.cs[2];
+      const double r2 = ax * ax + ay * ay + az * az;
+      if (r2 < tab.rc2[qt]) {
+        lj_factor<double>(tab, qt, r2, fr, v);
+        ddx = ax; ddy = ay; ddz = az;
+      }
+    }
+    Q.fr[lane] = fr;
+    Q.d[0][lane] = ddx; Q.d[1][lane] = ddy; Q.d[2][lane] = ddz;
+    if (ENERGY) Q.d[3][lane] = v;
+    const uint32_t prev = __shfl_up_sync(0xffffffffu, ow, 1);
+    const bool start = have && (lane == 0 || prev != ow);
+    const uint32_t starts = __ballot_sync(0xffffffffu, start);
+    Q.runn[lane] = 0;
+    __syncwarp();
+    if (start) {
+      const uint32_t after = starts & ~((2u << lane) - 1u);  // starts above this one
+      const uint32_t next = after ? (uint32_t)(__ffs(after) - 1) : k;
+      Q.run0[ow] = (uint8_t)lane;
+      Q.runn[ow] = (uint8_t)(next - lane);
+    }
+    __syncwarp();
+    const uint32_t r0 = Q.run0[lane], rn = Q.runn[lane];
+    for (uint32_t j = r0; j < r0 + rn; ++j) {
+      const double f = Q.fr[j];
+      fx = fma(f, Q.d[0][j], fx);
+      fy = fma(f, Q.d[1][j], fy);
+      fz = fma(f, Q.d[2][j], fz);
+      if (ENERGY) u = fma(0.5, Q.d[3][j], u);
+    }
+    __syncwarp();
+  };
+  uint32_t qn = 0;
+  for (uint32_t c = 0; c < total; c += (uint32_t)kNlqStage) {
+    uint32_t e[kNlqGroup], own[kNlqGroup];
+    float4 rj[kNlqGroup];
+    __syncwarp();  // (first round: the lanes' records are written)
+#pragma unroll
+    for (int g = 0; g < kNlqGroup; ++g) {
+      const uint32_t p = c + 32u * g + (uint32_t)lane;
+      uint32_t ow = 0;  // the particle of position p: the highest lane whose prefix is <= p
+#pragma unroll
+      for (int step = 16; step > 0; step >>= 1) {
+        const uint32_t cand = ow + (uint32_t)step;
+        const uint32_t pc = __shfl_sync(0xffffffffu, pre, (int)(cand & 31u));
+        if (cand < 32u && pc <= p) ow = cand;
+      }
+      own[g] = ow;
+      e[g] = p < total ? list[p] : 0u;
+    }
+#pragma unroll
+    for (int g = 0; g < kNlqGroup; ++g)
+      if (c + 32u * g + (uint32_t)lane < total) rj[g] = recf[e[g] >> 5];
+#pragma unroll
+    for (int g = 0; g < kNlqGroup; ++g) {
+      const uint32_t p = c + 32u * g + (uint32_t)lane;
+      bool hit = false;
+      const uint32_t code = e[g] & 31u;
+      if (p < total) {
+        const uint32_t ow = own[g];
+        const float4 ro = Q.ri[ow];
+        const int dz = (int)(code / 9u) - 1, dy = (int)(code / 3u % 3u) - 1, dx = (int)(code % 3u) - 1;
+        const float ddx = ro.x - rj[g].x - (float)dx * Q.csx[ow], ddy = ro.y - rj[g].y - (float)dy * Q.csy[ow],
+                    ddz = ro.z - rj[g].z - (float)dz * Q.csz[ow];
+        const float r2 = ddx * ddx + ddy * ddy + ddz * ddz;
+        hit = r2 < tab.acc.rc2m[(RecT<float>::bits(ro) & 7u) * kMaxTypes + (RecT<float>::bits(rj[g]) & 7u)];
+      }
+      const uint32_t mask = __ballot_sync(0xffffffffu, hit);
+      if (hit) {
+        const uint32_t at = qn + __popc(mask & ((1u << lane) - 1u));
+        Q.qt[at] = e[g] >> 5;
+        Q.qc[at] = (uint8_t)code;
+        Q.qo[at] = (uint8_t)own[g];
+      }
+      qn += __popc(mask);
+      if (qn >= 64u || (g == kNlqGroup - 1 && qn >= 32u)) {  // room for the next 32 and full warps of terms
+        uint32_t q0 = 0;
+        for (; qn - q0 >= 32u; q0 += 32u) drain(q0, 32u);
+        qn -= q0;
+        if ((uint32_t)lane < qn) {  // the rest moves to the front
+          Q.qt[lane] = Q.qt[q0 + lane];
+          Q.qc[lane] = Q.qc[q0 + lane];
+          Q.qo[lane] = Q.qo[q0 + lane];
+        }
+      }
+    }
+  }
+  if (qn) drain(0u, qn);
+  if (!valid) return;
+  const uint32_t tag = A.stag[s];
+  if (BONDS || WALLS) bonded_terms<double>(A, A.sys[meta_sys(m)], tag, m, BONDS, WALLS, fx, fy, fz, u);
+  store_f<double>(A.f, tag, fx, fy, fz, u);
+}
+
 // Bend-angle forces (and energy shares) added to the pair kernel's output.
 template <typename R>
 __global__ void k_bend(DevArrays A) {
@@ -2781,17 +2950,38 @@ template <> __device__ __forceinline__ double noise_amp<double>(const SysDev& S,
   return S.noise_unit * T->sqrt_mass[ty];
 }
 
+// Where the unit normals of the last integrated step are kept, by particle:
+// float4 on the mixed path, three float64 arrays on the float64 path.
+template <typename R> struct NoiseSlot;
+template <> struct NoiseSlot<float> {
+  float4* p;
+  __device__ __forceinline__ NoiseSlot(void* noise, int64_t, int64_t i) : p(reinterpret_cast<float4*>(noise) + i) {}
+  __device__ __forceinline__ void load(float& x, float& y, float& z) const {
+    const float4 w = *p;
+    x = w.x; y = w.y; z = w.z;
+  }
+  __device__ __forceinline__ void store(float x, float y, float z) const { *p = make_float4(x, y, z, 0.f); }
+};
+template <> struct NoiseSlot<double> {
+  double* p;
+  int64_t n;
+  __device__ __forceinline__ NoiseSlot(void* noise, int64_t n_, int64_t i)
+      : p(reinterpret_cast<double*>(noise) + i), n(n_) {}
+  __device__ __forceinline__ void load(double& x, double& y, double& z) const { x = p[0]; y = p[n]; z = p[2 * n]; }
+  __device__ __forceinline__ void store(double x, double y, double z) const { p[0] = x; p[n] = y; p[2 * n] = z; }
+};
+
 // Algorithm S1 force combination at step k for one particle, in R:
 //   first step after a set state:  F = f - gamma p + f_r^k
 //   otherwise:  F = [f - gamma p^{k-1/2} + (f_r^k + f_r^{k-1})/2] / (1 + gamma dt/2)
-// with f_r = sqrt(2 m kT gamma / dt) xi, xi drawn from Philox in R. Float32
-// only: with a slot xi, the normals of step k are stored there, and those of
-// step k-1 read from it when xi_prev (they were stored by the previous step:
-// the same values gauss3 would give again).
+// with f_r = sqrt(2 m kT gamma / dt) xi, xi drawn from Philox in R. With
+// xi_store the normals of step k are stored in xi, and with xi_prev those of
+// step k-1 are read from it (they were stored by the previous step: the same
+// values gauss3 would give again).
 template <typename R>
 __device__ __forceinline__ Force3<R> combine(const SysDev& S, const TypeTable* T, uint32_t ty, uint32_t pid,
                                              unsigned long long k, int mode, Force3<R> f, R px, R py, R pz,
-                                             float4* xi = nullptr, bool xi_prev = false) {
+                                             const NoiseSlot<R>& xi, bool xi_store, bool xi_prev) {
   R nx = 0, ny = 0, nz = 0;
   const R amp = noise_amp<R>(S, T, ty);
   if (amp > (R)0) {
@@ -2801,22 +2991,12 @@ __device__ __forceinline__ Force3<R> combine(const SysDev& S, const TypeTable* T
       nx = amp * gx; ny = amp * gy; nz = amp * gz;
     } else {
       R hx, hy, hz;
-      if constexpr (sizeof(R) == 4) {
-        if (xi_prev) {
-          const float4 w = *xi;
-          hx = w.x; hy = w.y; hz = w.z;
-        } else {
-          gauss3(S.seed_lo, S.replica, pid, k - 1ull, hx, hy, hz);
-        }
-      } else {
-        gauss3(S.seed_lo, S.replica, pid, k - 1ull, hx, hy, hz);
-      }
+      if (xi_prev) xi.load(hx, hy, hz);
+      else gauss3(S.seed_lo, S.replica, pid, k - 1ull, hx, hy, hz);
       const R ha = (R)0.5 * amp;
       nx = ha * (gx + hx); ny = ha * (gy + hy); nz = ha * (gz + hz);
     }
-    if constexpr (sizeof(R) == 4) {
-      if (xi) *xi = make_float4(gx, gy, gz, 0.f);
-    }
+    if (xi_store) xi.store(gx, gy, gz);
   }
   const R gam = sys_gamma<R>(S);
   Force3<R> F;
@@ -2908,12 +3088,18 @@ template <typename R> struct NlSink {
       d2 = fmaf(ex.h, ex.h, fmaf(ey.h, ey.h, ez.h * ez.h));
     } else {
       r.x += dx; r.y += dy; r.z += dz;
-      d2 = d2f_rn(fma(dx, dx, fma(dy, dy, dz * dz)));
+      const float ex = d2f_rn(dx), ey = d2f_rn(dy), ez = d2f_rn(dz);
+      d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+      if (rec_lo) rec_lo[s] = screen_rec(r);
     }
     rec[s] = r;
     if (!(d2 <= half_skin2)) atomicOr(dirty, 1u);
   }
 };
+
+__device__ __forceinline__ bool line_surface(int32_t kind) {
+  return kind == kPlane || kind == kSphere || kind == kEllipsoid || kind == kCylinder;
+}
 
 // Float64 path: combine + momentum half of step k + position half of step
 // k+1, then the cell of x^{k+1} and its rank in the bucket counter.
@@ -2927,7 +3113,8 @@ template <typename R> struct NlSink {
 // update falls under 4 ulp of the position (round-off floor).
 template <class Bin>
 __device__ __forceinline__ void integrate_particle_fp64(const DevArrays& A, int64_t i, Force3<double> fr_in,
-                                                        unsigned long long k, int mode, const Bin& bin) {
+                                                        unsigned long long k, int mode, const Bin& bin,
+                                                        bool xi_store = false, bool xi_prev = false) {
   const int64_t n = A.n;
   const uint32_t m = A.meta[i];
   const SysDev& S = A.sys[meta_sys(m)];
@@ -2935,61 +3122,146 @@ __device__ __forceinline__ void integrate_particle_fp64(const DevArrays& A, int6
   const uint32_t ty = meta_type(m);
   const double x = A.x[i], y = A.x[n + i], z = A.x[2 * n + i];
   double px = A.ph[i], py = A.ph[n + i], pz = A.ph[2 * n + i];
-  const Force3<double> Fr = combine<double>(S, T, ty, (uint32_t)(i - S.first), k, mode, fr_in, px, py, pz);
+  const Force3<double> Fr = combine<double>(S, T, ty, (uint32_t)(i - S.first), k, mode, fr_in, px, py, pz,
+                                            NoiseSlot<double>(A.noise, n, i), xi_store, xi_prev);
   const double Fx = Fr.x, Fy = Fr.y, Fz = S.kind == kXY2D ? 0.0 : Fr.z;  // 2D plane: no z update
   const double h = S.half_dt;
   const bool con = meta_con(m);
-  double n0x = 0.0, n0y = 0.0, n0z = 0.0, nn = 1.0, inv_nn = 0.0;
-  Piece q0{};
-  const bool held = S.kind == kThylakoid;  // composite surface: the piece at x^k for the whole solve
-  if (con) {
-    if (held) q0 = thyl_select(S, x, y, z);
-    surf_n(S, held ? thyl_geval(S, q0, x, y, z) : surf_g(S, x, y, z), n0x, n0y, n0z);
-    nn = fma(n0x, n0x, fma(n0y, n0y, n0z * n0z));
-    inv_nn = nr_rcp(nn);
-  }
-  if (mode != 0) momentum_half(h, Fx, Fy, Fz, con, n0x, n0y, n0z, inv_nn, px, py, pz);
-  double qx = fma(h, Fx, px), qy = fma(h, Fy, py), qz = fma(h, Fz, pz);  // p^{k+1/2} before the constraint
-  const double dtm = S.dt * T->inv_mass[ty];
-  double xn = fma(dtm, qx, x), yn = fma(dtm, qy, y), zn = fma(dtm, qz, z);
-  if (con) {
-    const double a = h * dtm;  // dt^2 / (2m)
-    const double yx = xn, yy = yn, yz = zn;
-    // |n1| and |n0| differ by about |x - x^k| times the curvature; the 2%
-    // margin on g^2 keeps |g| / |n(x^{k+1})| below eta.
-    const double tol2nn = 0.98 * S.tol2 * nn;
-    const double inv_a_nn = S.frozen ? inv_nn * nr_rcp(a) : 0.0;
-    double lam = 0.0;
-    bool ok = false;
-    for (int it = 0; it <= S.max_newton; ++it) {
-      const GEval e = held ? thyl_geval(S, q0, xn, yn, zn) : surf_g(S, xn, yn, zn);
-      if (e.g * e.g < tol2nn) {
-        ok = true;
+  const double dtm = S.dtm[ty];
+  double qx, qy, qz, xn, yn, zn;
+  if (con && line_surface(S.kind)) {
+    // Plane, sphere, ellipsoid, cylinder: with w = grad g(x^k) / 2 (the plane's
+    // normal itself) g on the line y - nu w is the exact quadratic gy - b nu + c
+    // nu^2. Newton runs on it in float32 first, then in float64 from the
+    // residual: three float64 operations an iteration instead of the about
+    // twenty-five of a point evaluation with its gradient and reciprocal.
+    double d[3] = {x, y, z}, w[3], ia[3];
+    if (!S.c_zero) {
+      d[0] -= S.c[0]; d[1] -= S.c[1]; d[2] -= S.c[2];
+    }
+    const bool plane = S.kind == kPlane, ell = S.kind == kEllipsoid;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const bool off = S.kind == kCylinder && a == S.axis;
+      ia[a] = S.inv_a2[a];
+      w[a] = plane ? S.p[a] : ell ? ia[a] * d[a] : off ? 0.0 : d[a];
+    }
+    const double ww = fma(w[0], w[0], fma(w[1], w[1], w[2] * w[2]));
+    if (mode != 0) momentum_half(h, Fx, Fy, Fz, true, w[0], w[1], w[2], nr_rcp(ww), px, py, pz);
+    qx = fma(h, Fx, px); qy = fma(h, Fy, py); qz = fma(h, Fz, pz);  // p^{k+1/2} before the constraint
+    xn = fma(dtm, qx, x); yn = fma(dtm, qy, y); zn = fma(dtm, qz, z);
+    double D[3] = {xn, yn, zn};
+    if (!S.c_zero) {
+      D[0] -= S.c[0]; D[1] -= S.c[1]; D[2] -= S.c[2];
+    }
+    double gy, b, c;  // halved for the plane: b = n.n, c = 0
+    if (plane) {
+      gy = fma(w[0], D[0], fma(w[1], D[1], w[2] * D[2]));
+      b = ww;
+      c = 0.0;
+    } else {
+      double u[3], v[3];  // grad g(y) / 2 and H w / 2
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const bool off = S.kind == kCylinder && a == S.axis;
+        u[a] = ell ? ia[a] * D[a] : off ? 0.0 : D[a];
+        v[a] = ell ? ia[a] * w[a] : w[a];
+      }
+      gy = fma(u[0], D[0], fma(u[1], D[1], fma(u[2], D[2], ell ? -1.0 : S.gconst)));
+      b = 2.0 * fma(u[0], w[0], fma(u[1], w[1], u[2] * w[2]));
+      c = ell ? fma(v[0], w[0], fma(v[1], w[1], v[2] * w[2])) : ww;
+    }
+    const float gyf = d2f_rn(gy), bf = d2f_rn(b), cf = d2f_rn(c), wwf = d2f_rn(ww);
+    // |n1| and |n0| differ by about |x - x^k| times the curvature; the 1% margin keeps |g| / |n(x^{k+1})| below eta
+    const float n0f = (plane ? 1.f : 2.f) * sqrtf(wwf);
+    const float tol_n = 0.99f * S.tol_f * n0f;
+    const float frozen_den = plane ? wwf : 2.f * wwf;  // b at x^k: n0.n0 in the units of b
+    const float wmax = fmaxf(fabsf(d2f_rn(w[0])), fmaxf(fabsf(d2f_rn(w[1])), fabsf(d2f_rn(w[2]))));
+    const float xmax = fmaxf(fabsf(d2f_rn(xn)), fmaxf(fabsf(d2f_rn(yn)), fabsf(d2f_rn(zn))));
+    const float floor_nu = 4.f * (float)DBL_EPSILON * xmax / wmax;  // an update under 4 ulp of the position
+    float nu0 = 0.f;
+    int it = 0;
+    for (; it < S.max_newton; ++it) {
+      const float gf = fmaf(fmaf(cf, nu0, -bf), nu0, gyf);
+      if (fabsf(gf) < 0.5f * tol_n) break;
+      const float dn = gf * __frcp_rn(S.frozen ? frozen_den : fmaf(-2.f * nu0, cf, bf));
+      nu0 += dn;
+      if (fabsf(dn) <= 0x1p-22f * fabsf(nu0)) {
+        ++it;
         break;
       }
-      if (it == S.max_newton) break;
-      double dl;
-      if (S.frozen) {
-        dl = e.g * inv_a_nn;
-      } else {
-        double n1x, n1y, n1z;
-        surf_n(S, e, n1x, n1y, n1z);
-        dl = e.g * nr_rcp(a * fma(n1x, n0x, fma(n1y, n0y, n1z * n0z)));
-      }
-      lam += dl;
-      const double al = a * lam;
-      xn = fma(-al, n0x, yx); yn = fma(-al, n0y, yy); zn = fma(-al, n0z, yz);
-      if (it > 0) {  // round-off floor: the update is below 4 ulp of the position
-        const double step = fabs(dl) * a * fmax(fabs(n0x), fmax(fabs(n0y), fabs(n0z)));
-        if (step <= 4.0 * DBL_EPSILON * fmax(fabs(xn), fmax(fabs(yn), fabs(zn)))) {
+    }
+    double nu = f2d(nu0);
+    bool ok = false;
+    for (;; ++it) {
+      const double g = fma(fma(c, nu, -b), nu, gy);
+      const float gf = d2f_rn(g);
+      const float rden = __frcp_rn(S.frozen ? frozen_den : fmaf(-2.f * d2f_rn(nu), cf, bf));
+      ok = fabsf(gf) < tol_n;
+      if (!ok && it >= S.max_newton) break;
+      nu = fma(g, f2d(rden), nu);  // (also where the test is met: the residual in hand takes g to its rounding)
+      if (ok) break;
+      if (it > 0 && fabsf(gf * rden) <= floor_nu) { ok = true; break; }
+    }
+    if (!ok) flag(A.status, kFlagRattle);
+    xn = fma(-nu, w[0], xn); yn = fma(-nu, w[1], yn); zn = fma(-nu, w[2], zn);
+    const double hl = nu * S.inv_dtm[ty];
+    qx = fma(-hl, w[0], qx); qy = fma(-hl, w[1], qy); qz = fma(-hl, w[2], qz);
+  } else {
+    double n0x = 0.0, n0y = 0.0, n0z = 0.0, nn = 1.0, inv_nn = 0.0;
+    Piece q0{};
+    const bool held = S.kind == kThylakoid;  // composite surface: the piece at x^k for the whole solve
+    if (con) {
+      if (held) q0 = thyl_select(S, x, y, z);
+      surf_n(S, held ? thyl_geval(S, q0, x, y, z) : surf_g(S, x, y, z), n0x, n0y, n0z);
+      nn = fma(n0x, n0x, fma(n0y, n0y, n0z * n0z));
+      inv_nn = nr_rcp(nn);
+    }
+    if (mode != 0) momentum_half(h, Fx, Fy, Fz, con, n0x, n0y, n0z, inv_nn, px, py, pz);
+    qx = fma(h, Fx, px); qy = fma(h, Fy, py); qz = fma(h, Fz, pz);  // p^{k+1/2} before the constraint
+    xn = fma(dtm, qx, x); yn = fma(dtm, qy, y); zn = fma(dtm, qz, z);
+    if (con) {
+      const double a = h * dtm;  // dt^2 / (2m)
+      const double yx = xn, yy = yn, yz = zn;
+      // |n1| and |n0| differ by about |x - x^k| times the curvature; the 2%
+      // margin on g^2 keeps |g| / |n(x^{k+1})| below eta.
+      const double tol2nn = 0.98 * S.tol2 * nn;
+      const double inv_a_nn = S.frozen ? inv_nn * nr_rcp(a) : 0.0;
+      const float af = d2f_rn(a);
+      const float n0max = fmaxf(fabsf(d2f_rn(n0x)), fmaxf(fabsf(d2f_rn(n0y)), fabsf(d2f_rn(n0z))));
+      double lam = 0.0;
+      bool ok = false;
+      for (int it = 0; it <= S.max_newton; ++it) {
+        const GEval e = held ? thyl_geval(S, q0, xn, yn, zn) : surf_g(S, xn, yn, zn);
+        if (e.g * e.g < tol2nn) {
           ok = true;
           break;
         }
+        if (it == S.max_newton) break;
+        double dl;
+        if (S.frozen) {
+          dl = e.g * inv_a_nn;
+        } else {
+          double n1x, n1y, n1z;
+          surf_n(S, e, n1x, n1y, n1z);
+          dl = e.g * nr_rcp(a * fma(n1x, n0x, fma(n1y, n0y, n1z * n0z)));
+        }
+        lam += dl;
+        const double al = a * lam;
+        xn = fma(-al, n0x, yx); yn = fma(-al, n0y, yy); zn = fma(-al, n0z, yz);
+        if (it > 0) {  // round-off floor: the update is below 4 ulp of the position
+          const float step = fabsf(d2f_rn(dl)) * af * n0max;
+          const float xmax = fmaxf(fabsf(d2f_rn(xn)), fmaxf(fabsf(d2f_rn(yn)), fabsf(d2f_rn(zn))));
+          if (step <= 4.f * (float)DBL_EPSILON * xmax) {
+            ok = true;
+            break;
+          }
+        }
       }
+      if (!ok) flag(A.status, kFlagRattle);
+      const double hl = h * lam;
+      qx = fma(-hl, n0x, qx); qy = fma(-hl, n0y, qy); qz = fma(-hl, n0z, qz);
     }
-    if (!ok) flag(A.status, kFlagRattle);
-    const double hl = h * lam;
-    qx = fma(-hl, n0x, qx); qy = fma(-hl, n0y, qy); qz = fma(-hl, n0z, qz);
   }
   if (!(finite_bits(xn) && finite_bits(yn) && finite_bits(zn) && finite_bits(qx) && finite_bits(qy) &&
         finite_bits(qz)))
@@ -3018,7 +3290,7 @@ __device__ __forceinline__ void integrate_particle_fp64(const DevArrays& A, int6
 template <bool COMPOSED, class Bin>
 __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int64_t i, Force3<float> fr_in,
                                                          unsigned long long k, int mode, const Bin& bin,
-                                                         float4* xi = nullptr, bool xi_prev = false) {
+                                                         bool xi_store = false, bool xi_prev = false) {
   const int64_t n = A.n;
   const uint32_t m = A.meta[i];
   const SysDev& S = A.sys[meta_sys(m)];
@@ -3027,7 +3299,8 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
   const double px = A.ph[i], py = A.ph[n + i], pz = A.ph[2 * n + i];
   const DF P[3] = {df_from(px), df_from(py), df_from(pz)};  // the high parts are p rounded to float32
   Force3<float> F =
-      combine<float>(S, A.types, ty, (uint32_t)(i - S.first), k, mode, fr_in, P[0].h, P[1].h, P[2].h, xi, xi_prev);
+      combine<float>(S, A.types, ty, (uint32_t)(i - S.first), k, mode, fr_in, P[0].h, P[1].h, P[2].h,
+                     NoiseSlot<float>(A.noise, n, i), xi_store, xi_prev);
   if (S.kind == kXY2D) F.z = 0.f;  // 2D plane: no z update
   double xn, yn, zn, qx, qy, qz;
   if (meta_con(m)) {
@@ -3060,32 +3333,32 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
 // COMPOSED (mixed path): some system's surface is a Gaussian bump or a
 // thylakoid composite (DevArrays::composed).
 template <typename R, bool COMPOSED>
-__global__ void __launch_bounds__(256, 4) k_integrate_nl(DevArrays A) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate_nl(DevArrays A) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   const unsigned long long k = *A.step;
   const int mode = *A.mode;
   const NlSink<R> bin(A);
-  if constexpr (sizeof(R) == 4) {
-    const bool store = A.noise && A.store_noise;
-    float4* xi = store ? A.noise + i : nullptr;
-    const bool xi_prev = store && k > 0ull && *A.noise_k == k - 1ull;  // ~0: none stored
-    integrate_particle_mixed<COMPOSED>(A, i, load_f3<float>(A.f, i), k, mode, bin, xi, xi_prev);
-  } else {
-    integrate_particle_fp64(A, i, load_f3<double>(A.f, i), k, mode, bin);
-  }
+  const bool store = A.noise && A.store_noise;
+  const bool prev = store && k > 0ull && *A.noise_k == k - 1ull;  // ~0: none stored
+  if constexpr (sizeof(R) == 4)
+    integrate_particle_mixed<COMPOSED>(A, i, load_f3<float>(A.f, i), k, mode, bin, store, prev);
+  else integrate_particle_fp64(A, i, load_f3<double>(A.f, i), k, mode, bin, store, prev);
 }
 
 template <typename R, bool BIN, bool COMPOSED>
-__global__ void __launch_bounds__(256, 4) k_integrate(DevArrays A) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate(DevArrays A) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   const unsigned long long k = *A.step;
   const int mode = *A.mode;
   using Bin = typename std::conditional<BIN, GlobalBin, NoBin>::type;
   const Bin bin(A);
-  if constexpr (sizeof(R) == 4) integrate_particle_mixed<COMPOSED>(A, i, load_f3<float>(A.f, i), k, mode, bin);
-  else integrate_particle_fp64(A, i, load_f3<double>(A.f, i), k, mode, bin);
+  const bool store = A.noise && A.store_noise;
+  const bool prev = store && k > 0ull && *A.noise_k == k - 1ull;
+  if constexpr (sizeof(R) == 4)
+    integrate_particle_mixed<COMPOSED>(A, i, load_f3<float>(A.f, i), k, mode, bin, store, prev);
+  else integrate_particle_fp64(A, i, load_f3<double>(A.f, i), k, mode, bin, store, prev);
 }
 
 // ---------------------------------------------------------------------------
@@ -3242,8 +3515,8 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 2) k_resident(DevArrays A
       bin.put(i, cell);
     }
     __syncthreads();
-    resident_cells<R>(A, S, first, n, T, s_start, s_cell, cstride, s_rank, s_tmp, s_stag, s_scell, s_rec, s_lo,
-                      warp_tot);
+    resident_cells<R>(A, S, first, n, T, s_start, s_cell, cstride, s_rank, s_tmp, s_stag, s_scell, s_rec,
+                      sizeof(R) == 4 ? s_lo : nullptr, warp_tot);
     for (int j = 0; j < J.nsteps; ++j) {
       for (uint32_t s = tid; s < n; s += bd) {
         R fx, fy, fz, u;
@@ -3275,7 +3548,7 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 2) k_resident(DevArrays A
       // the last step's list would only be rebuilt by the next launch
       if (j + 1 < J.nsteps)
         resident_cells<R>(A, S, first, n, T, s_start, s_cell, cstride, s_rank, s_tmp, s_stag, s_scell, s_rec,
-                          s_lo, warp_tot);
+                          sizeof(R) == 4 ? s_lo : nullptr, warp_tot);
     }
   }
 }
@@ -3376,7 +3649,8 @@ int resident_blocks_per_sm(int precision, int bonds, int walls, int excl, uint32
   return e == cudaSuccess ? per_sm : 0;
 }
 
-__global__ void k_advance(unsigned long long* step, int32_t* mode) {
+__global__ void k_advance(unsigned long long* step, int32_t* mode, unsigned long long* noise_k) {
+  if (noise_k) *noise_k = *step;  // this step's normals are stored
   *step += 1ull;
   *mode = 1;
 }
@@ -3401,7 +3675,7 @@ __global__ void k_finish(DevArrays A) {
   const double x = A.x[i], y = A.x[n + i], z = A.x[2 * n + i];
   double px = A.ph[i], py = A.ph[n + i], pz = A.ph[2 * n + i];
   Force3<R> Fr = combine<R>(S, A.types, ty, (uint32_t)(i - S.first), k, 1, load_f3<R>(A.f, i), (R)px, (R)py,
-                            (R)pz);
+                            (R)pz, NoiseSlot<R>(A.noise, n, i), false, false);
   if (S.kind == kXY2D) Fr.z = (R)0;
   const bool con = meta_con(m);
   double nx = 0.0, ny = 0.0, nz = 0.0, inv_nn = 0.0;
@@ -3757,8 +4031,42 @@ static void pair_dispatch(const DevArrays& A, int bonds, int walls, int excl, in
   }
 }
 
+template <bool ENERGY>
+static void pair_dispatch_nlq64(const DevArrays& A, int bonds, int walls, cudaStream_t st) {
+  const int64_t warps = (A.n + A.list_warp - 1) / A.list_warp;
+  const unsigned g = (unsigned)((warps + kQueueWarps - 1) / kQueueWarps);
+  const int b = kQueueWarps * 32;
+  switch ((bonds ? 2 : 0) | (walls ? 1 : 0)) {
+    case 0: k_pair_nlq64<false, false, ENERGY><<<g, b, 0, st>>>(A); break;
+    case 1: k_pair_nlq64<false, true, ENERGY><<<g, b, 0, st>>>(A); break;
+    case 2: k_pair_nlq64<true, false, ENERGY><<<g, b, 0, st>>>(A); break;
+    default: k_pair_nlq64<true, true, ENERGY><<<g, b, 0, st>>>(A); break;
+  }
+}
+
+// Particles per warp of the list walks (the same bits for any): at most
+// MD_OPT_LIST_WARP, fewer on small systems, whose walk is one wave of long
+// sequences, and up to twice the size where lists are long (max_neighbors >=
+// 128). Mixed path, 32 / 16 / 8 per warp, us: sphere of 1,000 11.4 / 9.2 / 8.6,
+// 40,000 9.7 / 9.9 / 13.4; bead molecules, 10,000 15.0 / 13.1 / 11.6, 40,000
+// 17.4 / 15.8 / 17.9; liquid of 27,000 187 / 111 / 71.
+static int32_t list_warp_of(const DevArrays& A) {
+  const int64_t n = A.nl_max >= 128 ? A.n / 2 : A.n;
+  return std::min(A.list_warp, n <= 16384 ? 8 : n <= 32768 ? 16 : 32);
+}
+
+// energy = 0 (a step's forces): the float64 list walk leaves the pair energies out.
 template <typename R>
-static void pair_dispatch_nl(const DevArrays& A, int bonds, int walls, cudaStream_t st) {
+static void pair_dispatch_nl(const DevArrays& H, int bonds, int walls, int energy, cudaStream_t st) {
+  DevArrays A = H;
+  A.list_warp = list_warp_of(H);
+  if constexpr (sizeof(R) == 8) {
+    if (A.pair_queue) {
+      if (energy) pair_dispatch_nlq64<true>(A, bonds, walls, st);
+      else pair_dispatch_nlq64<false>(A, bonds, walls, st);
+      return;
+    }
+  }
   const unsigned g = grid_for(A.n, 256);
   if constexpr (sizeof(R) == 4) {
     if (A.pair_queue) {
@@ -3794,12 +4102,12 @@ cudaError_t launch_nl_build(const DevArrays& A, int precision, int excl, cudaStr
   return cudaGetLastError();
 }
 
-cudaError_t launch_pair(const DevArrays& A, int precision, int has_pairs, int bonds, int walls, int excl,
+cudaError_t launch_pair(const DevArrays& A, int precision, int has_pairs, int bonds, int walls, int excl, int energy,
                         cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
   if (has_pairs && A.nl_dirty) {
-    if (precision == 0) pair_dispatch_nl<double>(A, bonds, walls, st);
-    else pair_dispatch_nl<float>(A, bonds, walls, st);
+    if (precision == 0) pair_dispatch_nl<double>(A, bonds, walls, energy, st);
+    else pair_dispatch_nl<float>(A, bonds, walls, energy, st);
     return cudaGetLastError();
   }
   if (!has_pairs) {
@@ -3844,7 +4152,7 @@ cudaError_t launch_integrate(const DevArrays& A, int precision, int has_pairs, c
 }
 
 cudaError_t launch_advance(const DevArrays& A, cudaStream_t st) {
-  k_advance<<<1, 1, 0, st>>>(A.step, A.mode);
+  k_advance<<<1, 1, 0, st>>>(A.step, A.mode, A.noise_k);
   return cudaGetLastError();
 }
 

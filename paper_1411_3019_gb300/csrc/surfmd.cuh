@@ -111,14 +111,14 @@ struct SysDev {
 
 // Pair tables shared by all systems of a handle (symmetric).
 struct TypeTable {
-  double eps[kMaxTypes][kMaxTypes];
-  double sig2[kMaxTypes][kMaxTypes];
+  double c24[kMaxTypes][kMaxTypes];  // 24 eps sigma^6
+  double c48[kMaxTypes][kMaxTypes];  // 48 eps sigma^12
+  double c4[kMaxTypes][kMaxTypes];   // 4 eps sigma^6
+  double c4b[kMaxTypes][kMaxTypes];  // 4 eps sigma^12
   double rc2[kMaxTypes][kMaxTypes];
   double shift[kMaxTypes][kMaxTypes];  // phi(r_c)
   double lin[kMaxTypes][kMaxTypes];    // phi'(r_c) for the linearly smoothed form, else 0
   double rc[kMaxTypes][kMaxTypes];
-  float eps_f[kMaxTypes][kMaxTypes];
-  float sig2_f[kMaxTypes][kMaxTypes];
   float rc2_f[kMaxTypes][kMaxTypes];
   float shift_f[kMaxTypes][kMaxTypes];
   float lin_f[kMaxTypes][kMaxTypes];
@@ -195,10 +195,10 @@ struct DevArrays {
   uint32_t* nl_pk;
   uint32_t* nl_off;     // [n] start of a slot's entries within its group's run
   uint32_t* smeta;      // [n] meta of each sorted slot (written with the records at a rebuild), or null
-  // mixed path with the list: the unit normals xi^k of the last integrated
-  // step k (by particle; the next step's force combination needs them again)
-  // and that step, ~0 when none is stored (after a state is set)
-  float4* noise;
+  // the unit normals xi^k of the last integrated step k (by particle; the next
+  // step's force combination needs them again; float4, or three float64 arrays
+  // on the float64 path) and that step, ~0 when none is stored (after a state is set)
+  void* noise;
   unsigned long long* noise_k;
   int32_t store_noise;  // 1: store and reuse the normals (MD_OPT_STORE_NOISE), 0: draw both steps' again
   void* rec0;           // [n] records at the last build, by particle
@@ -230,7 +230,8 @@ struct DevArrays {
   uint32_t* stag_tmp;   // [n] slot -> particle in atomic order (before the canonical sort)
   uint32_t* scell;      // [n] sorted slot -> cell id
   void* rec;            // [n] float4 / double4_32a cell-relative offsets + type/mol bits
-  float4* rec_lo;       // [n] mixed path: offset - record (the low parts; w unused), else null
+  float4* rec_lo;       // [n] mixed path: offset - record (the low parts; w unused); float64 path with the
+                        // list: the record rounded to float32 (the list walk's screen), else null
   float4* rec0_lo;      // [n] mixed path with the neighbour list: rec_lo at the last build, by particle
   int32_t ntypes;       // particle types in use (a type must lie in [0, ntypes))
   uint32_t spin_limit;  // reads of a predecessor's scan word before the wait gives up

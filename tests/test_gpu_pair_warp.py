@@ -39,7 +39,7 @@ def _forces(systems):
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("kind,n", [("sphere", 5), ("sphere", 1000), ("sphere", 8192), ("crowded", 33), ("crowded", 700),
-                                    ("liquid", 9), ("liquid", 16), ("smooth", 500), ("beads", 200), ("bump", 6000)])
+                                    ("liquid", 9), ("liquid", 12), ("smooth", 500), ("beads", 200), ("bump", 6000)])
 def test_same_bits_as_the_row_kernel(kind, n, precision):
     s = _system(kind, n, precision)
     assert s["n"] <= LIMIT[precision]
