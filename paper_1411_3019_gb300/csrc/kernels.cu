@@ -66,8 +66,8 @@ __device__ __forceinline__ void gauss3(uint32_t seed, uint32_t rep, uint32_t pid
 #if SURFMD_FAST_NOISE
   const float two_pi = 6.28318530717958648f;
   // (near u = 1 the fast logarithm's absolute error can exceed -ln u: clamp at 0)
-  const float r01 = sqrtf(fmaxf(-2.0f * __logf(u0), 0.0f));
-  const float r23 = sqrtf(fmaxf(-2.0f * __logf(u2), 0.0f));
+  const float r01 = sqrt_approx(fmaxf(-2.0f * __logf(u0), 0.0f));
+  const float r23 = sqrt_approx(fmaxf(-2.0f * __logf(u2), 0.0f));
   float sn, cs;
   __sincosf(two_pi * (u1 - 0.5f), &sn, &cs);
   gx = __fmul_rn(-r01, cs);  // rounded here, also where the next step's sum would take the product into an FMA:
@@ -149,17 +149,17 @@ __device__ __forceinline__ double f2d(float v) {
 // float64 -> double-float on the integer pipe: h = v rounded to float32 (as
 // d2f_rn) and l = the rest, for v = 0 or 2^-80 <= |v| < 2^128 (ok says so).
 // The fraction is cut after 23 bits (t) and the cut bits, an integer of units
-// 2^(E-1075) of v's binade (E = v's biased exponent), keep their leading 23:
-// rest >> 6 < 2^23, exact in float32 by the 2^23 bias, times 2^(E-1069); one
-// fast_two_sum then moves the rounding of h into place. h + l = v within
-// 2^-46 |v|.
+// 2^(E-1075) of v's binade (E = v's biased exponent), are rounded to 23 bits:
+// (rest + 32) >> 6 <= 2^23, exact in float32 by the 2^23 bias, times 2^(E-1069);
+// one fast_two_sum then moves the rounding of h into place. h + l = v within
+// 2^-47 |v|.
 __device__ __forceinline__ DF df_from_fast(double v, bool& ok) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
   const uint32_t e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
   const bool zero = ((hi << 1) | lo) == 0u;
   ok = ok && (e - 943u < 208u || zero);
   const uint32_t t = __funnelshift_l(lo, hi & 0x7fffffffu, 3) - 0xC0000000u;  // 896 << 23 modulo 2^32
-  const float k = __fsub_rn(__uint_as_float(0x4B000000u | ((lo >> 6) & 0x7fffffu)), 8388608.0f);
+  const float k = __fsub_rn(__uint_as_float(0x4B000000u + (((lo & 0x1fffffffu) + 32u) >> 6)), 8388608.0f);
   const DF r = df_fast_sum(__uint_as_float(sign | t), __fmul_rn(k, __uint_as_float(sign | ((e - 942u) << 23))));
   return zero ? DF{__uint_as_float(hi), 0.f} : r;
 }
@@ -3081,11 +3081,13 @@ template <typename R> struct NlSink {
     float d2;
     if constexpr (sizeof(R) == 4) {
       const float4 l = rec0_lo[i];
-      const DF ex = df_from(dx), ey = df_from(dy), ez = df_from(dz);
-      const DF ox = df_add(DF{r.x, l.x}, ex), oy = df_add(DF{r.y, l.y}, ey), oz = df_add(DF{r.z, l.z}, ez);
+      const double dv[3] = {dx, dy, dz};
+      DF e[3];
+      df_from3(dv, e);
+      const DF ox = df_add(DF{r.x, l.x}, e[0]), oy = df_add(DF{r.y, l.y}, e[1]), oz = df_add(DF{r.z, l.z}, e[2]);
       r.x = ox.h; r.y = oy.h; r.z = oz.h;
       rec_lo[s] = make_float4(ox.l, oy.l, oz.l, 0.f);
-      d2 = fmaf(ex.h, ex.h, fmaf(ey.h, ey.h, ez.h * ez.h));
+      d2 = fmaf(e[0].h, e[0].h, fmaf(e[1].h, e[1].h, e[2].h * e[2].h));
     } else {
       r.x += dx; r.y += dy; r.z += dz;
       const float ex = d2f_rn(dx), ey = d2f_rn(dy), ez = d2f_rn(dz);
@@ -3297,14 +3299,16 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
   const uint32_t ty = meta_type(m);
   const double x = A.x[i], y = A.x[n + i], z = A.x[2 * n + i];
   const double px = A.ph[i], py = A.ph[n + i], pz = A.ph[2 * n + i];
-  const DF P[3] = {df_from(px), df_from(py), df_from(pz)};  // the high parts are p rounded to float32
+  const double pv[3] = {px, py, pz};
+  DF P[3];
+  df_from3(pv, P);  // the high parts are p rounded to float32
   Force3<float> F =
       combine<float>(S, A.types, ty, (uint32_t)(i - S.first), k, mode, fr_in, P[0].h, P[1].h, P[2].h,
                      NoiseSlot<float>(A.noise, n, i), xi_store, xi_prev);
   if (S.kind == kXY2D) F.z = 0.f;  // 2D plane: no z update
   double xn, yn, zn, qx, qy, qz;
   if (meta_con(m)) {
-    const double xv[3] = {x, y, z}, pv[3] = {px, py, pz};
+    const double xv[3] = {x, y, z};
     const float Fv[3] = {F.x, F.y, F.z};
     double xo[3], qo[3];
     position_half_df<COMPOSED>(S, ty, mode, xv, pv, P, Fv, A.status, xo, qo);

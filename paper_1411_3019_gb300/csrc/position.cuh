@@ -52,7 +52,7 @@ struct DFTorusEval {
   }
   // n1.n0 = 2 (rho - R)/rho (e_xy . n0_xy) + 2 e_z n0_z
   __device__ __forceinline__ float n1n0(const DF N[3]) const {
-    return 2.f * ttf / rhof * fmaf(e0, N[0].h, e1 * N[1].h) + 2.f * e2 * N[2].h;
+    return 2.f * ttf * rcp_approx(rhof) * fmaf(e0, N[0].h, e1 * N[1].h) + 2.f * e2 * N[2].h;
   }
 };
 
@@ -188,11 +188,11 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
                                                  uint32_t* status, double xo[3], double qo[3]) {
   DF C[3], D[3], N[3], T[3];  // x - c, y - c, n0, y - x
   const DF kick = mode ? S.dt_df : S.half_dt_df;
+  df_from3(xv, C);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const DF q0 = df_add(P[d], df_mul_f(kick, F[d]));  // q0 = p + kick F
-    const DF X = df_from(xv[d]);
-    C[d] = S.c_zero ? X : df_sub(X, S.c_df[d]);
+    if (!S.c_zero) C[d] = df_sub(C[d], S.c_df[d]);
     T[d] = df_mul(S.dtm_df[ty], q0);
   }
   float pf[3] = {P[0].h, P[1].h, P[2].h}, Ff[3] = {F[0], F[1], F[2]};
@@ -285,19 +285,20 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
     float sp = 0.f;
 #pragma unroll
     for (int d = 0; d < 3; ++d) sp = fmaf(N[d].h, fmaf(S.half_dt_f, Ff[d], pf[d]), sp);
-    mu0 = S.dtm_f[ty] * sp / nnf;
+    mu0 = S.dtm_f[ty] * sp * rcp_approx(nnf);
   }
-  const float tol_n = 0.99f * S.tol_f * sqrtf(nnf);
+  const float tol_n = 0.99f * S.tol_f * sqrt_approx(nnf);
   // round-off floor: an update below 4 units of the double-float resolution of the position
   const float dmax = fmaxf(fabsf(D[0].h), fmaxf(fabsf(D[1].h), fabsf(D[2].h)));
-  const float floor_mu = 4.f * 0x1p-47f * dmax / fmaxf(fabsf(N[0].h), fmaxf(fabsf(N[1].h), fabsf(N[2].h)));
+  const float floor_mu =
+      4.f * 0x1p-47f * dmax * rcp_approx(fmaxf(fabsf(N[0].h), fmaxf(fabsf(N[1].h), fabsf(N[2].h))));
   const bool torus = shape == kTorus, bump = COMPOSED && shape == kBump, line = !torus && !bump;
   int it = 0;
   if (line) {  // float32 Newton on the line form g(y) - b mu + c mu^2
     for (; it < S.max_newton; ++it) {
       const float gf = fmaf(fmaf(c, mu0, -b.h), mu0, gy.h);
       if (fabsf(gf) < 0.5f * tol_n) break;
-      const float dmu = gf * __frcp_rn(S.frozen ? nnf : fmaf(-2.f * mu0, c, b.h));
+      const float dmu = gf * rcp_approx(S.frozen ? nnf : fmaf(-2.f * mu0, c, b.h));
       mu0 += dmu;
       if (fabsf(dmu) <= 0x1p-22f * fabsf(mu0)) {
         ++it;
@@ -314,7 +315,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
     if (fabsf(g.h) < tol_n) { ok = true; break; }
     if (it >= S.max_newton) break;
     const float den = S.frozen ? nnf : (torus ? Q.n1n0(N) : (bump ? B.n1n0(N) : fmaf(-2.f * mu.h, c, b.h)));
-    const float dmu = g.h * __frcp_rn(den);
+    const float dmu = g.h * rcp_approx(den);
     mu = df_add_f(mu, dmu);
     if (it > 0 && fabsf(dmu) <= floor_mu) { ok = true; break; }
   }
