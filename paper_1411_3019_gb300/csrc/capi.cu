@@ -45,7 +45,9 @@ struct md_handle {
   double* d_obs = nullptr;
   uint32_t* h_status = nullptr;  // pinned
   unsigned long long* h_resid = nullptr;  // pinned
-  cudaGraphExec_t graph = nullptr;
+  cudaGraphExec_t graph = nullptr;        // one step
+  cudaGraphExec_t graph_block = nullptr;  // kBlockSteps steps (built once a handle has run for a while)
+  int64_t steps_run = 0;                  // steps replayed by the graphs
   // visiting order of the pair kernel (refreshed every kOrderEvery steps)
   DevArrays O{};
   uint32_t order_coord_shift = 0, order_morton_drop = 0, order_sys_shift = 0;
@@ -77,6 +79,11 @@ struct md_handle {
 };
 
 static std::string g_create_err;
+// Steps of the longer graph: consecutive graph launches are ordered end to
+// start, while the kernels inside one graph overlap their launches. It is built
+// when a handle has run kBlockAfter steps, so that a short run does not pay for
+// it (about 0.1 ms).
+constexpr int64_t kBlockSteps = 8, kBlockAfter = 64;
 constexpr int64_t kOrderEvery = 16;  // steps between refreshes of the pair visiting order
 
 namespace {
@@ -521,31 +528,41 @@ cudaError_t enqueue_step(md_handle* h, cudaStream_t st) {
   return cudaSuccess;
 }
 
+// The captured steps no longer match the handle's settings.
+void drop_graphs(md_handle* h) {
+  if (h->graph) cudaGraphExecDestroy(h->graph);
+  if (h->graph_block) cudaGraphExecDestroy(h->graph_block);
+  h->graph = h->graph_block = nullptr;
+  h->steps_run = 0;
+}
+
+// Captures `steps` time steps into *out.
+cudaError_t capture_steps(md_handle* h, int64_t steps, cudaGraphExec_t* out) {
+  cudaGraph_t g = nullptr;
+  cudaError_t e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
+  for (int64_t s = 0; s < steps && e == cudaSuccess; ++s) e = enqueue_step(h, h->cap_stream);
+  const cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
+  if (e == cudaSuccess) e = e2;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+  if (g) cudaGraphDestroy(g);
+  if (e != cudaSuccess) *out = nullptr;
+  return e;
+}
+
 int build_graph(md_handle* h) {
   if (h->graph) return MD_OK;
   if (h->has_pairs && h->A.nl_dirty && h->fused_rebuild && h->rebuild_ctas == 0) {
     h->rebuild_ctas = rebuild_blocks(h->precision, h->excl, h->n);
     if (h->rebuild_ctas <= 0) h->fused_rebuild = 0;  // not launchable here: five separate launches
   }
-  cudaGraph_t g = nullptr;
-  CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = enqueue_step(h, h->cap_stream);
-  cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
-  if (e == cudaSuccess && e2 == cudaSuccess) {
-    e = cudaGraphInstantiate(&h->graph, g, 0);
-    cudaGraphDestroy(g);
-  } else if (g) {
-    cudaGraphDestroy(g);
-  }
-  const cudaError_t failed = e != cudaSuccess ? e : e2;
-  if (failed != cudaSuccess && h->A.nl_dirty && h->fused_rebuild) {
+  const cudaError_t e = capture_steps(h, 1, &h->graph);
+  if (e != cudaSuccess && h->A.nl_dirty && h->fused_rebuild) {
     // a cooperative launch that cannot be captured here: the separate rebuild kernels instead
     cudaGetLastError();
-    h->graph = nullptr;
     h->fused_rebuild = 0;
     return build_graph(h);
   }
-  if (e2 != cudaSuccess) return cuda_fail(h, e2, "capture of one step");
   if (e != cudaSuccess) return cuda_fail(h, e, "capture or instantiation of one step");
   return MD_OK;
 }
@@ -1112,10 +1129,21 @@ int md_step(md_handle* h, int64_t nsteps) {
   if (h->engine == 1) return resident_steps(h, nsteps);
   rc = build_graph(h);
   if (rc) return rc;
+  const bool ordered = h->has_pairs && h->A.order && !h->A.nl_dirty;  // the visiting order is refreshed between steps
   int64_t extra = 0;
-  for (int64_t s = 0; s < nsteps; ++s) {
-    CK(h, cudaGraphLaunch(h->graph, h->stream()));
-    if (h->has_pairs && h->A.order && !h->A.nl_dirty && ++h->steps_since_order >= kOrderEvery) {
+  for (int64_t s = 0; s < nsteps;) {
+    int64_t chunk = 1;
+    const int64_t room = std::min(nsteps - s, ordered ? kOrderEvery - h->steps_since_order : nsteps);
+    if (room >= kBlockSteps && h->steps_run >= kBlockAfter) {
+      if (!h->graph_block) CK(h, capture_steps(h, kBlockSteps, &h->graph_block));
+      chunk = kBlockSteps;
+    }
+    CK(h, cudaGraphLaunch(chunk == 1 ? h->graph : h->graph_block, h->stream()));
+    s += chunk;
+    h->steps_run += chunk;
+    if (!ordered) continue;
+    h->steps_since_order += chunk;
+    if (h->steps_since_order >= kOrderEvery) {
       // any permutation is a valid visiting order; a fresh one keeps it spatial
       CK(h, launch_order(h->A, h->O, h->order_coord_shift, h->order_morton_drop, h->order_sys_shift, h->d_order,
                      h->stream()));
@@ -1264,10 +1292,7 @@ int md_set_neighbor_list(md_handle* h, double skin, int32_t max_neighbors) {
       if (rc) return rc;
     }
   }
-  if (h->graph) {  // the captured step used the old mode
-    cudaGraphExecDestroy(h->graph);
-    h->graph = nullptr;
-  }
+  drop_graphs(h);  // the captured steps used the old setting
   return check_device_status(h);
 }
 
@@ -1347,10 +1372,7 @@ int md_set_option(md_handle* h, int32_t key, int64_t value) {
     default:
       return fail(h, MD_ERR_INVALID_ARG, "unknown option");
   }
-  if (h->graph) {  // the captured step used the old setting
-    cudaGraphExecDestroy(h->graph);
-    h->graph = nullptr;
-  }
+  drop_graphs(h);  // the captured steps used the old setting
   return MD_OK;
 }
 
@@ -1608,7 +1630,7 @@ void md_destroy(md_handle* h) {
   cudaSetDevice(h->dev);
   if (h->own_stream) cudaStreamSynchronize(h->own_stream);
   if (h->user_stream) cudaStreamSynchronize(h->user_stream);
-  if (h->graph) cudaGraphExecDestroy(h->graph);
+  drop_graphs(h);
   for (void* p : h->allocs) cudaFree(p);
   if (h->h_status) cudaFreeHost(h->h_status);
   if (h->h_resid) cudaFreeHost(h->h_resid);

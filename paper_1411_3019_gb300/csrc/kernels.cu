@@ -25,6 +25,21 @@
 namespace surfmd {
 
 
+// Programmatic dependent launch. The kernels of a step are launched so that a
+// kernel's CTAs may start, and run up to pdl_wait, while the last CTAs of the
+// kernel before it still run (griddepcontrol): the launch latency and the
+// prologue of each overlap the tail of the one before. pdl_wait returns when
+// every kernel the launch depends on has ended and its writes are visible;
+// nothing that another kernel of the step writes, and nothing that one reads,
+// is touched before it. Every kernel of the chain waits, so the order of a
+// step's kernels is the stream's.
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_enter() {
+  pdl_launch_next();
+  pdl_wait();
+}
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds, each two
 // 32x32 -> 64-bit products with the published multipliers; the key is bumped
@@ -514,6 +529,7 @@ __device__ __forceinline__ void bin_one(const DevArrays& A, int64_t i) {
 
 template <typename R>
 __global__ void k_bin(DevArrays A) {
+  pdl_enter();
   if (A.nl_dirty && *A.nl_dirty == 0u) return;  // neighbour-list mode, no rebuild this step
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < A.n) bin_one<R>(A, i);
@@ -570,6 +586,7 @@ __device__ __forceinline__ unsigned long long tile_word(uint32_t epoch, uint32_t
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_onepass(DevArrays A, int advance) {
+  pdl_enter();
   __shared__ uint32_t warp_tot[33];
   __shared__ uint32_t s_tile, s_prefix;
   uint32_t* __restrict__ count = A.count;
@@ -698,6 +715,7 @@ __device__ __forceinline__ void scatter_one(const DevArrays& A, int64_t i) {
 }
 
 __global__ void k_scatter(DevArrays A) {
+  pdl_enter();
   if (A.nl_dirty && *A.nl_dirty == 0u) return;  // neighbour-list mode, no rebuild this step
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < A.n) scatter_one(A, i);
@@ -775,6 +793,7 @@ __device__ __forceinline__ void bucket_build_one(const DevArrays& A, int64_t s) 
 
 template <typename R>
 __global__ void k_bucket_build(DevArrays A) {
+  pdl_enter();
   if (A.nl_dirty && *A.nl_dirty == 0u) return;  // neighbour-list mode, no rebuild this step
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s < A.n) bucket_build_one<R>(A, s);
@@ -869,12 +888,14 @@ __device__ __forceinline__ uint32_t order_key(const DevArrays& A, const OrderKey
 }
 
 __global__ void k_order_hist(DevArrays A, DevArrays O, OrderKey K) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   A.rank[i] = atomicAdd(&O.count[order_key(A, K, i)], 1u);
 }
 
 __global__ void k_order_scatter(DevArrays A, DevArrays O, OrderKey K, uint32_t* order) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   order[O.start[order_key(A, K, i)] + A.rank[i]] = (uint32_t)i;
@@ -1533,7 +1554,9 @@ __device__ __forceinline__ uint32_t pair_slot(const DevArrays& A, const Cells& C
 template <typename R, bool BONDS, bool WALLS, bool EXCL>
 __global__ void __launch_bounds__(256) k_pair_row(DevArrays A) {
   __shared__ PairTab<R> tab;
+  pdl_launch_next();
   load_tab<R>(tab, A.types);
+  pdl_wait();  // the table is constant; everything below may be written by the kernels before
   __syncthreads();
   const uint32_t t_id = blockIdx.x * blockDim.x + threadIdx.x;
   if (t_id >= (uint32_t)A.n) return;
@@ -1577,7 +1600,9 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_pair_warp(DevArrays A) {
   constexpr unsigned kAll = 0xffffffffu;
   __shared__ PairTab<R> tab;
   __shared__ __align__(16) PairWarp<R> buf[kPairWarps];
+  pdl_launch_next();
   load_tab<R>(tab, A.types);
+  pdl_wait();  // the table is constant; everything below may be written by the kernels before
   __syncthreads();
   const int lane = (int)(threadIdx.x & 31u);
   PairWarp<R>& W = buf[threadIdx.x >> 5];
@@ -1877,6 +1902,7 @@ __device__ __forceinline__ void nl_pack_warp(const DevArrays& A, uint32_t s, boo
 
 template <typename R, bool EXCL>
 __global__ void __launch_bounds__(256) k_nl_build(DevArrays A) {
+  pdl_enter();
   __shared__ PairTab<R> tab;
   if (*A.nl_dirty == 0u) return;  // uniform: nothing moved far enough
   if (blockIdx.x == 0 && threadIdx.x == 0) *A.nl_builds += 1ull;
@@ -1939,6 +1965,7 @@ __global__ void __launch_bounds__(kRebuildThreads) k_rebuild(DevArrays A) {
   __shared__ uint32_t warp_tot[33];
   __shared__ int s_ok;
   __shared__ uint32_t s_pre;
+  pdl_launch_next();  // (launched with full ordering itself: a cooperative launch)
   const uint32_t G = gridDim.x, tid = threadIdx.x, bd = blockDim.x;
   const bool lead = blockIdx.x == 0 && tid == 0;
   if (*A.nl_dirty == 0u) {  // uniform: nothing moved far enough; only the step advances
@@ -2048,7 +2075,9 @@ cudaError_t launch_rebuild(const DevArrays& A, int precision, int excl, int bloc
 template <typename R, bool BONDS, bool WALLS>
 __global__ void __launch_bounds__(256, SURFMD_PAIR_NL_MINB) k_pair_nl(DevArrays A) {
   __shared__ PairTab<R> tab;
+  pdl_launch_next();
   load_tab<R>(tab, A.types);
+  pdl_wait();  // the table is constant; everything below may be written by the kernels before
   if (blockIdx.x == 0 && threadIdx.x == 0) *A.nl_dirty = 0u;  // the previous step's rebuild is done
   __syncthreads();
   using Rec = typename RecT<R>::T;
@@ -2158,7 +2187,9 @@ template <bool BONDS, bool WALLS>
 __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(DevArrays A) {
   __shared__ PairTab<float> tab;
   __shared__ QueueWarp qw_all[kQueueWarps];
+  pdl_launch_next();
   load_tab<float>(tab, A.types);
+  pdl_wait();  // the table is constant; everything below may be written by the kernels before
   if (blockIdx.x == 0 && threadIdx.x == 0) *A.nl_dirty = 0u;  // the previous step's rebuild is done
   const int lane = (int)(threadIdx.x & 31u);
   QueueWarp& Q = qw_all[threadIdx.x >> 5];
@@ -2320,7 +2351,9 @@ template <bool BONDS, bool WALLS, bool ENERGY>
 __global__ void __launch_bounds__(kQueueWarps * 32) k_pair_nlq64(DevArrays A) {
   __shared__ PairTab<double> tab;
   __shared__ QueueWarp64 qw_all[kQueueWarps];
+  pdl_launch_next();
   load_tab<double>(tab, A.types);
+  pdl_wait();  // the table is constant; everything below may be written by the kernels before
   if (blockIdx.x == 0 && threadIdx.x == 0) *A.nl_dirty = 0u;  // the previous step's rebuild is done
   const int lane = (int)(threadIdx.x & 31u);
   QueueWarp64& Q = qw_all[threadIdx.x >> 5];
@@ -2469,6 +2502,7 @@ __global__ void __launch_bounds__(kQueueWarps * 32) k_pair_nlq64(DevArrays A) {
 // Bend-angle forces (and energy shares) added to the pair kernel's output.
 template <typename R>
 __global__ void k_bend(DevArrays A) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   const SysDev& S = A.sys[meta_sys(A.meta[i])];
@@ -2489,7 +2523,9 @@ __global__ void k_bend(DevArrays A) {
 template <typename R, bool BONDS, bool WALLS, bool EXCL, int L>
 __global__ void __launch_bounds__(256) k_pair_lanes(DevArrays A) {
   __shared__ PairTab<R> tab;
+  pdl_launch_next();
   load_tab<R>(tab, A.types);
+  pdl_wait();  // the table is constant; everything below may be written by the kernels before
   __syncthreads();
   const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t s = (uint32_t)(g / L);
@@ -2795,7 +2831,9 @@ __global__ void __launch_bounds__(kTileWarps * 32, sizeof(R) == 4 ? 6 : 4) k_pai
   __shared__ Rec stage_all[kTileWarps][tile_cap<R>()];
   __shared__ uint32_t code_all[kTileWarps][tile_cap<R>()];
   __shared__ typename V4<R>::T f_all[kTileWarps][kTileSlots];
+  pdl_launch_next();
   load_tab<R>(tab, A.types);
+  pdl_wait();  // the table is constant; everything below may be written by the kernels before
   __syncthreads();
   const int lane = (int)(threadIdx.x & 31u);
   const uint32_t wib = threadIdx.x >> 5;
@@ -2838,6 +2876,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, sizeof(R) == 4 ? 6 : 4) k_pai
 // No pair term anywhere: only bonds and walls, in particle order.
 template <typename R>
 __global__ void k_nopair(DevArrays A, int bonds, int walls) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   const uint32_t m = A.meta[i];
@@ -3338,6 +3377,7 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
 // thylakoid composite (DevArrays::composed).
 template <typename R, bool COMPOSED>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate_nl(DevArrays A) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   const unsigned long long k = *A.step;
@@ -3352,6 +3392,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate_nl(De
 
 template <typename R, bool BIN, bool COMPOSED>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate(DevArrays A) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   const unsigned long long k = *A.step;
@@ -3654,6 +3695,7 @@ int resident_blocks_per_sm(int precision, int bonds, int walls, int excl, uint32
 }
 
 __global__ void k_advance(unsigned long long* step, int32_t* mode, unsigned long long* noise_k) {
+  pdl_enter();
   if (noise_k) *noise_k = *step;  // this step's normals are stored
   *step += 1ull;
   *mode = 1;
@@ -3664,6 +3706,7 @@ __global__ void k_advance(unsigned long long* step, int32_t* mode, unsigned long
 // normal at x^k in both precisions.
 template <typename R>
 __global__ void k_finish(DevArrays A) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t n = A.n;
   if (i >= n) return;
@@ -3695,6 +3738,7 @@ __global__ void k_finish(DevArrays A) {
 // read-out
 // ---------------------------------------------------------------------------
 __global__ void k_get_state(DevArrays A, double* xa, double* va, double* pa) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t n = A.n;
   if (i >= n) return;
@@ -3708,6 +3752,7 @@ __global__ void k_get_state(DevArrays A, double* xa, double* va, double* pa) {
 
 template <typename R>
 __global__ void k_get_forces(DevArrays A, double* fa, double* ua) {
+  pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   using V = typename V4<R>::T;
@@ -3850,6 +3895,28 @@ __global__ void k_observables(DevArrays A, double* obs) {
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
+// Launch with programmatic dependent launch allowed (see pdl_wait) for grids of
+// up to kPdlThreads threads. Larger ones gain nothing from a hidden launch
+// latency and lose where a kernel's first CTAs start under the shared-memory
+// split of the kernel before. Microseconds a step without and with it (and the
+// blocks of steps of capi.cu): 1,000 particles in float64 27.5 and 24.0, 100,000
+// bead molecules 38.2 and 36.7, 250,000 38.6 and 36.0, but 588,000 85.2 and 86.5,
+// a million 134.5 and 137.6.
+constexpr int64_t kPdlThreads = 400000;
+template <class... P, class... Q>
+static cudaError_t go(void (*kernel)(P...), unsigned grid, int block, cudaStream_t st, Q... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = (int64_t)grid * block <= kPdlThreads ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 static inline unsigned grid_for(int64_t n, int block) { return (unsigned)((n + block - 1) / block); }
 
 // Threads per block of the per-particle step kernels: 256, or fewer (a
@@ -3890,8 +3957,8 @@ cudaError_t launch_restore(const DevArrays& A, const double* d_x, const double* 
 cudaError_t launch_bin(const DevArrays& A, int precision, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
   const int b = block_for(A.n);
-  if (precision == 0) k_bin<double><<<grid_for(A.n, b), b, 0, st>>>(A);
-  else k_bin<float><<<grid_for(A.n, b), b, 0, st>>>(A);
+  if (precision == 0) go(k_bin<double>, grid_for(A.n, b), b, st, A);
+  else go(k_bin<float>, grid_for(A.n, b), b, st, A);
   return cudaGetLastError();
 }
 
@@ -3900,13 +3967,13 @@ static inline uint32_t scan_blocks_of(const DevArrays& A) {
 }
 
 cudaError_t launch_scan(const DevArrays& A, int advance, cudaStream_t st) {
-  k_scan_onepass<<<scan_blocks_of(A), kScanThreads, 0, st>>>(A, advance);
+  go(k_scan_onepass, scan_blocks_of(A), kScanThreads, st, A, advance);
   return cudaGetLastError();
 }
 
 cudaError_t launch_scatter(const DevArrays& A, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
-  k_scatter<<<grid_for(A.n, block_for(A.n)), block_for(A.n), 0, st>>>(A);
+  go(k_scatter, grid_for(A.n, block_for(A.n)), block_for(A.n), st, A);
   return cudaGetLastError();
 }
 
@@ -3914,11 +3981,11 @@ cudaError_t launch_order(const DevArrays& A, const DevArrays& O, uint32_t coord_
                          uint32_t sys_shift, uint32_t* order, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
   const OrderKey K{coord_shift, morton_drop, sys_shift};
-  k_order_hist<<<grid_for(A.n, 256), 256, 0, st>>>(A, O, K);
+  go(k_order_hist, grid_for(A.n, 256), 256, st, A, O, K);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = launch_scan(O, 0, st);
   if (e != cudaSuccess) return e;
-  k_order_scatter<<<grid_for(A.n, 256), 256, 0, st>>>(A, O, K, order);
+  go(k_order_scatter, grid_for(A.n, 256), 256, st, A, O, K, order);
   return cudaGetLastError();
 }
 
@@ -3931,8 +3998,8 @@ cudaError_t launch_cells_after_bin(const DevArrays& A, int advance, cudaStream_t
 cudaError_t launch_bucket_build(const DevArrays& A, int precision, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
   const int b = block_for(A.n);
-  if (precision == 0) k_bucket_build<double><<<grid_for(A.n, b), b, 0, st>>>(A);
-  else k_bucket_build<float><<<grid_for(A.n, b), b, 0, st>>>(A);
+  if (precision == 0) go(k_bucket_build<double>, grid_for(A.n, b), b, st, A);
+  else go(k_bucket_build<float>, grid_for(A.n, b), b, st, A);
   return cudaGetLastError();
 }
 
@@ -3942,14 +4009,14 @@ static void pair_dispatch_row(const DevArrays& A, int bonds, int walls, int excl
   const unsigned g = grid_for(A.n, b);
   const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
   switch (key) {
-    case 0: k_pair_row<R, false, false, false><<<g, b, 0, st>>>(A); break;
-    case 1: k_pair_row<R, false, false, true><<<g, b, 0, st>>>(A); break;
-    case 2: k_pair_row<R, false, true, false><<<g, b, 0, st>>>(A); break;
-    case 3: k_pair_row<R, false, true, true><<<g, b, 0, st>>>(A); break;
-    case 4: k_pair_row<R, true, false, false><<<g, b, 0, st>>>(A); break;
-    case 5: k_pair_row<R, true, false, true><<<g, b, 0, st>>>(A); break;
-    case 6: k_pair_row<R, true, true, false><<<g, b, 0, st>>>(A); break;
-    default: k_pair_row<R, true, true, true><<<g, b, 0, st>>>(A); break;
+    case 0: go(k_pair_row<R, false, false, false>, g, b, st, A); break;
+    case 1: go(k_pair_row<R, false, false, true>, g, b, st, A); break;
+    case 2: go(k_pair_row<R, false, true, false>, g, b, st, A); break;
+    case 3: go(k_pair_row<R, false, true, true>, g, b, st, A); break;
+    case 4: go(k_pair_row<R, true, false, false>, g, b, st, A); break;
+    case 5: go(k_pair_row<R, true, false, true>, g, b, st, A); break;
+    case 6: go(k_pair_row<R, true, true, false>, g, b, st, A); break;
+    default: go(k_pair_row<R, true, true, true>, g, b, st, A); break;
   }
 }
 
@@ -3967,14 +4034,14 @@ static void pair_dispatch_warp(const DevArrays& A, int bonds, int walls, int exc
   const unsigned g = grid_for(A.n, kPairWarps);
   const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
   switch (key) {
-    case 0: k_pair_warp<R, false, false, false><<<g, b, 0, st>>>(A); break;
-    case 1: k_pair_warp<R, false, false, true><<<g, b, 0, st>>>(A); break;
-    case 2: k_pair_warp<R, false, true, false><<<g, b, 0, st>>>(A); break;
-    case 3: k_pair_warp<R, false, true, true><<<g, b, 0, st>>>(A); break;
-    case 4: k_pair_warp<R, true, false, false><<<g, b, 0, st>>>(A); break;
-    case 5: k_pair_warp<R, true, false, true><<<g, b, 0, st>>>(A); break;
-    case 6: k_pair_warp<R, true, true, false><<<g, b, 0, st>>>(A); break;
-    default: k_pair_warp<R, true, true, true><<<g, b, 0, st>>>(A); break;
+    case 0: go(k_pair_warp<R, false, false, false>, g, b, st, A); break;
+    case 1: go(k_pair_warp<R, false, false, true>, g, b, st, A); break;
+    case 2: go(k_pair_warp<R, false, true, false>, g, b, st, A); break;
+    case 3: go(k_pair_warp<R, false, true, true>, g, b, st, A); break;
+    case 4: go(k_pair_warp<R, true, false, false>, g, b, st, A); break;
+    case 5: go(k_pair_warp<R, true, false, true>, g, b, st, A); break;
+    case 6: go(k_pair_warp<R, true, true, false>, g, b, st, A); break;
+    default: go(k_pair_warp<R, true, true, true>, g, b, st, A); break;
   }
 }
 
@@ -3984,14 +4051,14 @@ static void pair_dispatch_l(const DevArrays& A, int bonds, int walls, int excl, 
   const unsigned g = grid_for((int64_t)A.n * L, b);
   const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
   switch (key) {
-    case 0: k_pair_lanes<R, false, false, false, L><<<g, b, 0, st>>>(A); break;
-    case 1: k_pair_lanes<R, false, false, true, L><<<g, b, 0, st>>>(A); break;
-    case 2: k_pair_lanes<R, false, true, false, L><<<g, b, 0, st>>>(A); break;
-    case 3: k_pair_lanes<R, false, true, true, L><<<g, b, 0, st>>>(A); break;
-    case 4: k_pair_lanes<R, true, false, false, L><<<g, b, 0, st>>>(A); break;
-    case 5: k_pair_lanes<R, true, false, true, L><<<g, b, 0, st>>>(A); break;
-    case 6: k_pair_lanes<R, true, true, false, L><<<g, b, 0, st>>>(A); break;
-    default: k_pair_lanes<R, true, true, true, L><<<g, b, 0, st>>>(A); break;
+    case 0: go(k_pair_lanes<R, false, false, false, L>, g, b, st, A); break;
+    case 1: go(k_pair_lanes<R, false, false, true, L>, g, b, st, A); break;
+    case 2: go(k_pair_lanes<R, false, true, false, L>, g, b, st, A); break;
+    case 3: go(k_pair_lanes<R, false, true, true, L>, g, b, st, A); break;
+    case 4: go(k_pair_lanes<R, true, false, false, L>, g, b, st, A); break;
+    case 5: go(k_pair_lanes<R, true, false, true, L>, g, b, st, A); break;
+    case 6: go(k_pair_lanes<R, true, true, false, L>, g, b, st, A); break;
+    default: go(k_pair_lanes<R, true, true, true, L>, g, b, st, A); break;
   }
 }
 
@@ -4002,14 +4069,14 @@ static void pair_dispatch_cell(const DevArrays& A, int bonds, int walls, int exc
   const int b = kTileWarps * 32;
   const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
   switch (key) {
-    case 0: k_pair_cell<R, false, false, false><<<g, b, 0, st>>>(A); break;
-    case 1: k_pair_cell<R, false, false, true><<<g, b, 0, st>>>(A); break;
-    case 2: k_pair_cell<R, false, true, false><<<g, b, 0, st>>>(A); break;
-    case 3: k_pair_cell<R, false, true, true><<<g, b, 0, st>>>(A); break;
-    case 4: k_pair_cell<R, true, false, false><<<g, b, 0, st>>>(A); break;
-    case 5: k_pair_cell<R, true, false, true><<<g, b, 0, st>>>(A); break;
-    case 6: k_pair_cell<R, true, true, false><<<g, b, 0, st>>>(A); break;
-    default: k_pair_cell<R, true, true, true><<<g, b, 0, st>>>(A); break;
+    case 0: go(k_pair_cell<R, false, false, false>, g, b, st, A); break;
+    case 1: go(k_pair_cell<R, false, false, true>, g, b, st, A); break;
+    case 2: go(k_pair_cell<R, false, true, false>, g, b, st, A); break;
+    case 3: go(k_pair_cell<R, false, true, true>, g, b, st, A); break;
+    case 4: go(k_pair_cell<R, true, false, false>, g, b, st, A); break;
+    case 5: go(k_pair_cell<R, true, false, true>, g, b, st, A); break;
+    case 6: go(k_pair_cell<R, true, true, false>, g, b, st, A); break;
+    default: go(k_pair_cell<R, true, true, true>, g, b, st, A); break;
   }
 }
 
@@ -4041,10 +4108,10 @@ static void pair_dispatch_nlq64(const DevArrays& A, int bonds, int walls, cudaSt
   const unsigned g = (unsigned)((warps + kQueueWarps - 1) / kQueueWarps);
   const int b = kQueueWarps * 32;
   switch ((bonds ? 2 : 0) | (walls ? 1 : 0)) {
-    case 0: k_pair_nlq64<false, false, ENERGY><<<g, b, 0, st>>>(A); break;
-    case 1: k_pair_nlq64<false, true, ENERGY><<<g, b, 0, st>>>(A); break;
-    case 2: k_pair_nlq64<true, false, ENERGY><<<g, b, 0, st>>>(A); break;
-    default: k_pair_nlq64<true, true, ENERGY><<<g, b, 0, st>>>(A); break;
+    case 0: go(k_pair_nlq64<false, false, ENERGY>, g, b, st, A); break;
+    case 1: go(k_pair_nlq64<false, true, ENERGY>, g, b, st, A); break;
+    case 2: go(k_pair_nlq64<true, false, ENERGY>, g, b, st, A); break;
+    default: go(k_pair_nlq64<true, true, ENERGY>, g, b, st, A); break;
   }
 }
 
@@ -4077,19 +4144,19 @@ static void pair_dispatch_nl(const DevArrays& H, int bonds, int walls, int energ
       const int64_t warps = (A.n + A.list_warp - 1) / A.list_warp;
       const unsigned gq = (unsigned)((warps + kQueueWarps - 1) / kQueueWarps);
       switch ((bonds ? 2 : 0) | (walls ? 1 : 0)) {
-        case 0: k_pair_nlq<false, false><<<gq, kQueueWarps * 32, 0, st>>>(A); break;
-        case 1: k_pair_nlq<false, true><<<gq, kQueueWarps * 32, 0, st>>>(A); break;
-        case 2: k_pair_nlq<true, false><<<gq, kQueueWarps * 32, 0, st>>>(A); break;
-        default: k_pair_nlq<true, true><<<gq, kQueueWarps * 32, 0, st>>>(A); break;
+        case 0: go(k_pair_nlq<false, false>, gq, kQueueWarps * 32, st, A); break;
+        case 1: go(k_pair_nlq<false, true>, gq, kQueueWarps * 32, st, A); break;
+        case 2: go(k_pair_nlq<true, false>, gq, kQueueWarps * 32, st, A); break;
+        default: go(k_pair_nlq<true, true>, gq, kQueueWarps * 32, st, A); break;
       }
       return;
     }
   }
   switch ((bonds ? 2 : 0) | (walls ? 1 : 0)) {
-    case 0: k_pair_nl<R, false, false><<<g, 256, 0, st>>>(A); break;
-    case 1: k_pair_nl<R, false, true><<<g, 256, 0, st>>>(A); break;
-    case 2: k_pair_nl<R, true, false><<<g, 256, 0, st>>>(A); break;
-    default: k_pair_nl<R, true, true><<<g, 256, 0, st>>>(A); break;
+    case 0: go(k_pair_nl<R, false, false>, g, 256, st, A); break;
+    case 1: go(k_pair_nl<R, false, true>, g, 256, st, A); break;
+    case 2: go(k_pair_nl<R, true, false>, g, 256, st, A); break;
+    default: go(k_pair_nl<R, true, true>, g, 256, st, A); break;
   }
 }
 
@@ -4097,11 +4164,11 @@ cudaError_t launch_nl_build(const DevArrays& A, int precision, int excl, cudaStr
   if (A.n == 0) return cudaSuccess;
   const unsigned g = grid_for(A.n, 256);
   if (precision == 0) {
-    if (excl) k_nl_build<double, true><<<g, 256, 0, st>>>(A);
-    else k_nl_build<double, false><<<g, 256, 0, st>>>(A);
+    if (excl) go(k_nl_build<double, true>, g, 256, st, A);
+    else go(k_nl_build<double, false>, g, 256, st, A);
   } else {
-    if (excl) k_nl_build<float, true><<<g, 256, 0, st>>>(A);
-    else k_nl_build<float, false><<<g, 256, 0, st>>>(A);
+    if (excl) go(k_nl_build<float, true>, g, 256, st, A);
+    else go(k_nl_build<float, false>, g, 256, st, A);
   }
   return cudaGetLastError();
 }
@@ -4116,8 +4183,8 @@ cudaError_t launch_pair(const DevArrays& A, int precision, int has_pairs, int bo
   }
   if (!has_pairs) {
     const int b = block_for(A.n);
-    if (precision == 0) k_nopair<double><<<grid_for(A.n, b), b, 0, st>>>(A, bonds, walls);
-    else k_nopair<float><<<grid_for(A.n, b), b, 0, st>>>(A, bonds, walls);
+    if (precision == 0) go(k_nopair<double>, grid_for(A.n, b), b, st, A, bonds, walls);
+    else go(k_nopair<float>, grid_for(A.n, b), b, st, A, bonds, walls);
   } else if (precision == 0) {
     pair_dispatch<double>(A, bonds, walls, excl, A.pair_lanes, st);
   } else {
@@ -4129,8 +4196,8 @@ cudaError_t launch_pair(const DevArrays& A, int precision, int has_pairs, int bo
 cudaError_t launch_bend(const DevArrays& A, int precision, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
   const int b = block_for(A.n);
-  if (precision == 0) k_bend<double><<<grid_for(A.n, b), b, 0, st>>>(A);
-  else k_bend<float><<<grid_for(A.n, b), b, 0, st>>>(A);
+  if (precision == 0) go(k_bend<double>, grid_for(A.n, b), b, st, A);
+  else go(k_bend<float>, grid_for(A.n, b), b, st, A);
   return cudaGetLastError();
 }
 
@@ -4139,38 +4206,38 @@ cudaError_t launch_integrate(const DevArrays& A, int precision, int has_pairs, c
   const int b = block_for(A.n);
   const unsigned g = grid_for(A.n, b);
   if (A.nl_dirty && has_pairs) {
-    if (precision == 0) k_integrate_nl<double, false><<<g, b, 0, st>>>(A);
-    else if (A.composed) k_integrate_nl<float, true><<<g, b, 0, st>>>(A);
-    else k_integrate_nl<float, false><<<g, b, 0, st>>>(A);
+    if (precision == 0) go(k_integrate_nl<double, false>, g, b, st, A);
+    else if (A.composed) go(k_integrate_nl<float, true>, g, b, st, A);
+    else go(k_integrate_nl<float, false>, g, b, st, A);
   } else if (precision == 0) {
-    if (has_pairs) k_integrate<double, true, false><<<g, b, 0, st>>>(A);
-    else k_integrate<double, false, false><<<g, b, 0, st>>>(A);
+    if (has_pairs) go(k_integrate<double, true, false>, g, b, st, A);
+    else go(k_integrate<double, false, false>, g, b, st, A);
   } else if (has_pairs) {
-    if (A.composed) k_integrate<float, true, true><<<g, b, 0, st>>>(A);
-    else k_integrate<float, true, false><<<g, b, 0, st>>>(A);
+    if (A.composed) go(k_integrate<float, true, true>, g, b, st, A);
+    else go(k_integrate<float, true, false>, g, b, st, A);
   } else {
-    if (A.composed) k_integrate<float, false, true><<<g, b, 0, st>>>(A);
-    else k_integrate<float, false, false><<<g, b, 0, st>>>(A);
+    if (A.composed) go(k_integrate<float, false, true>, g, b, st, A);
+    else go(k_integrate<float, false, false>, g, b, st, A);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_advance(const DevArrays& A, cudaStream_t st) {
-  k_advance<<<1, 1, 0, st>>>(A.step, A.mode, A.noise_k);
+  go(k_advance, 1, 1, st, A.step, A.mode, A.noise_k);
   return cudaGetLastError();
 }
 
 cudaError_t launch_finish(const DevArrays& A, int precision, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
   const int b = block_for(A.n);
-  if (precision == 0) k_finish<double><<<grid_for(A.n, b), b, 0, st>>>(A);
-  else k_finish<float><<<grid_for(A.n, b), b, 0, st>>>(A);
+  if (precision == 0) go(k_finish<double>, grid_for(A.n, b), b, st, A);
+  else go(k_finish<float>, grid_for(A.n, b), b, st, A);
   return cudaGetLastError();
 }
 
 cudaError_t launch_get_state(const DevArrays& A, double* xa, double* va, double* pa, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
-  k_get_state<<<grid_for(A.n, 256), 256, 0, st>>>(A, xa, va, pa);
+  go(k_get_state, grid_for(A.n, 256), 256, st, A, xa, va, pa);
   return cudaGetLastError();
 }
 
@@ -4191,8 +4258,8 @@ cudaError_t launch_check_conversions(const double* in, int64_t n, float* out_f, 
 
 cudaError_t launch_get_forces(const DevArrays& A, int precision, double* fa, double* ua, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
-  if (precision == 0) k_get_forces<double><<<grid_for(A.n, 256), 256, 0, st>>>(A, fa, ua);
-  else k_get_forces<float><<<grid_for(A.n, 256), 256, 0, st>>>(A, fa, ua);
+  if (precision == 0) go(k_get_forces<double>, grid_for(A.n, 256), 256, st, A, fa, ua);
+  else go(k_get_forces<float>, grid_for(A.n, 256), 256, st, A, fa, ua);
   return cudaGetLastError();
 }
 
