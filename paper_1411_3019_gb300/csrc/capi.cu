@@ -402,9 +402,13 @@ bool same_interactions(const md_params& a, const md_params& b) {
   return true;
 }
 
-int check_device_status(md_handle* h) {
+// Copy of the device status word, to be waited for; report_status reads it.
+int enqueue_status(md_handle* h) {
   CK(h, cudaMemcpyAsync(h->h_status, h->A.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream()));
-  CK(h, cudaStreamSynchronize(h->stream()));
+  return MD_OK;
+}
+
+int report_status(md_handle* h) {
   const uint32_t st = *h->h_status;
   if (st == 0) return MD_OK;
   CK(h, cudaMemsetAsync(h->A.status, 0, sizeof(uint32_t), h->stream()));
@@ -423,19 +427,30 @@ int check_device_status(md_handle* h) {
   return MD_OK;
 }
 
-// Cell list of the current positions (no step advance).
-int rebuild_cells(md_handle* h) {
+int check_device_status(md_handle* h) {
+  int rc = enqueue_status(h);
+  if (rc) return rc;
+  CK(h, cudaStreamSynchronize(h->stream()));
+  return report_status(h);
+}
+
+// Cell list of the current positions (no step advance). flagged: the rebuild
+// controls are already set (launch_set_clock).
+int rebuild_cells(md_handle* h, bool flagged = false) {
   if (!h->has_pairs) return MD_OK;
-  // the fused rebuild's grid barrier starts from zero (a timed-out launch may have left arrivals)
-  CK(h, cudaMemsetAsync(h->A.gbar, 0, sizeof(GridBar), h->stream()));
-  if (h->A.nl_dirty) {  // neighbour-list mode: raise the flag so every rebuild kernel runs
-    const uint32_t one = 1u;
-    CK(h, cudaMemcpyAsync(h->A.nl_dirty, &one, sizeof(one), cudaMemcpyHostToDevice, h->stream()));
+  if (!flagged) {
+    // the fused rebuild's grid barrier starts from zero (a timed-out launch may have left arrivals)
+    CK(h, cudaMemsetAsync(h->A.gbar, 0, sizeof(GridBar), h->stream()));
+    if (h->A.nl_dirty) {  // neighbour-list mode: raise the flag so every rebuild kernel runs
+      const uint32_t one = 1u;
+      CK(h, cudaMemcpyAsync(h->A.nl_dirty, &one, sizeof(one), cudaMemcpyHostToDevice, h->stream()));
+    }
   }
   CK(h, launch_bin(h->A, h->precision, h->stream()));
   CK(h, launch_cells_after_bin(h->A, 0, h->stream()));
   CK(h, launch_bucket_build(h->A, h->precision, h->stream()));
   if (h->A.nl_dirty) CK(h, launch_nl_build(h->A, h->precision, h->excl, h->stream()));
+  if (h->A.nl_dirty) return MD_OK;  // (the list walk takes the slots in order; switching the list off comes back here)
   CK(h, launch_order(h->A, h->O, h->order_coord_shift, h->order_morton_drop, h->order_sys_shift, h->d_order,
                      h->stream()));
   h->steps_since_order = 0;
@@ -668,7 +683,19 @@ int forces_now(md_handle* h) {
 int momenta_now(md_handle* h) {
   int rc = forces_now(h);
   if (rc) return rc;
-  CK(h, launch_finish(h->A, h->precision, h->stream()));
+  CK(h, launch_finish(h->A, h->precision, nullptr, nullptr, nullptr, h->stream()));
+  return MD_OK;
+}
+
+// The state at the current step into device arrays [n][3] (any may be null).
+int read_state(md_handle* h, double* d_x, double* d_v, double* d_ph) {
+  if (d_v) {
+    int rc = forces_now(h);
+    if (rc) return rc;
+    CK(h, launch_finish(h->A, h->precision, d_x, d_v, d_ph, h->stream()));
+  } else if (d_x || d_ph) {
+    CK(h, launch_get_state(h->A, d_x, d_ph, h->stream()));
+  }
   return MD_OK;
 }
 
@@ -1056,11 +1083,8 @@ static int set_state_common(md_handle* h, const double* d_x, const double* d_v, 
   CK(h, cudaMemsetAsync(h->A.sys_free, 0, sizeof(int32_t) * (size_t)h->nsys, st));
   CK(h, launch_build_meta(h->A, h->d_first, h->nsys, d_type, d_con, d_mol, 0, st));
   CK(h, launch_set_state(h->A, d_x, d_v, st));
-  const unsigned long long k = step0;
-  CK(h, cudaMemcpyAsync(h->A.step, &k, sizeof(k), cudaMemcpyHostToDevice, st));
-  CK(h, cudaMemsetAsync(h->A.mode, 0, sizeof(int32_t), st));
-  if (h->A.noise_k) CK(h, cudaMemsetAsync(h->A.noise_k, 0xff, sizeof(unsigned long long), st));  // none stored
-  int rc = rebuild_cells(h);
+  CK(h, launch_set_clock(h->A, step0, 0, st));
+  int rc = rebuild_cells(h, true);
   if (rc) return rc;
   h->state_set = true;
   rc = check_device_status(h);
@@ -1105,12 +1129,8 @@ int md_restore(md_handle* h, const double* x, const double* p_half, uint64_t ste
     CK(h, cudaMemcpyAsync(h->d_stage + 3 * n, p_half, 3 * n * sizeof(double), cudaMemcpyHostToDevice, st));
   }
   CK(h, launch_restore(h->A, h->d_stage, h->d_stage + 3 * n, st));
-  const unsigned long long k = step;
-  const int32_t one = 1;
-  CK(h, cudaMemcpyAsync(h->A.step, &k, sizeof(k), cudaMemcpyHostToDevice, st));
-  CK(h, cudaMemcpyAsync(h->A.mode, &one, sizeof(one), cudaMemcpyHostToDevice, st));
-  if (h->A.noise_k) CK(h, cudaMemsetAsync(h->A.noise_k, 0xff, sizeof(unsigned long long), st));  // none stored
-  rc = rebuild_cells(h);
+  CK(h, launch_set_clock(h->A, step, 1, st));
+  rc = rebuild_cells(h, true);
   if (rc) return rc;
   return check_device_status(h);
 }
@@ -1423,11 +1443,8 @@ int md_status(md_handle* h, uint32_t* flags) {
 int md_get_state_device(md_handle* h, double* d_x, double* d_v, double* d_p_half) {
   int rc = require_state(h);
   if (rc) return rc;
-  if (d_v) {
-    rc = momenta_now(h);
-    if (rc) return rc;
-  }
-  CK(h, launch_get_state(h->A, d_x, d_v, d_p_half, h->stream()));
+  rc = read_state(h, d_x, d_v, d_p_half);
+  if (rc) return rc;
   return check_device_status(h);
 }
 
@@ -1439,19 +1456,18 @@ int md_get_state(md_handle* h, double* x, double* v, double* p_half, uint64_t* s
   double* sx = h->d_stage;
   double* sv = h->d_stage + 3 * n;
   double* sp = h->d_stage + 6 * n;
-  if (v) {
-    rc = momenta_now(h);
-    if (rc) return rc;
-  }
-  CK(h, launch_get_state(h->A, x ? sx : nullptr, v ? sv : nullptr, p_half ? sp : nullptr, st));
+  rc = read_state(h, x ? sx : nullptr, v ? sv : nullptr, p_half ? sp : nullptr);
+  if (rc) return rc;
+  // the status and the step before the arrays: copies to pageable memory hold the host until they are done
+  rc = enqueue_status(h);
+  if (rc) return rc;
+  CK(h, cudaMemcpyAsync(h->h_resid, h->A.step, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
   if (x && n) CK(h, cudaMemcpyAsync(x, sx, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (v && n) CK(h, cudaMemcpyAsync(v, sv, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (p_half && n) CK(h, cudaMemcpyAsync(p_half, sp, 3 * n * sizeof(double), cudaMemcpyDeviceToHost, st));
-  unsigned long long k = 0;
-  CK(h, cudaMemcpyAsync(&k, h->A.step, sizeof(k), cudaMemcpyDeviceToHost, st));
   CK(h, cudaStreamSynchronize(st));
-  if (step) *step = k;
-  return check_device_status(h);
+  if (step) *step = h->h_resid[0];
+  return report_status(h);
 }
 
 int md_forces(md_handle* h, double* f_out, double* u_out) {

@@ -59,12 +59,16 @@ cudaError_t launch_integrate(const DevArrays& A, int precision, int has_pairs, c
 // Step counter on by one, mode = 1 (used when there is no cell list).
 cudaError_t launch_advance(const DevArrays& A, cudaStream_t st);
 
-// p^k into A.pk from the state and A.f (momentum half only).
-cudaError_t launch_finish(const DevArrays& A, int precision, cudaStream_t st);
+// Step counter, first-step flag and rebuild controls of a state that was just
+// set: step k, no stored normals, rebuild flag raised, barrier at zero.
+cudaError_t launch_set_clock(const DevArrays& A, uint64_t k, int32_t mode, cudaStream_t st);
 
-// SoA -> [n][3] for x, v = p^k / m and p^{k-1/2}; outputs may be null.
-cudaError_t launch_get_state(const DevArrays& A, double* d_x_aos, double* d_v_aos, double* d_ph_aos,
-                             cudaStream_t st);
+// Momentum half from the state and A.f: p^k into A.pk, or with va the read-out
+// v = p^k / m [n][3], beside x and p^{k-1/2} (xa, pa may be null).
+cudaError_t launch_finish(const DevArrays& A, int precision, double* xa, double* va, double* pa, cudaStream_t st);
+
+// SoA -> [n][3] for x and p^{k-1/2}; outputs may be null.
+cudaError_t launch_get_state(const DevArrays& A, double* d_x_aos, double* d_ph_aos, cudaStream_t st);
 
 // Forces A.f -> [n][3] float64 and per-particle energies.
 cudaError_t launch_get_forces(const DevArrays& A, int precision, double* d_f_aos, double* d_u,

@@ -3704,48 +3704,55 @@ __global__ void k_advance(unsigned long long* step, int32_t* mode, unsigned long
 // p^k = momentum half of Algorithm 1 from p^{k-1/2} and F^k (state unchanged):
 // the force combination as in k_integrate, the projection with the float64
 // normal at x^k in both precisions.
+// With va (a state read-out) v = p^k / m goes straight to the caller's [n][3]
+// array, x and p^{k-1/2} beside it where asked for, in one pass; without it p^k
+// goes to A.pk (residuals, observables).
 template <typename R>
-__global__ void k_finish(DevArrays A) {
+__global__ void k_finish(DevArrays A, double* xa, double* va, double* pa) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t n = A.n;
   if (i >= n) return;
   const int mode = *A.mode;
-  if (mode == 0) {
-    A.pk[i] = A.ph[i]; A.pk[n + i] = A.ph[n + i]; A.pk[2 * n + i] = A.ph[2 * n + i];
-    return;
-  }
-  const unsigned long long k = *A.step;
   const uint32_t m = A.meta[i];
-  const SysDev& S = A.sys[meta_sys(m)];
   const uint32_t ty = meta_type(m);
   const double x = A.x[i], y = A.x[n + i], z = A.x[2 * n + i];
-  double px = A.ph[i], py = A.ph[n + i], pz = A.ph[2 * n + i];
-  Force3<R> Fr = combine<R>(S, A.types, ty, (uint32_t)(i - S.first), k, 1, load_f3<R>(A.f, i), (R)px, (R)py,
-                            (R)pz, NoiseSlot<R>(A.noise, n, i), false, false);
-  if (S.kind == kXY2D) Fr.z = (R)0;
-  const bool con = meta_con(m);
-  double nx = 0.0, ny = 0.0, nz = 0.0, inv_nn = 0.0;
-  if (con) {  // the float64 normal in both precisions: n.p^k = 0 to float64 rounding
-    surf_eval(S, x, y, z, nx, ny, nz);
-    inv_nn = 1.0 / fma(nx, nx, fma(ny, ny, nz * nz));
+  const double hx = A.ph[i], hy = A.ph[n + i], hz = A.ph[2 * n + i];
+  double px = hx, py = hy, pz = hz;
+  if (mode != 0) {
+    const unsigned long long k = *A.step;
+    const SysDev& S = A.sys[meta_sys(m)];
+    Force3<R> Fr = combine<R>(S, A.types, ty, (uint32_t)(i - S.first), k, 1, load_f3<R>(A.f, i), (R)px, (R)py, (R)pz,
+                              NoiseSlot<R>(A.noise, n, i), false, false);
+    if (S.kind == kXY2D) Fr.z = (R)0;
+    const bool con = meta_con(m);
+    double nx = 0.0, ny = 0.0, nz = 0.0, inv_nn = 0.0;
+    if (con) {  // the float64 normal in both precisions: n.p^k = 0 to float64 rounding
+      surf_eval(S, x, y, z, nx, ny, nz);
+      inv_nn = nr_rcp(fma(nx, nx, fma(ny, ny, nz * nz)));
+    }
+    momentum_half(S.half_dt, (double)Fr.x, (double)Fr.y, (double)Fr.z, con, nx, ny, nz, inv_nn, px, py, pz);
   }
-  momentum_half(S.half_dt, (double)Fr.x, (double)Fr.y, (double)Fr.z, con, nx, ny, nz, inv_nn, px, py, pz);
-  A.pk[i] = px; A.pk[n + i] = py; A.pk[2 * n + i] = pz;
+  if (!va) {
+    A.pk[i] = px; A.pk[n + i] = py; A.pk[2 * n + i] = pz;
+    return;
+  }
+  const double inv_m = A.types->inv_mass[ty];
+  va[3 * i] = px * inv_m; va[3 * i + 1] = py * inv_m; va[3 * i + 2] = pz * inv_m;
+  if (xa) { xa[3 * i] = x; xa[3 * i + 1] = y; xa[3 * i + 2] = z; }
+  if (pa) { pa[3 * i] = hx; pa[3 * i + 1] = hy; pa[3 * i + 2] = hz; }
 }
 
 // ---------------------------------------------------------------------------
 // read-out
 // ---------------------------------------------------------------------------
-__global__ void k_get_state(DevArrays A, double* xa, double* va, double* pa) {
+__global__ void k_get_state(DevArrays A, double* xa, double* pa) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t n = A.n;
   if (i >= n) return;
-  const double inv_m = A.types->inv_mass[meta_type(A.meta[i])];
   for (int d = 0; d < 3; ++d) {
     if (xa) xa[3 * i + d] = A.x[d * n + i];
-    if (va) va[3 * i + d] = A.pk[d * n + i] * inv_m;
     if (pa) pa[3 * i + d] = A.ph[d * n + i];
   }
 }
@@ -4227,17 +4234,30 @@ cudaError_t launch_advance(const DevArrays& A, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_finish(const DevArrays& A, int precision, cudaStream_t st) {
+cudaError_t launch_finish(const DevArrays& A, int precision, double* xa, double* va, double* pa, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
   const int b = block_for(A.n);
-  if (precision == 0) go(k_finish<double>, grid_for(A.n, b), b, st, A);
-  else go(k_finish<float>, grid_for(A.n, b), b, st, A);
-  return cudaGetLastError();
+  if (precision == 0) return go(k_finish<double>, grid_for(A.n, b), b, st, A, xa, va, pa);
+  return go(k_finish<float>, grid_for(A.n, b), b, st, A, xa, va, pa);
 }
 
-cudaError_t launch_get_state(const DevArrays& A, double* xa, double* va, double* pa, cudaStream_t st) {
+cudaError_t launch_get_state(const DevArrays& A, double* xa, double* pa, cudaStream_t st) {
   if (A.n == 0) return cudaSuccess;
-  go(k_get_state, grid_for(A.n, 256), 256, st, A, xa, va, pa);
+  return go(k_get_state, grid_for(A.n, 256), 256, st, A, xa, pa);
+}
+
+__global__ void k_set_clock(unsigned long long* step, int32_t* mode, unsigned long long* noise_k, uint32_t* nl_dirty,
+                            GridBar* gbar, unsigned long long k, int32_t mode_value) {
+  *step = k;
+  *mode = mode_value;
+  *noise_k = ~0ull;
+  if (nl_dirty) *nl_dirty = 1u;
+  gbar->count = 0u;
+  gbar->gen = 0u;
+}
+
+cudaError_t launch_set_clock(const DevArrays& A, uint64_t k, int32_t mode, cudaStream_t st) {
+  k_set_clock<<<1, 1, 0, st>>>(A.step, A.mode, A.noise_k, A.nl_dirty, A.gbar, (unsigned long long)k, mode);
   return cudaGetLastError();
 }
 

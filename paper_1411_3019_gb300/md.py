@@ -300,8 +300,15 @@ def md_info(h):
     return {"n": n.value, "nsys": ns.value, "step": st.value}
 
 
+def _particles(h) -> int:
+    """The handle's particle count (md_info without the step counter, which waits for the stream)."""
+    n = C.c_int64()
+    _check(h, lib().md_info(h, C.byref(n), None, None))
+    return n.value
+
+
 def md_get_state(h, want=("x", "v", "p_half")):
-    n = md_info(h)["n"]
+    n = _particles(h)
     out = {k: np.zeros((n, 3)) for k in want}
     ptr = {k: (out[k].ctypes.data_as(C.c_void_p) if k in out else None) for k in ("x", "v", "p_half")}
     st = C.c_uint64()
@@ -315,7 +322,7 @@ def md_get_state_device(h, d_x=None, d_v=None, d_p_half=None) -> None:
 
 
 def md_forces(h):
-    n = md_info(h)["n"]
+    n = _particles(h)
     f, u = np.zeros((n, 3)), np.zeros(n)
     _check(h, lib().md_forces(h, f.ctypes.data_as(C.c_void_p), u.ctypes.data_as(C.c_void_p)))
     return f, u
