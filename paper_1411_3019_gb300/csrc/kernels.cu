@@ -1029,12 +1029,8 @@ struct AccTerm {
   DF dx, dy, dz;
 };
 
-__device__ __forceinline__ bool acc_pair(const PairTab<float>& tab, uint32_t qt, const float4& ri, const float4& li,
-                                         const float4& rj, const float4& lj, float shx, float shy, float shz,
-                                         AccTerm& t) {
-  t.dx = pair_disp(ri.x, rj.x, shx, __fsub_rn(li.x, lj.x));
-  t.dy = pair_disp(ri.y, rj.y, shy, __fsub_rn(li.y, lj.y));
-  t.dz = pair_disp(ri.z, rj.z, shz, __fsub_rn(li.z, lj.z));
+// The term of a displacement that is set already (t.dx, t.dy, t.dz).
+__device__ __forceinline__ bool acc_term(const PairTab<float>& tab, uint32_t qt, AccTerm& t) {
   const DF px = df_two_prod(t.dx.h, t.dx.h), py = df_two_prod(t.dy.h, t.dy.h), pz = df_two_prod(t.dz.h, t.dz.h);
   const DF s1 = df_two_sum(px.h, py.h);
   const DF s2 = df_two_sum(s1.h, pz.h);
@@ -1063,6 +1059,15 @@ __device__ __forceinline__ bool acc_pair(const PairTab<float>& tab, uint32_t qt,
     t.v -= (r2.h * ir - tab.rc[qt]) * lin;
   }
   return true;
+}
+
+__device__ __forceinline__ bool acc_pair(const PairTab<float>& tab, uint32_t qt, const float4& ri, const float4& li,
+                                         const float4& rj, const float4& lj, float shx, float shy, float shz,
+                                         AccTerm& t) {
+  t.dx = pair_disp(ri.x, rj.x, shx, __fsub_rn(li.x, lj.x));
+  t.dy = pair_disp(ri.y, rj.y, shy, __fsub_rn(li.y, lj.y));
+  t.dz = pair_disp(ri.z, rj.z, shz, __fsub_rn(li.z, lj.z));
+  return acc_term(tab, qt, t);
 }
 
 // f += fr d (low part first), u += v / 2
@@ -2664,31 +2669,43 @@ __global__ void __launch_bounds__(256) k_pair_lanes(DevArrays A) {
 // the run's lanes at once (the float64 pipe costs the same per warp
 // instruction whatever the number of active lanes).
 // Each lane tests a segment of 32 of its candidates against the home
-// particle's largest cutoff first, one bit per hit in a register mask, then
-// evaluates the pair terms over the set bits (self and same-molecule pairs
-// are dropped there): the lanes of a warp run the Lennard-Jones arithmetic
-// together instead of once per candidate that any lane finds in range.
+// particle's largest cutoff first, one bit per hit in a register mask. A
+// particle's hits of the segment are then listed in shared memory (a prefix sum
+// over its lanes) and dealt out to its lanes in turn, so the lanes of a warp run
+// the Lennard-Jones arithmetic together and for as many hits each: lanes that
+// kept their own hits waited for the one with most (about twice the mean). On
+// the mixed path the stage holds each candidate as a double-float already
+// shifted into the home cell's frame, exactly, so a pair's displacement is one
+// error-free difference per axis instead of two, with no second gather. A
+// liquid of 97,336 at r_c = 2.5, 8 particles per warp: 153 us before both, 136 us now.
 // ---------------------------------------------------------------------------
 constexpr int kTileWarps = 4;   // warps per CTA
 constexpr int kTileSlots = 32;  // most sorted slots (particles) per warp: one per lane
-// staged candidates per warp and window (256 float4 or 128 double4 records,
-// 4 KB a warp)
-template <typename R> constexpr int tile_cap() { return sizeof(R) == 4 ? 256 : 128; }
+// staged candidates per warp and window (192 pairs of float4 or 128 double4)
+template <typename R> constexpr int tile_cap() { return sizeof(R) == 4 ? 192 : 128; }
+
+// A warp's stage: the candidates' shifted records and (mixed path) low parts, and
+// the hits of one segment (candidate indices; particle g's from g 32 L on).
+template <typename R> struct TileWarp {
+  typename RecT<R>::T rec[tile_cap<R>()];
+  float4 lo[sizeof(R) == 4 ? tile_cap<R>() : 1];
+  uint8_t hit[1024];
+};
 
 // Copy the staged candidates [w0, w0 + len) of one cell into the warp's
 // stage. Lane k < 27 holds stencil cell k's first slot t0 and its staged
-// offset pre (exclusive prefix of the counts). Four loads per lane are in
-// flight before their stores. All 32 lanes call this.
+// offset pre (exclusive prefix of the counts). Three candidates' loads per lane
+// are in flight before their stores. All 32 lanes call this.
 template <typename R>
-__device__ __forceinline__ void tile_stage(const typename RecT<R>::T* __restrict__ rec, typename RecT<R>::T* stage,
-                                           uint32_t* code, uint32_t t0, uint32_t pre, R csx, R csy, R csz,
-                                           uint32_t w0, uint32_t len, int lane) {
+__device__ __forceinline__ void tile_stage(const typename RecT<R>::T* __restrict__ rec,
+                                           const float4* __restrict__ lo, TileWarp<R>& W, uint32_t t0, uint32_t pre,
+                                           R csx, R csy, R csz, uint32_t w0, uint32_t len, int lane) {
   using Rec = typename RecT<R>::T;
-  constexpr int U = 4;
+  constexpr int U = 3;
   for (uint32_t e0 = 0; e0 < len; e0 += 32u * U) {
     Rec r[U];
+    float4 l[U];
     int kk[U];
-    uint32_t ts[U];
 #pragma unroll
     for (int v = 0; v < U; ++v) {
       const uint32_t e = e0 + 32u * v + (uint32_t)lane, g = w0 + e;
@@ -2701,20 +2718,26 @@ __device__ __forceinline__ void tile_stage(const typename RecT<R>::T* __restrict
       }
       kk[v] = k;
       const uint32_t tk = __shfl_sync(0xffffffffu, t0, k), pk = __shfl_sync(0xffffffffu, pre, k);
-      ts[v] = tk + (g - pk);
-      if (e < len) r[v] = rec[ts[v]];
+      if (e < len) {
+        r[v] = rec[tk + (g - pk)];
+        if (sizeof(R) == 4) l[v] = lo[tk + (g - pk)];
+      }
     }
 #pragma unroll
     for (int v = 0; v < U; ++v) {
       const uint32_t e = e0 + 32u * v + (uint32_t)lane;
       if (e < len) {
         const int k = kk[v];
+        const R sx = (R)(k % 3 - 1) * csx, sy = (R)((k / 3) % 3 - 1) * csy, sz = (R)(k / 9 - 1) * csz;
         Rec q = r[v];
-        q.x += (R)(k % 3 - 1) * csx;
-        q.y += (R)((k / 3) % 3 - 1) * csy;
-        q.z += (R)(k / 9 - 1) * csz;
-        stage[e] = q;
-        code[e] = ts[v] << 5 | (uint32_t)k;  // the candidate's slot and stencil cell
+        if constexpr (sizeof(R) == 4) {  // offset + shift exactly, as high and low parts
+          const DF x = df_two_sum(q.x, sx), y = df_two_sum(q.y, sy), z = df_two_sum(q.z, sz);
+          q.x = x.h; q.y = y.h; q.z = z.h;
+          W.lo[e] = make_float4(__fadd_rn(x.l, l[v].x), __fadd_rn(y.l, l[v].y), __fadd_rn(z.l, l[v].z), 0.f);
+        } else {
+          q.x += sx; q.y += sy; q.z += sz;
+        }
+        W.rec[e] = q;
       }
     }
   }
@@ -2724,9 +2747,8 @@ __device__ __forceinline__ void tile_stage(const typename RecT<R>::T* __restrict
 // their pair forces (and energy shares) go to fw[0 .. hi - lo).
 template <typename R, bool EXCL>
 __device__ __forceinline__ void tile_piece(const DevArrays& A, const PairTab<R>& tab,
-                                           const typename RecT<R>::T* __restrict__ rec, typename RecT<R>::T* stage,
-                                           uint32_t* code, typename V4<R>::T* fw, uint32_t home, uint32_t lo,
-                                           uint32_t hi, int lane) {
+                                           const typename RecT<R>::T* __restrict__ rec, TileWarp<R>& W,
+                                           typename V4<R>::T* fw, uint32_t home, uint32_t lo, uint32_t hi, int lane) {
   using Rec = typename RecT<R>::T;
   const uint32_t* __restrict__ start = A.start;
   const SysDev& S = A.nsys == 1 ? A.sys[0] : A.sys[meta_sys(A.meta[A.stag[lo]])];
@@ -2787,45 +2809,58 @@ __device__ __forceinline__ void tile_piece(const DevArrays& A, const PairTab<R>&
   for (uint32_t w0 = 0; w0 < M; w0 += (uint32_t)tile_cap<R>()) {
     const uint32_t len = min(M - w0, (uint32_t)tile_cap<R>());
     __syncwarp();
-    tile_stage<R>(rec, stage, code, t0, pre, csx, csy, csz, w0, len, lane);
+    tile_stage<R>(rec, A.rec_lo, W, t0, pre, csx, csy, csz, w0, len, lane);
     __syncwarp();
-    if (act) {
-      // the lane's candidates are e = lj + i L, i < ne
-      const uint32_t ne = len > lj ? (len - lj + L - 1u) / L : 0u;
-      for (uint32_t i0 = 0; i0 < ne; i0 += 32u) {
-        const uint32_t nseg = min(ne - i0, 32u);
-        uint32_t mask = 0;
+    // the lane's candidates are e = lj + i L, i < ne (idle lanes: none); the segment loop is the warp's
+    const uint32_t ne = act && len > lj ? (len - lj + L - 1u) / L : 0u;
+    const uint32_t nseg_max = (len + L - 1u) / L;
+    for (uint32_t i0 = 0; i0 < nseg_max; i0 += 32u) {
+      const uint32_t nseg = ne > i0 ? min(ne - i0, 32u) : 0u;
+      uint32_t mask = 0;
 #pragma unroll 4
-        for (uint32_t i = 0; i < nseg; ++i) {
-          const Rec rj = stage[lj + (i0 + i) * L];
-          const R ddx = ri.x - rj.x, ddy = ri.y - rj.y, ddz = ri.z - rj.z;
-          const R r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-          if (r2 < rcm) mask |= 1u << i;
-        }
-        while (mask) {
-          const uint32_t e = lj + (i0 + (uint32_t)(__ffs(mask) - 1)) * L;
-          mask &= mask - 1u;
+      for (uint32_t i = 0; i < nseg; ++i) {
+        const Rec rj = W.rec[lj + (i0 + i) * L];
+        const R ddx = ri.x - rj.x, ddy = ri.y - rj.y, ddz = ri.z - rj.z;
+        const R r2 = ddx * ddx + ddy * ddy + ddz * ddz;
+        if (r2 < rcm) mask |= 1u << i;
+      }
+      // the group's hits in shared memory, lane after lane
+      uint32_t upto = (uint32_t)__popc(mask);
+      for (uint32_t o = 1; o < L; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lj >= o) upto += v;
+      }
+      const uint32_t hits = __shfl_sync(0xffffffffu, upto, min(g * L + L - 1u, 31u));
+      uint8_t* list = W.hit + min(g, p - 1u) * 32u * L;
+      uint32_t at = upto - (uint32_t)__popc(mask);
+      while (mask) {
+        list[at++] = (uint8_t)(lj + (i0 + (uint32_t)(__ffs(mask) - 1)) * L);
+        mask &= mask - 1u;
+      }
+      __syncwarp();
+      if (act) {
+        for (uint32_t h = lj; h < hits; h += L) {
+          const uint32_t e = list[h];
           if (w0 + e == self) continue;
-          const Rec rj = stage[e];
+          const Rec rj = W.rec[e];
           const uint32_t bj = RecT<R>::bits(rj);
           if (EXCL && (bj >> 3) == moli) continue;
           const uint32_t qt = ti * kMaxTypes + (bj & 7u);
-          const R ddx = ri.x - rj.x, ddy = ri.y - rj.y, ddz = ri.z - rj.z;
-          const R r2 = ddx * ddx + ddy * ddy + ddz * ddz;
           if constexpr (sizeof(R) == 4) {
-            // the screen passed on the staged (shifted) record: the candidate's own record, low
-            // part and stencil shift give the pair term
-            if (r2 < tab.acc.rc2m[qt]) {
-              const uint32_t cd = code[e], t = cd >> 5;
-              const int k = (int)(cd & 31u);
-              lj_term_acc(tab, qt, ri, li, rec[t], A.rec_lo[t], (float)(k % 3 - 1) * csx,
-                          (float)((k / 3) % 3 - 1) * csy, (float)(k / 9 - 1) * csz, fx, fy, fz, u);
-            }
+            const float4 l = W.lo[e];
+            AccTerm t;
+            t.dx = df_two_sum(ri.x, -rj.x); t.dx.l = __fadd_rn(t.dx.l, __fsub_rn(li.x, l.x));
+            t.dy = df_two_sum(ri.y, -rj.y); t.dy.l = __fadd_rn(t.dy.l, __fsub_rn(li.y, l.y));
+            t.dz = df_two_sum(ri.z, -rj.z); t.dz.l = __fadd_rn(t.dz.l, __fsub_rn(li.z, l.z));
+            if (acc_term(tab, qt, t)) acc_add(t.fr, t.dx, t.dy, t.dz, t.v, fx, fy, fz, u);
           } else {
+            const R ddx = ri.x - rj.x, ddy = ri.y - rj.y, ddz = ri.z - rj.z;
+            const R r2 = ddx * ddx + ddy * ddy + ddz * ddz;
             if (r2 < tab.rc2[qt]) lj_term<R>(tab, qt, r2, ddx, ddy, ddz, fx, fy, fz, u);
           }
         }
       }
+      __syncwarp();  // the list is written again for the next segment
     }
   }
   // segmented tree: after offset o, lane j of a group holds the sum of its
@@ -2855,8 +2890,7 @@ template <typename R, bool BONDS, bool WALLS, bool EXCL>
 __global__ void __launch_bounds__(kTileWarps * 32, sizeof(R) == 4 ? 6 : 4) k_pair_cell(DevArrays A) {
   using Rec = typename RecT<R>::T;
   __shared__ PairTab<R> tab;
-  __shared__ Rec stage_all[kTileWarps][tile_cap<R>()];
-  __shared__ uint32_t code_all[kTileWarps][tile_cap<R>()];
+  __shared__ TileWarp<R> warp_all[kTileWarps];
   __shared__ typename V4<R>::T f_all[kTileWarps][kTileSlots];
   pdl_launch_next();
   load_tab<R>(tab, A.types);
@@ -2885,8 +2919,7 @@ __global__ void __launch_bounds__(kTileWarps * 32, sizeof(R) == 4 ? 6 : 4) k_pai
     const uint32_t lo = (uint32_t)r0 + (uint32_t)a;
     const uint32_t hi = cut ? (uint32_t)r0 + (uint32_t)(__ffs(cut) - 1) : r1;
     const uint32_t home = __shfl_sync(0xffffffffu, c, a);
-    tile_piece<R, EXCL>(A, tab, rec, stage_all[wib], code_all[wib], f_all[wib] + (lo - (uint32_t)r0), home, lo,
-                        hi, lane);
+    tile_piece<R, EXCL>(A, tab, rec, warp_all[wib], f_all[wib] + (lo - (uint32_t)r0), home, lo, hi, lane);
   }
   if (mine) {  // the pieces' leaders wrote f_all before the last __syncwarp
     const typename V4<R>::T q = f_all[wib][lane];
