@@ -2193,7 +2193,10 @@ __global__ void __launch_bounds__(256, SURFMD_PAIR_NL_MINB) k_pair_nl(DevArrays 
 // run of terms in order: every particle adds its terms in list order with the
 // same arithmetic as k_pair_nl (the same bits), while no lane idles on a short
 // list or on a pair that fails the screen.
-constexpr int kQueueWarps = 8;
+// Warps per CTA of the list walks. Mixed path: four instead of eight spread more
+// evenly over the SMs (588,000 particles 75.4 -> 74.5 us a step, a million 112.0 ->
+// 110.9); float64: eight (60,000 particles 57.6 us a step, four 60.3).
+constexpr int kQueueWarps = 4, kQueueWarps64 = 8;
 #ifndef SURFMD_NLQ_GROUP
 #define SURFMD_NLQ_GROUP 3
 #endif
@@ -2391,9 +2394,9 @@ struct QueueWarp64 {
 };
 
 template <bool BONDS, bool WALLS, bool ENERGY>
-__global__ void __launch_bounds__(kQueueWarps * 32) k_pair_nlq64(DevArrays A) {
+__global__ void __launch_bounds__(kQueueWarps64 * 32) k_pair_nlq64(DevArrays A) {
   __shared__ PairTab<double> tab;
-  __shared__ QueueWarp64 qw_all[kQueueWarps];
+  __shared__ QueueWarp64 qw_all[kQueueWarps64];
   pdl_launch_next();
   load_tab<double>(tab, A.types);
   pdl_wait();  // the table is constant; everything below may be written by the kernels before
@@ -4236,8 +4239,8 @@ static void pair_dispatch(const DevArrays& A, int bonds, int walls, int excl, in
 template <bool ENERGY>
 static void pair_dispatch_nlq64(const DevArrays& A, int bonds, int walls, cudaStream_t st) {
   const int64_t warps = (A.n + A.list_warp - 1) / A.list_warp;
-  const unsigned g = (unsigned)((warps + kQueueWarps - 1) / kQueueWarps);
-  const int b = kQueueWarps * 32;
+  const unsigned g = (unsigned)((warps + kQueueWarps64 - 1) / kQueueWarps64);
+  const int b = kQueueWarps64 * 32;
   switch ((bonds ? 2 : 0) | (walls ? 1 : 0)) {
     case 0: go(k_pair_nlq64<false, false, ENERGY>, g, b, st, A); break;
     case 1: go(k_pair_nlq64<false, true, ENERGY>, g, b, st, A); break;
