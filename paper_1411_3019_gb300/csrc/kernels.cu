@@ -99,22 +99,6 @@ __device__ __forceinline__ void gauss3(uint32_t seed, uint32_t rep, uint32_t pid
 #endif
 }
 
-__device__ __forceinline__ void gauss3(uint32_t seed, uint32_t rep, uint32_t pid, uint64_t k,
-                                       double& gx, double& gy, double& gz) {
-  const uint4 w = philox4x32_10(make_uint4(pid, (uint32_t)k, (uint32_t)(k >> 32), 0u),
-                                make_uint2(seed, rep));
-  const double s = 1.0 / 8388608.0;
-  const double u0 = ((double)(w.x >> 9) + 0.5) * s, u1 = ((double)(w.y >> 9) + 0.5) * s;
-  const double u2 = ((double)(w.z >> 9) + 0.5) * s, u3 = ((double)(w.w >> 9) + 0.5) * s;
-  const double r01 = sqrt(-2.0 * log(u0));
-  const double r23 = sqrt(-2.0 * log(u2));
-  double sn, cs;
-  sincospi(2.0 * u1, &sn, &cs);
-  gx = __dmul_rn(r01, cs);
-  gy = __dmul_rn(r01, sn);
-  gz = __dmul_rn(r23, cospi(2.0 * u3));
-}
-
 // Format conversions on the integer pipe. On this GPU a float64 <-> float32
 // conversion issues on the float64 pipe at the float64 rate (two lanes per SM
 // per clock), as costly as a DFMA; the mixed integrator converts a dozen
@@ -820,6 +804,24 @@ __device__ __forceinline__ double nr_rsqrt(double v) {
   const double r = f2d(rsqrtf(vf));
   const double e = fma(-v * r, r, 1.0);
   return fma(r * e, fma(0.375, e, 0.5), r);
+}
+
+// Float64 normals: as gauss3 above with the library's logarithm, sine and cosine.
+__device__ __forceinline__ void gauss3(uint32_t seed, uint32_t rep, uint32_t pid, uint64_t k,
+                                       double& gx, double& gy, double& gz) {
+  const uint4 w = philox4x32_10(make_uint4(pid, (uint32_t)k, (uint32_t)(k >> 32), 0u),
+                                make_uint2(seed, rep));
+  // (exact in float32, widened on the integer pipe: no float64 conversion, sum or product)
+  const float s = 1.0f / 8388608.0f;
+  const double u0 = f2d(((float)(w.x >> 9) + 0.5f) * s), u1 = f2d(((float)(w.y >> 9) + 0.5f) * s);
+  const double u2 = f2d(((float)(w.z >> 9) + 0.5f) * s), u3 = f2d(((float)(w.w >> 9) + 0.5f) * s);
+  const double a = -2.0 * log(u0), b = -2.0 * log(u2);  // at least 2^-23
+  const double r01 = a * nr_rsqrt(a), r23 = b * nr_rsqrt(b);
+  double sn, cs;
+  sincospi(2.0 * u1, &sn, &cs);
+  gx = __dmul_rn(r01, cs);
+  gy = __dmul_rn(r01, sn);
+  gz = __dmul_rn(r23, cospi(2.0 * u3));
 }
 
 // Surface direction in float32 (mixed path): the gradient of g at a point
@@ -3459,7 +3461,7 @@ __device__ __forceinline__ void integrate_particle_fp64(const DevArrays& A, int6
 // The position half of a constrained particle is position.cuh; a free particle
 // drifts in float64.
 // ---------------------------------------------------------------------------
-template <bool COMPOSED, class Bin>
+template <int SURF, class Bin>
 __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int64_t i, Force3<float> fr_in,
                                                          unsigned long long k, int mode, const Bin& bin,
                                                          bool xi_store = false, bool xi_prev = false) {
@@ -3481,7 +3483,7 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
     const double xv[3] = {x, y, z};
     const float Fv[3] = {F.x, F.y, F.z};
     double xo[3], qo[3];
-    position_half_df<COMPOSED>(S, ty, mode, xv, pv, P, Fv, A.status, xo, qo);
+    position_half_df<SURF>(S, ty, mode, xv, pv, P, Fv, A.status, xo, qo);
     xn = xo[0]; yn = xo[1]; zn = xo[2];
     qx = qo[0]; qy = qo[1]; qz = qo[2];
   } else {
@@ -3504,10 +3506,13 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
   }
 }
 
-// COMPOSED (mixed path): some system's surface is a Gaussian bump or a
-// thylakoid composite (DevArrays::composed).
-template <typename R, bool COMPOSED>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate_nl(DevArrays A) {
+// SURF (mixed path): DevArrays::composed, 1 where some system's surface is a
+// Gaussian bump, 2 where one is a thylakoid composite, else 0; a kernel holds no
+// more surfaces than it needs, and the thylakoid's, the longest, takes 80 registers
+// (128 thylakoids: 66.9 us a step at 64 with spills, 63.8 at 80; a million with a bump
+// 118.2, without the thylakoid compiled in 117.0).
+template <typename R, int SURF>
+__global__ void __launch_bounds__(256, sizeof(R) == 4 && SURF < 2 ? 4 : 3) k_integrate_nl(DevArrays A) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
@@ -3517,12 +3522,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate_nl(De
   const bool store = A.noise && A.store_noise;
   const bool prev = store && k > 0ull && *A.noise_k == k - 1ull;  // ~0: none stored
   if constexpr (sizeof(R) == 4)
-    integrate_particle_mixed<COMPOSED>(A, i, load_f3<float>(A.f, i), k, mode, bin, store, prev);
+    integrate_particle_mixed<SURF>(A, i, load_f3<float>(A.f, i), k, mode, bin, store, prev);
   else integrate_particle_fp64(A, i, load_f3<double>(A.f, i), k, mode, bin, store, prev);
 }
 
-template <typename R, bool BIN, bool COMPOSED>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate(DevArrays A) {
+template <typename R, bool BIN, int SURF>
+__global__ void __launch_bounds__(256, sizeof(R) == 4 && SURF < 2 ? 4 : 3) k_integrate(DevArrays A) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
@@ -3533,7 +3538,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 3) k_integrate(DevAr
   const bool store = A.noise && A.store_noise;
   const bool prev = store && k > 0ull && *A.noise_k == k - 1ull;
   if constexpr (sizeof(R) == 4)
-    integrate_particle_mixed<COMPOSED>(A, i, load_f3<float>(A.f, i), k, mode, bin, store, prev);
+    integrate_particle_mixed<SURF>(A, i, load_f3<float>(A.f, i), k, mode, bin, store, prev);
   else integrate_particle_fp64(A, i, load_f3<double>(A.f, i), k, mode, bin, store, prev);
 }
 
@@ -3717,7 +3722,7 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 2) k_resident(DevArrays A
       const int mode = j == 0 ? mode0 : 1;
       for (uint32_t li = tid; li < n; li += bd) {
         const Force3<R> f{s_fx[li], s_fy[li], s_fz[li]};
-        if constexpr (sizeof(R) == 4) integrate_particle_mixed<true>(A, first + li, f, k, mode, bin);
+        if constexpr (sizeof(R) == 4) integrate_particle_mixed<2>(A, first + li, f, k, mode, bin);
         else integrate_particle_fp64(A, first + li, f, k, mode, bin);
       }
       __syncthreads();
@@ -4350,18 +4355,21 @@ cudaError_t launch_integrate(const DevArrays& A, int precision, int has_pairs, c
   const int b = integrate_block(A.n, precision);
   const unsigned g = grid_for(A.n, b);
   if (A.nl_dirty && has_pairs) {
-    if (precision == 0) go(k_integrate_nl<double, false>, g, b, st, A);
-    else if (A.composed) go(k_integrate_nl<float, true>, g, b, st, A);
-    else go(k_integrate_nl<float, false>, g, b, st, A);
+    if (precision == 0) go(k_integrate_nl<double, 0>, g, b, st, A);
+    else if (A.composed == 2) go(k_integrate_nl<float, 2>, g, b, st, A);
+    else if (A.composed) go(k_integrate_nl<float, 1>, g, b, st, A);
+    else go(k_integrate_nl<float, 0>, g, b, st, A);
   } else if (precision == 0) {
-    if (has_pairs) go(k_integrate<double, true, false>, g, b, st, A);
-    else go(k_integrate<double, false, false>, g, b, st, A);
+    if (has_pairs) go(k_integrate<double, true, 0>, g, b, st, A);
+    else go(k_integrate<double, false, 0>, g, b, st, A);
   } else if (has_pairs) {
-    if (A.composed) go(k_integrate<float, true, true>, g, b, st, A);
-    else go(k_integrate<float, true, false>, g, b, st, A);
+    if (A.composed == 2) go(k_integrate<float, true, 2>, g, b, st, A);
+    else if (A.composed) go(k_integrate<float, true, 1>, g, b, st, A);
+    else go(k_integrate<float, true, 0>, g, b, st, A);
   } else {
-    if (A.composed) go(k_integrate<float, false, true>, g, b, st, A);
-    else go(k_integrate<float, false, false>, g, b, st, A);
+    if (A.composed == 2) go(k_integrate<float, false, 2>, g, b, st, A);
+    else if (A.composed) go(k_integrate<float, false, 1>, g, b, st, A);
+    else go(k_integrate<float, false, 0>, g, b, st, A);
   }
   return cudaGetLastError();
 }

@@ -178,11 +178,11 @@ __device__ __forceinline__ DFPiece df_thyl_piece(const SysDev& S, DF C[3], DF T[
 // differs from the handle's) x^k + (y - x^k - mu n0) in float64;
 // p^{k+1/2} = p + (kick F - (m/dt) mu n0) adds a float32 increment to the
 // float64 momentum.
-// COMPOSED = false leaves out the bump and the thylakoid: a handle without
+// SURF = 0 leaves out the bump and the thylakoid, 1 the thylakoid: a handle without
 // them runs the integrator at fewer registers (with them compiled in, the
 // 250,000-particle ellipsoid + torus step takes 44.0 us, without
 // 39.4).
-template <bool COMPOSED>
+template <int SURF>
 __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, int mode, const double xv[3],
                                                  const double pv[3], const DF P[3], const float F[3],
                                                  uint32_t* status, double xo[3], double qo[3]) {
@@ -199,7 +199,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
   int32_t shape = S.kind;
   DF gconst = S.gconst_df, R = S.R_df;
   int axis = S.axis;
-  const bool moved = COMPOSED && (shape == kThylakoid || shape == kBump);  // C is not x - c componentwise
+  const bool moved = (SURF == 2 && shape == kThylakoid) || (SURF >= 1 && shape == kBump);  // C is not x - c componentwise
   DFPiece piece{};
   if (moved) {
 #pragma unroll
@@ -208,7 +208,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
       const float k = rintf(C[d].h / S.box_len_df[d].h);
       if (k != 0.f) C[d] = df_from(fma(-f2d(k), S.box_len[d], xv[d] - S.c[d]));
     }
-    if (shape == kThylakoid) {
+    if (SURF == 2 && shape == kThylakoid) {
       piece = df_thyl_piece(S, C, T);
       shape = piece.shape;
       gconst = piece.gconst;
@@ -254,7 +254,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
       N[2] = df_scale2(C[2], 2.f);
       break;
     }
-    case kBump: if constexpr (COMPOSED) {
+    case kBump: if constexpr (SURF >= 1) {
       const DF s = df_neg(df_mul(df_add(df_mul(C[0], C[0]), df_mul(C[1], C[1])), S.half_iw2_df));
       B.E = df_mul(S.bumpA_df, df_exp_neg(s));
       B.g0 = df_sub(C[2], B.E);
@@ -292,7 +292,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
   const float dmax = fmaxf(fabsf(D[0].h), fmaxf(fabsf(D[1].h), fabsf(D[2].h)));
   const float floor_mu =
       4.f * 0x1p-47f * dmax * rcp_approx(fmaxf(fabsf(N[0].h), fmaxf(fabsf(N[1].h), fabsf(N[2].h))));
-  const bool torus = shape == kTorus, bump = COMPOSED && shape == kBump, line = !torus && !bump;
+  const bool torus = shape == kTorus, bump = SURF >= 1 && shape == kBump, line = !torus && !bump;
   int it = 0;
   if (line) {  // float32 Newton on the line form g(y) - b mu + c mu^2
     for (; it < S.max_newton; ++it) {
@@ -327,7 +327,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
     float nf[3] = {N[0].h, N[1].h, N[2].h};
 #pragma unroll
     for (int d = 0; d < 3; ++d) e[d] = df_sub(T[d], df_mul(N[d], mu));  // (y - x) - mu n0
-    if (S.kind == kThylakoid) {  // back from the piece's frame
+    if (SURF == 2 && S.kind == kThylakoid) {  // back from the piece's frame
       const DF r[3] = {e[0], e[1], e[2]};
       const float nr[3] = {nf[0], nf[1], nf[2]};
       const float s[3] = {piece.fx, piece.fy, 1.f};
