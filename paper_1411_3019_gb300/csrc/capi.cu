@@ -54,6 +54,11 @@ struct md_handle {
   uint32_t* d_order = nullptr;
   int64_t steps_since_order = 0;
   int64_t last_launches = 0;
+  // Records of the cell list alone, and on the mixed path with the list (record
+  // and low part of a slot side by side); A.rec and A.rec_lo point at one of them.
+  void* rec_plain = nullptr;
+  float4* rec_lo_plain = nullptr;
+  float4* rec_pair = nullptr;
   // Verlet neighbour list (md_set_neighbor_list); A.nl_dirty != null when on
   uint32_t* d_nl_dirty = nullptr;
   int32_t nl_capacity = 0;  // entries per particle the allocated list holds
@@ -79,6 +84,13 @@ struct md_handle {
 };
 
 static std::string g_create_err;
+// With the list, a handle of more particles than this keeps a slot's record and
+// low part side by side in one 32-byte sector: one sector to fetch for a neighbour
+// and one whole sector to write, where the two arrays' traffic outgrows the L2.
+// Microseconds a step, apart and side by side: 588,000 particles 76.1 and 75.0, a
+// million 117.0 and 111.9; at 250,000 no gain, and long lists whose neighbours are
+// found in L1 (245,760 beads of capsids) lose 1.5 %: two arrays coalesce better there.
+constexpr int64_t kPairedRecords = 400000;
 // Steps of the longer graph: consecutive graph launches are ordered end to
 // start, while the kernels inside one graph overlap their launches. It is built
 // when a handle has run kBlockAfter steps, so that a short run does not pay for
@@ -899,6 +911,7 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
   }
   if (!h->has_pairs) A.nbucket = 1;
   A.pair_lanes = 1;
+  A.rec_stride = 1;
   A.pair_queue = 1;
   A.list_warp = 32;
   A.store_noise = 1;
@@ -948,6 +961,8 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
                                     : dalloc(h, reinterpret_cast<float4**>(&r), n));
     A.rec = r;
     if (h->precision != MD_PREC_FP64) al(dalloc(h, &A.rec_lo, n));
+    h->rec_plain = A.rec;
+    h->rec_lo_plain = A.rec_lo;
   }
   {  // unit normals of the last step
     void* w = nullptr;
@@ -1261,6 +1276,9 @@ int md_set_neighbor_list(md_handle* h, double skin, int32_t max_neighbors) {
   if (!(skin > 0.0)) {  // off: back to the per-step cell list
     if (h->A.nl_dirty) {
       h->A.nl_dirty = nullptr;
+      h->A.rec = h->rec_plain;
+      h->A.rec_lo = h->rec_lo_plain;
+      h->A.rec_stride = 1;
       if (h->state_set) {
         int rc = rebuild_cells(h);
         if (rc) return rc;
@@ -1298,8 +1316,9 @@ int md_set_neighbor_list(md_handle* h, double skin, int32_t max_neighbors) {
       if (e == cudaSuccess)
         e = h->precision == MD_PREC_FP64 ? dalloc(h, reinterpret_cast<double4_32a**>(&A.rec0), n)
                                          : dalloc(h, reinterpret_cast<float4**>(&A.rec0), n);
-      if (e == cudaSuccess && h->precision != MD_PREC_FP64) e = dalloc(h, &A.rec0_lo, n);
-      if (e == cudaSuccess && h->precision == MD_PREC_FP64) e = dalloc(h, &A.rec_lo, n);
+      if (e == cudaSuccess && h->precision != MD_PREC_FP64 && h->n > kPairedRecords && !h->rec_pair)
+        e = dalloc(h, &h->rec_pair, 2 * n);
+      if (e == cudaSuccess && h->precision == MD_PREC_FP64 && !h->rec_pair) e = dalloc(h, &h->rec_pair, n);  // screen copies
       if (e != cudaSuccess) return cuda_fail(h, e, "neighbour list allocation");
       h->nl_capacity = max_neighbors;
     }
@@ -1307,6 +1326,13 @@ int md_set_neighbor_list(md_handle* h, double skin, int32_t max_neighbors) {
     A.nl_skin = skin;
     A.nl_half_skin2 = (float)(0.25 * skin * skin);
     A.nl_dirty = h->d_nl_dirty;
+    if (h->precision == MD_PREC_FP64) {
+      A.rec_lo = h->rec_pair;
+    } else if (h->rec_pair) {
+      A.rec = h->rec_pair;
+      A.rec_lo = h->rec_pair + 1;
+      A.rec_stride = 2;
+    }
     if (h->state_set) {
       int rc = rebuild_cells(h);
       if (rc) return rc;
@@ -1808,6 +1834,7 @@ extern "C" int md_forces_noalloc(const md_surface* surf, const md_params* prm, i
   A.n = n;
   A.nsys = 1;
   A.pair_lanes = 1;
+  A.rec_stride = 1;
   if (cells <= kNaMaxBuckets) {
     A.hashed = 0;
     A.nbucket = (uint32_t)cells;

@@ -772,7 +772,8 @@ __device__ __forceinline__ void bucket_build_one(const DevArrays& A, int64_t s) 
   A.scell[d] = cell;
   if (A.slot_of) A.slot_of[tag] = d;
   if (A.smeta) A.smeta[d] = m;
-  put_rec<R>(A.rec, A.rec_lo, d, o[0], o[1], o[2], meta_type(m) | ((A.rec_cell ? cell : mol) << 3));
+  // (the float64 path's screen copies are one float4 per slot: stride 1 there)
+  put_rec<R>(A.rec, A.rec_lo, d * A.rec_stride, o[0], o[1], o[2], meta_type(m) | ((A.rec_cell ? cell : mol) << 3));
 }
 
 template <typename R>
@@ -1806,7 +1807,8 @@ __device__ __forceinline__ uint32_t nl_build_one(const DevArrays& A, const PairT
   const uint32_t tag = C.tag(s);
   const uint32_t cell = C.scell(s);
   const Rec* __restrict__ rec = sizeof(R) == 4 ? reinterpret_cast<const Rec*>(A.rec) : A.rec_lo;
-  const Rec ri = rec[s];
+  const uint32_t stride = A.rec_stride;
+  const Rec ri = rec[s * stride];
   const uint32_t bi = RecT<float>::bits(ri);
   const uint32_t ti = bi & 7u, moli = bi >> 3;
   const SysDev& S = A.sys[meta_sys(A.meta[tag])];
@@ -1831,7 +1833,7 @@ __device__ __forceinline__ uint32_t nl_build_one(const DevArrays& A, const PairT
 #pragma unroll
       for (int q = 0; q < kNlBuildBatch; ++q) {
         if (t0 + q < t1) {
-          rb[q] = rec[t0 + q];
+          rb[q] = rec[(t0 + q) * stride];
           cb[q] = A.rec_cell ? RecT<float>::bits(rb[q]) >> 3 : C.scell(t0 + q);
         }
       }
@@ -1902,11 +1904,18 @@ __device__ __forceinline__ uint32_t nl_build_one(const DevArrays& A, const PairT
   if (cnt > cap) flag(A.status, kFlagNlistFull);
   A.nl_cnt[s] = min(cnt, cap);
   using Full = typename RecT<R>::T;  // by particle: the integrator reads it in particle order
-  reinterpret_cast<Full*>(A.rec0)[tag] = reinterpret_cast<const Full*>(A.rec)[s];
-  if (sizeof(R) == 4) A.rec0_lo[tag] = A.rec_lo[s];
-  A.xb[tag] = A.x[tag];
-  A.xb[n + tag] = A.x[n + tag];
-  A.xb[2 * n + tag] = A.x[2 * n + tag];
+  reinterpret_cast<Full*>(A.rec0)[tag] = reinterpret_cast<const Full*>(A.rec)[s * stride];
+  const double x[3] = {A.x[tag], A.x[n + tag], A.x[2 * n + tag]};
+  if constexpr (sizeof(R) == 4) {  // the origin of the record: position minus record
+    const float4 lo = A.rec_lo[s * stride];
+    A.xb[tag] = x[0] - df_to(DF{ri.x, lo.x});
+    A.xb[n + tag] = x[1] - df_to(DF{ri.y, lo.y});
+    A.xb[2 * n + tag] = x[2] - df_to(DF{ri.z, lo.z});
+  } else {
+    A.xb[tag] = x[0];
+    A.xb[n + tag] = x[1];
+    A.xb[2 * n + tag] = x[2];
+  }
   return min(cnt, cap);
 }
 
@@ -2136,9 +2145,10 @@ __global__ void __launch_bounds__(256, SURFMD_PAIR_NL_MINB) k_pair_nl(DevArrays 
   const uint32_t tag = A.stag[s];
   const uint32_t m = A.meta[tag];
   const SysDev& S = A.sys[meta_sys(m)];
-  const Rec ri = rec[s];
+  const uint32_t kStride = A.rec_stride;
+  const Rec ri = rec[s * kStride];
   const float4* __restrict__ lo = A.rec_lo;
-  const float4 li = rec_lo_at<R>(lo, s);
+  const float4 li = rec_lo_at<R>(lo, s * kStride);
   const uint32_t ti = RecT<R>::bits(ri) & 7u;
   const R csx = sizeof(R) == 4 ? (R)S.cs_f[0] : (R)S.cs[0];
   const R csy = sizeof(R) == 4 ? (R)S.cs_f[1] : (R)S.cs[1];
@@ -2159,8 +2169,8 @@ __global__ void __launch_bounds__(256, SURFMD_PAIR_NL_MINB) k_pair_nl(DevArrays 
     for (int q = 0; q < kNlBatch; ++q) e[q] = nl[k + q];
 #pragma unroll
     for (int q = 0; q < kNlBatch; ++q) {
-      rj[q] = rec[e[q] >> 5];
-      lj[q] = rec_lo_at<R>(lo, e[q] >> 5);
+      rj[q] = rec[(e[q] >> 5) * kStride];
+      lj[q] = rec_lo_at<R>(lo, (e[q] >> 5) * kStride);
     }
 #pragma unroll
     for (int q = 0; q < kNlBatch; ++q) {
@@ -2173,10 +2183,10 @@ __global__ void __launch_bounds__(256, SURFMD_PAIR_NL_MINB) k_pair_nl(DevArrays 
   for (; k < cnt; ++k) {
     const uint32_t e = nl[k];
     const uint32_t code = e & 31u;
-    const Rec rj = rec[e >> 5];
+    const Rec rj = rec[(e >> 5) * kStride];
     const int dz = (int)(code / 9u) - 1, dy = (int)(code / 3u % 3u) - 1, dx = (int)(code % 3u) - 1;
     const uint32_t qt = ti * kMaxTypes + (RecT<R>::bits(rj) & 7u);
-    pair_term<R>(tab, qt, ri, li, rj, lo, e >> 5, (R)dx * csx, (R)dy * csy, (R)dz * csz, fx, fy, fz, u);
+    pair_term<R>(tab, qt, ri, li, rj, lo, (e >> 5) * kStride, (R)dx * csx, (R)dy * csy, (R)dz * csz, fx, fy, fz, u);
   }
   if (BONDS || WALLS) bonded_terms<R>(A, S, tag, m, BONDS, WALLS, fx, fy, fz, u);
   store_f<R>(A.f, tag, fx, fy, fz, u);
@@ -2235,7 +2245,7 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
 }
 
-template <bool BONDS, bool WALLS>
+template <bool BONDS, bool WALLS, uint32_t STRIDE>
 __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(DevArrays A) {
   __shared__ PairTab<float> tab;
   __shared__ QueueWarp qw_all[kQueueWarps];
@@ -2253,14 +2263,15 @@ __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(
   const bool valid = (uint32_t)lane < P && s < (uint32_t)A.n;
   const float4* __restrict__ rec = reinterpret_cast<const float4*>(A.rec);
   const float4* __restrict__ lo = A.rec_lo;
+  constexpr uint32_t stride = STRIDE;  // A.rec_stride
   uint32_t m = 0, cnt = 0, off = 0;
   float csx = 0.f, csy = 0.f, csz = 0.f;
   if (valid) {
     off = A.nl_off[s];
     m = A.smeta[s];  // sorted copy: no gather through the particle's tag
     const SysDev& S = A.sys[meta_sys(m)];
-    Q.ri[lane] = rec[s];
-    Q.li[lane] = lo[s];
+    Q.ri[lane] = rec[s * stride];
+    Q.li[lane] = lo[s * stride];
     csx = S.cs_f[0]; csy = S.cs_f[1]; csz = S.cs_f[2];
     cnt = A.nl_cnt[s];
   }
@@ -2348,8 +2359,9 @@ __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(
       if (p < total) {
         const uint32_t x = 32u * g + (uint32_t)lane;
         Q.code[x] = (uint8_t)(e[g] & 31u);
-        cp_async16(&Q.sr[x], &rec[e[g] >> 5]);
-        cp_async16(&Q.sl[x], &lo[e[g] >> 5]);
+        const uint32_t at = (e[g] >> 5) * stride;
+        cp_async16(&Q.sr[x], rec + at);
+        cp_async16(&Q.sl[x], lo + at);
       }
     }
     cp_async_wait_all();
@@ -3224,50 +3236,48 @@ struct GlobalBin {
   }
 };
 
-// Neighbour-list mode: the particle keeps its cell until the next rebuild;
-// its record moves with it (record at the build + the float64 displacement
-// since the build; on the mixed path the sum is formed as a double-float and
-// split again into the high and low parts), and a displacement beyond skin / 2
-// raises the rebuild flag for this step's cell-list kernels.
+// Neighbour-list mode: the particle keeps its cell until the next rebuild and
+// its record moves with it: float64 path, record of the build + displacement
+// since; mixed path, position minus the record's origin (formed in float64, split
+// into the two parts and written as one 32-byte sector). A displacement beyond
+// skin / 2 raises the rebuild flag for this step's cell-list kernels. On large
+// systems the record's traffic bounds this part (588,000 particles: integrator
+// 39.8 us with it, 30.8 without).
 template <typename R> struct NlSink {
   static constexpr bool kOn = false, kPos = true;
   using Rec = typename RecT<R>::T;
   const uint32_t* slot_of;
   const double* xb;
   const Rec* rec0;
-  const float4* rec0_lo;
   Rec* rec;
   float4* rec_lo;
   uint32_t* dirty;
   float half_skin2;
+  uint32_t stride;
   int64_t n;
   __device__ __forceinline__ explicit NlSink(const DevArrays& A)
-      : slot_of(A.slot_of), xb(A.xb), rec0(reinterpret_cast<const Rec*>(A.rec0)), rec0_lo(A.rec0_lo),
-        rec(reinterpret_cast<Rec*>(A.rec)), rec_lo(A.rec_lo), dirty(A.nl_dirty), half_skin2(A.nl_half_skin2),
-        n(A.n) {}
+      : slot_of(A.slot_of), xb(A.xb), rec0(reinterpret_cast<const Rec*>(A.rec0)), rec(reinterpret_cast<Rec*>(A.rec)),
+        rec_lo(A.rec_lo), dirty(A.nl_dirty), half_skin2(A.nl_half_skin2), stride(A.rec_stride), n(A.n) {}
   __device__ __forceinline__ void put(int64_t, uint32_t) const {}
   __device__ __forceinline__ void pos(int64_t i, double xn, double yn, double zn) const {
     const uint32_t s = slot_of[i];
-    const double dx = xn - xb[i], dy = yn - xb[n + i], dz = zn - xb[2 * n + i];
-    Rec r = rec0[i];
-    float d2;
+    const double d[3] = {xn - xb[i], yn - xb[n + i], zn - xb[2 * n + i]};
+    const Rec r0 = rec0[i];
+    float ex, ey, ez;
     if constexpr (sizeof(R) == 4) {
-      const float4 l = rec0_lo[i];
-      const double dv[3] = {dx, dy, dz};
-      DF e[3];
-      df_from3(dv, e);
-      const DF ox = df_add(DF{r.x, l.x}, e[0]), oy = df_add(DF{r.y, l.y}, e[1]), oz = df_add(DF{r.z, l.z}, e[2]);
-      r.x = ox.h; r.y = oy.h; r.z = oz.h;
-      rec_lo[s] = make_float4(ox.l, oy.l, oz.l, 0.f);
-      d2 = fmaf(e[0].h, e[0].h, fmaf(e[1].h, e[1].h, e[2].h * e[2].h));
+      DF o[3];
+      df_from3(d, o);
+      rec[s * stride] = make_float4(o[0].h, o[1].h, o[2].h, r0.w);
+      rec_lo[s * stride] = make_float4(o[0].l, o[1].l, o[2].l, 0.f);
+      ex = o[0].h - r0.x; ey = o[1].h - r0.y; ez = o[2].h - r0.z;
     } else {
-      r.x += dx; r.y += dy; r.z += dz;
-      const float ex = d2f_rn(dx), ey = d2f_rn(dy), ez = d2f_rn(dz);
-      d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+      Rec r = r0;
+      r.x += d[0]; r.y += d[1]; r.z += d[2];
+      rec[s] = r;
       if (rec_lo) rec_lo[s] = screen_rec(r);
+      ex = d2f_rn(d[0]); ey = d2f_rn(d[1]); ez = d2f_rn(d[2]);
     }
-    rec[s] = r;
-    if (!(d2 <= half_skin2)) atomicOr(dirty, 1u);
+    if (!(fmaf(ex, ex, fmaf(ey, ey, ez * ez)) <= half_skin2)) atomicOr(dirty, 1u);
   }
 };
 
@@ -4286,11 +4296,15 @@ static void pair_dispatch_nl(const DevArrays& H, int bonds, int walls, int energ
     if (A.pair_queue) {
       const int64_t warps = (A.n + A.list_warp - 1) / A.list_warp;
       const unsigned gq = (unsigned)((warps + kQueueWarps - 1) / kQueueWarps);
-      switch ((bonds ? 2 : 0) | (walls ? 1 : 0)) {
-        case 0: go(k_pair_nlq<false, false>, gq, kQueueWarps * 32, st, A); break;
-        case 1: go(k_pair_nlq<false, true>, gq, kQueueWarps * 32, st, A); break;
-        case 2: go(k_pair_nlq<true, false>, gq, kQueueWarps * 32, st, A); break;
-        default: go(k_pair_nlq<true, true>, gq, kQueueWarps * 32, st, A); break;
+      switch ((bonds ? 2 : 0) | (walls ? 1 : 0) | (A.rec_stride == 2 ? 4 : 0)) {
+        case 0: go(k_pair_nlq<false, false, 1>, gq, kQueueWarps * 32, st, A); break;
+        case 1: go(k_pair_nlq<false, true, 1>, gq, kQueueWarps * 32, st, A); break;
+        case 2: go(k_pair_nlq<true, false, 1>, gq, kQueueWarps * 32, st, A); break;
+        case 3: go(k_pair_nlq<true, true, 1>, gq, kQueueWarps * 32, st, A); break;
+        case 4: go(k_pair_nlq<false, false, 2>, gq, kQueueWarps * 32, st, A); break;
+        case 5: go(k_pair_nlq<false, true, 2>, gq, kQueueWarps * 32, st, A); break;
+        case 6: go(k_pair_nlq<true, false, 2>, gq, kQueueWarps * 32, st, A); break;
+        default: go(k_pair_nlq<true, true, 2>, gq, kQueueWarps * 32, st, A); break;
       }
       return;
     }

@@ -202,7 +202,8 @@ struct DevArrays {
   unsigned long long* noise_k;
   int32_t store_noise;  // 1: store and reuse the normals (MD_OPT_STORE_NOISE), 0: draw both steps' again
   void* rec0;           // [n] records at the last build, by particle
-  double* xb;           // [3][n] positions at the last build (user order)
+  double* xb;           // [3][n] by particle: float64 path, the positions at the last build; mixed path, the
+                        // origin of the particle's record (position minus record)
   unsigned long long* nl_builds;  // list builds so far (counter)
   int32_t nl_max;
   float nl_half_skin2;  // (skin / 2)^2
@@ -229,10 +230,11 @@ struct DevArrays {
   uint32_t* stag;       // [n] sorted slot -> particle (canonical order)
   uint32_t* stag_tmp;   // [n] slot -> particle in atomic order (before the canonical sort)
   uint32_t* scell;      // [n] sorted slot -> cell id
+  uint32_t rec_stride;  // float4 (double4) elements from one slot's record to the next: 2 where a slot's record and low
+                        // part share one 32-byte sector (rec_lo = rec + 1; see kPairedRecords), else 1
   void* rec;            // [n] float4 / double4_32a cell-relative offsets + type/mol bits
   float4* rec_lo;       // [n] mixed path: offset - record (the low parts; w unused); float64 path with the
                         // list: the record rounded to float32 (the list walk's screen), else null
-  float4* rec0_lo;      // [n] mixed path with the neighbour list: rec_lo at the last build, by particle
   int32_t ntypes;       // particle types in use (a type must lie in [0, ntypes))
   uint32_t spin_limit;  // reads of a predecessor's scan word before the wait gives up
   GridBar* gbar;        // fused rebuild: grid barrier
