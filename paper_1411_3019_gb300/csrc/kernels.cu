@@ -1794,10 +1794,20 @@ constexpr int kNlBuildBatch = SURFMD_NL_BUILD_BATCH;
 // 250,000 particles on an ellipsoid and a torus took 77 us.)
 constexpr uint32_t kNlStageLen = 32;
 
+// What a float32 r^2 of two records (offsets from their cells' centres, below a
+// cell edge c each) can be wrong by, where r <= c: per axis 2^-24 c for each of
+// the two roundings of the records (drifted by up to c/2), of their difference, of
+// the shift and of the shifted difference, times 2 sqrt(3) c, and the products:
+// below 24 * 2^-24 c^2 for fresh records, 40 * 2^-24 c^2 for drifted ones.
+__device__ __forceinline__ float screen_pad(float cx, float cy, float cz) {
+  const float c = fmaxf(cx, fmaxf(cy, cz));
+  return 0x1p-18f * c * c;
+}
+
 // Both paths test in float32: the mixed path its records, the float64 path their
-// rounded copies (16 bytes each instead of 32, no float64 operation; 60,000
-// particles: 57.8 -> 53.4 us a step), against r_c + skin with a 2^-20 margin over
-// that rounding; an entry too many adds no term.
+// rounded copies (16 bytes each instead of 32, almost no float64 operation; 60,000
+// particles: 57.8 -> 53.4 us a step), where a pair within the rounding of
+// r_c + skin is decided from the float64 records.
 template <typename R, bool EXCL>
 __device__ __forceinline__ uint32_t nl_build_one(const DevArrays& A, const PairTab<R>& tab, uint32_t s,
                                                  uint32_t* stage) {
@@ -1816,6 +1826,16 @@ __device__ __forceinline__ uint32_t nl_build_one(const DevArrays& A, const PairT
   cell_decode(S, cell, c[0], c[1], c[2]);
   const float csx = S.cs_f[0], csy = S.cs_f[1], csz = S.cs_f[2];
   const float skin = (float)A.nl_skin;
+  const float pad = sizeof(R) == 4 ? 0.f : screen_pad(csx, csy, csz);
+  // the float64 decision of the pair of slots s and t, in cells (dx, dy, dz) apart
+  auto within64 = [&](uint32_t t, uint32_t qt, int dx, int dy, int dz) {
+    const double4_32a* __restrict__ full = reinterpret_cast<const double4_32a*>(A.rec);
+    const double4_32a a = full[s], b = full[t];
+    const double ex = a.x - b.x - (double)dx * S.cs[0], ey = a.y - b.y - (double)dy * S.cs[1],
+                 ez = a.z - b.z - (double)dz * S.cs[2];
+    const double rs = (double)tab.rc[qt] + A.nl_skin;
+    return ex * ex + ey * ey + ez * ez < rs * rs;
+  };
   const uint32_t cap = (uint32_t)A.nl_max;
   uint32_t cnt = 0;
   // the candidates of a run of len cells with consecutive ids and consecutive
@@ -1847,12 +1867,14 @@ __device__ __forceinline__ uint32_t nl_build_one(const DevArrays& A, const PairT
         const uint32_t bj = RecT<float>::bits(rj);
         if (EXCL && (bj >> 3) == moli) continue;
         const uint32_t qt = ti * kMaxTypes + (bj & 7u);
-        if (!((float)tab.rc2[qt] > 0.f)) continue;
+        if (sizeof(R) == 4 ? !((float)tab.rc2[qt] > 0.f) : __double2hiint((double)tab.rc2[qt]) <= 0) continue;
         const int dx = dx0 + (int)k;
         const float ddx = ri.x - rj.x - (float)dx * csx, ddy = ri.y - rj.y - shy, ddz = ri.z - rj.z - shz;
         const float r2 = ddx * ddx + ddy * ddy + ddz * ddz;
         const float rs = (float)tab.rc[qt] + skin;
-        if (r2 < rs * rs * (sizeof(R) == 4 ? 1.f : 1.f + 0x1p-20f)) {
+        bool in = r2 < rs * rs - pad;
+        if (sizeof(R) == 8 && !in && r2 < rs * rs + pad) in = within64(t, qt, dx, dy, dz);
+        if (in) {
           const uint32_t entry = t << 5 | (uint32_t)(9 * (dz + 1) + 3 * (dy + 1) + dx + 1);
           if (cnt < kNlStageLen) stage[cnt * 32u + (threadIdx.x & 31u)] = entry;
           else if (cnt < cap) A.nl[(int64_t)s * cap + cnt] = entry;
@@ -2405,6 +2427,7 @@ __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(
 struct QueueWarp64 {
   float4 ri[32];                    // the lanes' own rounded records
   float csx[32], csy[32], csz[32];  // the lanes' cell edges
+  float pad[32];                    // and their screens' margins over the rounding
   double fr[32], d[4][32];          // evaluated terms: factor, displacement, energy
   uint32_t qt[kNlqStage];           // queue: the neighbour's slot
   uint8_t qc[kNlqStage], qo[kNlqStage];  // queue: its stencil cell and the pair's particle (lane)
@@ -2441,6 +2464,7 @@ __global__ void __launch_bounds__(kQueueWarps64 * 32) k_pair_nlq64(DevArrays A) 
   }
   Q.ri[lane] = rif;
   Q.csx[lane] = csx; Q.csy[lane] = csy; Q.csz[lane] = csz;
+  Q.pad[lane] = screen_pad(csx, csy, csz);
   uint32_t incl = cnt;  // prefix sums of the list lengths over the warp
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -2534,7 +2558,7 @@ __global__ void __launch_bounds__(kQueueWarps64 * 32) k_pair_nlq64(DevArrays A) 
         const float ddx = ro.x - rj[g].x - (float)dx * Q.csx[ow], ddy = ro.y - rj[g].y - (float)dy * Q.csy[ow],
                     ddz = ro.z - rj[g].z - (float)dz * Q.csz[ow];
         const float r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-        hit = r2 < tab.acc.rc2m[(RecT<float>::bits(ro) & 7u) * kMaxTypes + (RecT<float>::bits(rj[g]) & 7u)];
+        hit = r2 < tab.acc.rc2m[(RecT<float>::bits(ro) & 7u) * kMaxTypes + (RecT<float>::bits(rj[g]) & 7u)] + Q.pad[ow];
       }
       const uint32_t mask = __ballot_sync(0xffffffffu, hit);
       if (hit) {
