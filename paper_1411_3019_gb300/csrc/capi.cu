@@ -563,17 +563,26 @@ void drop_graphs(md_handle* h) {
   h->steps_run = 0;
 }
 
-// Captures `steps` time steps into *out.
+// Captures `steps` time steps into *out. (The thread's capture mode is relaxed
+// meanwhile, so that a capture another thread has open neither forbids this one
+// nor is invalidated by it.)
 cudaError_t capture_steps(md_handle* h, int64_t steps, cudaGraphExec_t* out) {
-  cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
   if (e != cudaSuccess) return e;
+  cudaGraph_t g = nullptr;
+  e = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) {
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return e;
+  }
   for (int64_t s = 0; s < steps && e == cudaSuccess; ++s) e = enqueue_step(h, h->cap_stream);
   const cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
   if (g) cudaGraphDestroy(g);
   if (e != cudaSuccess) *out = nullptr;
+  cudaThreadExchangeStreamCaptureMode(&mode);
   return e;
 }
 
@@ -919,9 +928,9 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
   // per warp) instead of the row kernel, whose lanes diverge over hundreds of
   // candidates. The line is the mean number of candidates in the 27 cells,
   // measured on a periodic liquid of 97,336 particles, row and tiled, us: mixed
-  // 383 candidates 271 and 153, 216: 104 and 91, 108: 114 and 92, 56: 65 and 95;
-  // float64 383: 2661 and 1262, 108: 1040 and 515, 56: 547 and 399, 22: 144 and
-  // 396. The two add a particle's terms in different orders, so a handle whose
+  // 383 candidates 271 and 133, 216: 104 and 67, 108: 114 and 83, 56: 65 and 87;
+  // float64 383: 2661 and 974, 108: 1040 and 366, 56: 547 and 306, 22: 128 and
+  // 366. The two add a particle's terms in different orders, so a handle whose
   // systems the resident engine could hold keeps the row kernel's order, which
   // that engine repeats bit for bit.
   if (h->has_pairs && !A.hashed && cell_total > 0) {
@@ -1170,8 +1179,11 @@ int md_step(md_handle* h, int64_t nsteps) {
     int64_t chunk = 1;
     const int64_t room = std::min(nsteps - s, ordered ? kOrderEvery - h->steps_since_order : nsteps);
     if (room >= kBlockSteps && h->steps_run >= kBlockAfter) {
-      if (!h->graph_block) CK(h, capture_steps(h, kBlockSteps, &h->graph_block));
-      chunk = kBlockSteps;
+      if (!h->graph_block && capture_steps(h, kBlockSteps, &h->graph_block) != cudaSuccess) {
+        cudaGetLastError();
+        h->steps_run = 0;  // single steps for now
+      }
+      if (h->graph_block) chunk = kBlockSteps;
     }
     CK(h, cudaGraphLaunch(chunk == 1 ? h->graph : h->graph_block, h->stream()));
     s += chunk;
