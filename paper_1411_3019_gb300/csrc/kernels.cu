@@ -2243,17 +2243,22 @@ constexpr int kQueueWarps = 4, kQueueWarps64 = 8;
 #endif
 constexpr int kNlqGroup = SURFMD_NLQ_GROUP;
 constexpr int kNlqStage = 32 * kNlqGroup;  // staged positions per warp
+// Terms of a particle's run that its lane loads together, before it adds them one
+// by one. With long lists most of a warp waits on that chain: capsids 83.2 us a
+// step with one load after another (through the queue), 77.5 with two together,
+// 76.8 with four; bead molecules 34.7, 33.7 and 33.1.
+constexpr uint32_t kRunBatch = 4;
 
 struct QueueWarp {
   float4 ri[32], li[32];  // the lanes' own records and low parts
-  // staged pairs: the neighbour's record and low part; an evaluation
-  // overwrites a staged pair with its term, (fr, dx.h, dy.h, dz.h) and
-  // (dx.l, dy.l, dz.l, v)
+  // staged pairs: the neighbour's record and low part; an evaluation leaves
+  // its terms at the queue positions, (fr, dx.h, dy.h, dz.h) and (dx.l, dy.l,
+  // dz.l, v). (A staged pair at such a place has been read: its own queue
+  // position is no larger than its place.)
   float4 sr[kNlqStage], sl[kNlqStage];
   float csx[32], csy[32], csz[32];  // the lanes' cell edges (their systems')
   uint8_t code[kNlqStage];          // staged pair: stencil cell of the neighbour
   uint8_t own[kNlqStage];           // staged pair: its particle (lane)
-  uint8_t in[kNlqStage];            // staged pair: evaluated term is inside the cutoff
   uint8_t q[kNlqStage];             // queue: staged pairs that passed the screen, in order
   uint8_t run0[32], runn[32];       // per particle: first queue position and length of its run
 };
@@ -2316,6 +2321,7 @@ __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(
     __syncwarp();
     const bool have = (uint32_t)lane < k;
     uint32_t ow = 0;
+    AccTerm t = {};  // a pair outside the cutoff adds zeros
     if (have) {
       const uint32_t x = Q.q[q0 + lane];
       ow = Q.own[x];
@@ -2324,19 +2330,19 @@ __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(
       const float4 rj = Q.sr[x], lj = Q.sl[x];
       const int dz = (int)(code / 9u) - 1, dy = (int)(code / 3u % 3u) - 1, dx = (int)(code % 3u) - 1;
       const uint32_t qt = (RecT<float>::bits(ro) & 7u) * kMaxTypes + (RecT<float>::bits(rj) & 7u);
-      AccTerm t;
-      const bool in = acc_pair(tab, qt, ro, lio, rj, lj, (float)dx * Q.csx[ow], (float)dy * Q.csy[ow],
-                               (float)dz * Q.csz[ow], t);
-      Q.sr[x] = make_float4(t.fr, t.dx.h, t.dy.h, t.dz.h);
-      Q.sl[x] = make_float4(t.dx.l, t.dy.l, t.dz.l, t.v);
-      Q.in[x] = in ? 1 : 0;
+      if (!acc_pair(tab, qt, ro, lio, rj, lj, (float)dx * Q.csx[ow], (float)dy * Q.csy[ow], (float)dz * Q.csz[ow], t))
+        t = {};
     }
     // runs: a queue position starts one where its particle differs from the previous position's
     const uint32_t prev = __shfl_up_sync(0xffffffffu, ow, 1);
     const bool start = have && (lane == 0 || prev != ow);
     const uint32_t starts = __ballot_sync(0xffffffffu, start);
     Q.runn[lane] = 0;
-    __syncwarp();
+    __syncwarp();  // (and every lane has read its staged pair)
+    if (have) {
+      Q.sr[q0 + lane] = make_float4(t.fr, t.dx.h, t.dy.h, t.dz.h);
+      Q.sl[q0 + lane] = make_float4(t.dx.l, t.dy.l, t.dz.l, t.v);
+    }
     if (start) {
       const uint32_t after = starts & ~((2u << lane) - 1u);  // starts above this one
       const uint32_t next = after ? (uint32_t)(__ffs(after) - 1) : k;
@@ -2344,16 +2350,18 @@ __global__ void __launch_bounds__(kQueueWarps * 32, SURFMD_NLQ_MINB) k_pair_nlq(
       Q.runn[ow] = (uint8_t)(next - lane);
     }
     __syncwarp();
-    const uint32_t r0 = Q.run0[lane], rn = Q.runn[lane];
-    const uint32_t longest = __reduce_max_sync(0xffffffffu, rn);
-    for (uint32_t j = 0; j < longest; ++j) {
-      if (j < rn) {
-        const uint32_t x = Q.q[q0 + r0 + j];
-        if (Q.in[x]) {
-          const float4 a = Q.sr[x], b = Q.sl[x];
-          acc_add(a.x, DF{a.y, b.x}, DF{a.z, b.y}, DF{a.w, b.z}, b.w, fx, fy, fz, u);
-        }
+    const uint32_t r0 = q0 + Q.run0[lane], rn = Q.runn[lane];
+    for (uint32_t j = 0; j < rn; j += kRunBatch) {
+      float4 a[kRunBatch], b[kRunBatch];
+#pragma unroll
+      for (uint32_t i = 0; i < kRunBatch; ++i) {
+        const uint32_t x = r0 + min(j + i, rn - 1u);
+        a[i] = Q.sr[x];
+        b[i] = Q.sl[x];
       }
+#pragma unroll
+      for (uint32_t i = 0; i < kRunBatch; ++i)
+        if (j + i < rn) acc_add(a[i].x, DF{a[i].y, b[i].x}, DF{a[i].z, b[i].y}, DF{a[i].w, b[i].z}, b[i].w, fx, fy, fz, u);
     }
     __syncwarp();
   };
