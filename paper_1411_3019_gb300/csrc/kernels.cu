@@ -81,8 +81,8 @@ __device__ __forceinline__ void gauss3(uint32_t seed, uint32_t rep, uint32_t pid
 #if SURFMD_FAST_NOISE
   const float two_pi = 6.28318530717958648f;
   // (near u = 1 the fast logarithm's absolute error can exceed -ln u: clamp at 0)
-  const float r01 = sqrt_approx(fmaxf(-2.0f * __logf(u0), 0.0f));
-  const float r23 = sqrt_approx(fmaxf(-2.0f * __logf(u2), 0.0f));
+  const float r01 = sqrt_newton(fmaxf(-2.0f * __logf(u0), 0.0f));
+  const float r23 = sqrt_newton(fmaxf(-2.0f * __logf(u2), 0.0f));
   float sn, cs;
   __sincosf(two_pi * (u1 - 0.5f), &sn, &cs);
   gx = __fmul_rn(-r01, cs);  // rounded here, also where the next step's sum would take the product into an FMA:
