@@ -3345,12 +3345,17 @@ __device__ __forceinline__ void integrate_particle_fp64(const DevArrays& A, int6
   const bool con = meta_con(m);
   const double dtm = S.dtm[ty];
   double qx, qy, qz, xn, yn, zn;
+  bool solved = false;
   if (con && line_surface(S.kind)) {
     // Plane, sphere, ellipsoid, cylinder: with w = grad g(x^k) / 2 (the plane's
     // normal itself) g on the line y - nu w is the exact quadratic gy - b nu + c
     // nu^2. Newton runs on it in float32 first, then in float64 from the
     // residual: three float64 operations an iteration instead of the about
-    // twenty-five of a point evaluation with its gradient and reciprocal.
+    // twenty-five of a point evaluation with its gradient and reciprocal. The
+    // iterations of both count towards max_newton, so what converges here
+    // converges within that many updates of Algorithm 1; a solve that does not
+    // (the float32 updates took the last of a small max_newton, or a coefficient
+    // is outside float32's range) is done again below, all in float64.
     double d[3] = {x, y, z}, w[3], ia[3];
     if (!S.c_zero) {
       d[0] -= S.c[0]; d[1] -= S.c[1]; d[2] -= S.c[2];
@@ -3396,7 +3401,9 @@ __device__ __forceinline__ void integrate_particle_fp64(const DevArrays& A, int6
     const float xmax = fmaxf(fabsf(d2f_rn(xn)), fmaxf(fabsf(d2f_rn(yn)), fabsf(d2f_rn(zn))));
     const float floor_nu = 4.f * (float)DBL_EPSILON * xmax / wmax;  // an update under 4 ulp of the position
     float nu0 = 0.f;
-    int it = 0;
+    // (a coefficient beyond float32 would make the tolerance or an update meaningless)
+    const bool in_range = fmaxf(fmaxf(fabsf(gyf), fabsf(bf)), fmaxf(cf, wwf)) <= FLT_MAX && wwf >= FLT_MIN;
+    int it = in_range ? 0 : S.max_newton;
     for (; it < S.max_newton; ++it) {
       const float gf = fmaf(fmaf(cf, nu0, -bf), nu0, gyf);
       if (fabsf(gf) < 0.5f * tol_n) break;
@@ -3408,22 +3415,22 @@ __device__ __forceinline__ void integrate_particle_fp64(const DevArrays& A, int6
       }
     }
     double nu = f2d(nu0);
-    bool ok = false;
-    for (;; ++it) {
+    for (; in_range; ++it) {
       const double g = fma(fma(c, nu, -b), nu, gy);
       const float gf = d2f_rn(g);
       const float rden = __frcp_rn(S.frozen ? frozen_den : fmaf(-2.f * d2f_rn(nu), cf, bf));
-      ok = fabsf(gf) < tol_n;
-      if (!ok && it >= S.max_newton) break;
+      solved = fabsf(gf) < tol_n;
+      if (!solved && it >= S.max_newton) break;
       nu = fma(g, f2d(rden), nu);  // (also where the test is met: the residual in hand takes g to its rounding)
-      if (ok) break;
-      if (it > 0 && fabsf(gf * rden) <= floor_nu) { ok = true; break; }
+      if (solved) break;
+      if (it > 0 && fabsf(gf * rden) <= floor_nu) { solved = true; break; }
     }
-    if (!ok) flag(A.status, kFlagRattle);
     xn = fma(-nu, w[0], xn); yn = fma(-nu, w[1], yn); zn = fma(-nu, w[2], zn);
     const double hl = nu * S.inv_dtm[ty];
     qx = fma(-hl, w[0], qx); qy = fma(-hl, w[1], qy); qz = fma(-hl, w[2], qz);
-  } else {
+    if (!solved) { px = A.ph[i]; py = A.ph[n + i]; pz = A.ph[2 * n + i]; }  // (the momentum half has moved them)
+  }
+  if (!solved) {
     double n0x = 0.0, n0y = 0.0, n0z = 0.0, nn = 1.0, inv_nn = 0.0;
     Piece q0{};
     const bool held = S.kind == kThylakoid;  // composite surface: the piece at x^k for the whole solve

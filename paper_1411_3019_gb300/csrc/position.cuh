@@ -294,6 +294,8 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
       4.f * 0x1p-47f * dmax * rcp_approx(fmaxf(fabsf(N[0].h), fmaxf(fabsf(N[1].h), fabsf(N[2].h))));
   const bool torus = shape == kTorus, bump = SURF >= 1 && shape == kBump, line = !torus && !bump;
   int it = 0;
+  const float seed = mu0;
+  bool redo = SURF == 2 && moved && line;  // a thylakoid piece whose updates run out: once more, all in double-float
   if (line) {  // float32 Newton on the line form g(y) - b mu + c mu^2
     for (; it < S.max_newton; ++it) {
       const float gf = fmaf(fmaf(c, mu0, -b.h), mu0, gy.h);
@@ -313,7 +315,13 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
     const DF g = torus ? Q.g(R, gconst, D, N, mu)
                        : (bump ? B.g(S, C, T, N, mu) : df_add_f(df_sub(gy, df_mul(b, mu)), c * mu.h * mu.h));
     if (fabsf(g.h) < tol_n) { ok = true; break; }
-    if (it >= S.max_newton) break;
+    if (it >= S.max_newton) {
+      if (!redo) break;
+      redo = false;
+      mu = {seed, 0.f};
+      it = -1;
+      continue;
+    }
     const float den = S.frozen ? nnf : (torus ? Q.n1n0(N) : (bump ? B.n1n0(N) : fmaf(-2.f * mu.h, c, b.h)));
     const float dmu = g.h * rcp_approx(den);
     mu = df_add_f(mu, dmu);
