@@ -22,7 +22,8 @@
 //   Gaussian bump  from its value at x^k: with E = A exp(-rho^2 / 2w^2) at
 //     x^k (the one exponential of a step) and the displacement e = x(mu) - x^k,
 //     g = g(x^k) + e_z - E expm1(-(2 rho.e + |e_xy|^2) / 2w^2), a short
-//     argument (a displacement of 0.1 sigma on a width of 25 sigma: 4e-3)
+//     argument (a displacement of 0.1 sigma on a width of 25 sigma: 4e-3); where
+//     the step crosses half the box from the bump, from the nearer image of it
 //   thylakoid composite  its piece, chosen at x^k and held for the solve, is a
 //     plane, a cylinder or a torus in coordinates mirrored into the block's
 //     first quadrant and rotated so that the piece's axis is the third
@@ -69,16 +70,22 @@ struct DFBumpEval {
     // -(2 rho.e + |e_xy|^2) / 2w^2
     const DF sx = df_mul(df_add(df_scale2(C[0], 2.f), e[0]), e[0]), sy = df_mul(df_add(df_scale2(C[1], 2.f), e[1]), e[1]);
     const DF ds = df_neg(df_mul(df_add(sx, sy), S.half_iw2_df));
+    float dx = C[0].h + e[0].h, dy = C[1].h + e[1].h;
     DF dE;  // E(x(mu)) - E
-    if (fabsf(ds.h) <= 0.35f) {
+    if (fabsf(ds.h) <= 0.35f && fabsf(dx) <= 0.5f * S.box_len_df[0].h && fabsf(dy) <= 0.5f * S.box_len_df[1].h) {
       dE = df_mul(E, df_expm1_small(ds));
-    } else {  // a displacement of the order of the bump's width: the exponential anew
-      const DF r2 = df_add(df_mul(df_add(C[0], e[0]), df_add(C[0], e[0])), df_mul(df_add(C[1], e[1]), df_add(C[1], e[1])));
+    } else {  // a displacement of the order of the bump's width, or into another image of it: the exponential anew
+      const float kx = rintf(dx / S.box_len_df[0].h), ky = rintf(dy / S.box_len_df[1].h);
+      const DF wx = df_sub(df_add(C[0], e[0]), df_mul_f(S.box_len_df[0], kx));
+      const DF wy = df_sub(df_add(C[1], e[1]), df_mul_f(S.box_len_df[1], ky));
+      const DF r2 = df_add(df_mul(wx, wx), df_mul(wy, wy));
       dE = df_sub(df_mul(S.bumpA_df, df_exp_neg(df_neg(df_mul(r2, S.half_iw2_df)))), E);
+      dx = wx.h;
+      dy = wy.h;
     }
     const float q = 2.f * S.half_iw2_df.h * (E.h + dE.h);  // E(x(mu)) / w^2
-    n1x = q * (C[0].h + e[0].h);
-    n1y = q * (C[1].h + e[1].h);
+    n1x = q * dx;
+    n1y = q * dy;
     return df_sub(df_add(g0, e[2]), dE);
   }
   __device__ __forceinline__ float n1n0(const DF N[3]) const {  // n1 = (E dx / w^2, E dy / w^2, 1), n0_z = 1
