@@ -1468,6 +1468,15 @@ template <typename R> struct GlobalCells {
   __device__ __forceinline__ uint32_t bucket(uint32_t cell) const { return bucket_of(cell, hashed, log_t); }
 };
 
+// Candidates in a stencil cell, from its bucket's bounds. After a scan that timed
+// out the starts are in [0, n] but need not ascend: a falling pair counts as empty,
+// and 27 counts never add up beyond 32 bits, so a warp's walk over the stencil's
+// candidates as one sequence stays inside the cells' slots (the kernels that walk
+// cell by cell end at once).
+__device__ __forceinline__ uint32_t cell_count(uint32_t t0, uint32_t t1) {
+  return t1 > t0 ? min(t1 - t0, 0xffffffffu / 27u) : 0u;
+}
+
 // Tangent-slab pruning of a surface-bound particle's stencil (no free particle
 // in its system): a cell farther from the tangent plane than a neighbour can
 // be holds none.
@@ -1657,7 +1666,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_pair_warp(DevArrays A) {
       nb = cell_id(S, x, y, z);
       const uint32_t b = bucket_of(nb, A.hashed, A.log_t);
       t0 = A.start[b];
-      cl = A.start[b + 1] - t0;
+      cl = cell_count(t0, A.start[b + 1]);
     }
   }
   __syncwarp();
@@ -2891,7 +2900,7 @@ __device__ __forceinline__ void tile_piece(const DevArrays& A, const PairTab<R>&
     if (ok) {
       const uint32_t nb = cell_id(S, x, y, z);
       t0 = start[nb];
-      cnt = start[nb + 1] - t0;
+      cnt = cell_count(t0, start[nb + 1]);
     }
   }
   const R csx = sizeof(R) == 4 ? (R)S.cs_f[0] : (R)S.cs[0];

@@ -1,0 +1,44 @@
+"""GPU: steps that go on after a scan of the bucket counters has timed out. The
+bucket bounds are then in range but need not ascend; every pair kernel stays in
+bounds and ends, the next synchronising call reports MD_ERR_TIMEOUT, and after a
+restore the run repeats one that never timed out bit for bit."""
+import numpy as np
+import pytest
+
+from paper_1411_3019_gb300 import inputs as I, md
+
+pytestmark = pytest.mark.gpu
+
+
+def _systems(kind, precision):
+    if kind == "surfaces":
+        return I.c2_ellipsoid_torus(n_ell=4000, n_tor=1500, seed=8, precision=precision)
+    return I.lj_lattice(52, rc=2.5, seed=3, precision=precision)  # the tiled kernel by default
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("kind,options", [("surfaces", {}), ("surfaces", {md.MD_OPT_PAIR_TILE: 8}),
+                                          ("surfaces", {md.MD_OPT_PAIR_TILE: 32}), ("surfaces", {md.MD_OPT_PAIR_LANES: 4}),
+                                          ("liquid", {})])
+def test_steps_after_a_timed_out_scan(kind, options, precision):
+    with md.Simulation(_systems(kind, precision)) as sim:
+        for key, val in options.items():
+            md.md_set_option(sim.h, key, val)
+        sim.set_state()
+        assert md.md_cell_list(sim.h)["bucket_start"].shape[0] - 1 > 8192  # more than one scan tile
+        sim.step(2)
+        start = sim.state()
+        sim.step(3)
+        sim.sync()
+        want = sim.state()
+        md.md_restore(sim.h, start["x"], start["p_half"], start["step"])
+        md.md_set_option(sim.h, md.MD_OPT_SPIN_LIMIT, 0)
+        sim.step(4)  # the second step's pair kernel takes the first one's broken list
+        assert md.md_status(sim.h) & md.MD_FLAG_TIMEOUT
+        md.md_set_option(sim.h, md.MD_OPT_SPIN_LIMIT, 1 << 22)
+        md.md_restore(sim.h, start["x"], start["p_half"], start["step"])
+        sim.step(3)
+        sim.sync()
+        got = sim.state()
+    for key in ("x", "v", "p_half"):
+        assert np.array_equal(got[key], want[key]), key
