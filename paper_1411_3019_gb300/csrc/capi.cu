@@ -1051,6 +1051,9 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
   if (e == cudaSuccess) e = cudaMemset(A.tile_state, 0, sizeof(unsigned long long) * (size_t)nblk);
   if (e == cudaSuccess) e = cudaMemset(A.scan, 0, sizeof(ScanCtl));
   if (e == cudaSuccess) e = cudaMemset(A.gbar, 0, sizeof(GridBar));
+  // slots that a first list cut short by a timeout leaves unwritten name particle 0 in cell 0
+  for (uint32_t* p : {A.cell, A.stag, A.stag_tmp, A.slot_of, A.scell, h->d_order})
+    if (e == cudaSuccess) e = cudaMemset(p, 0, sizeof(uint32_t) * std::max<size_t>(n, 1));
   if (e == cudaSuccess) e = cudaMemset(h->O.count, 0, sizeof(uint32_t) * h->O.nbucket);
   if (e == cudaSuccess)
     e = cudaMemset(h->O.tile_state, 0,

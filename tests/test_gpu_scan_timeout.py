@@ -42,3 +42,28 @@ def test_steps_after_a_timed_out_scan(kind, options, precision):
         got = sim.state()
     for key in ("x", "v", "p_half"):
         assert np.array_equal(got[key], want[key]), key
+
+
+@pytest.mark.parametrize("skin", [0.0, 0.3])
+def test_first_list_timed_out(skin):
+    """A state whose first cell list is cut short is refused with MD_ERR_TIMEOUT; set again, the run is the usual one."""
+    systems = _systems("surfaces", "mixed")
+    if skin:
+        for s in systems:
+            s["params"] = dict(s["params"], cell_size=float(np.max(s["params"]["rcut"])) + skin)
+    got = []
+    for limit in (1 << 22, 0):
+        with md.Simulation(systems) as sim:
+            if skin:
+                md.md_set_neighbor_list(sim.h, skin, 64)
+            md.md_set_option(sim.h, md.MD_OPT_SPIN_LIMIT, limit)
+            if limit == 0:
+                with pytest.raises(md.MdError) as e:
+                    sim.set_state()
+                assert e.value.code == md.MD_ERR_TIMEOUT
+                md.md_set_option(sim.h, md.MD_OPT_SPIN_LIMIT, 1 << 22)
+            sim.set_state()
+            sim.step(3)
+            sim.sync()
+            got.append(sim.state()["x"])
+    assert np.array_equal(got[0], got[1])
