@@ -1768,6 +1768,7 @@ __global__ void __launch_bounds__(kPairWarps * 32) k_pair_warp(DevArrays A) {
         W.qt[lane] = W.qt[32 + lane];
         W.qc[lane] = W.qc[32 + lane];
       }
+      __syncwarp();  // the next hits are written over the places just read
     }
   }
   if (qn) drain(qn);
@@ -2594,6 +2595,7 @@ __global__ void __launch_bounds__(kQueueWarps64 * 32) k_pair_nlq64(DevArrays A) 
           Q.qc[lane] = Q.qc[q0 + lane];
           Q.qo[lane] = Q.qo[q0 + lane];
         }
+        __syncwarp();  // the next hits are written over the places just read
       }
     }
   }
