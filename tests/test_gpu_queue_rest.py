@@ -34,8 +34,8 @@ def test_float64_list_walk_of_a_dense_liquid(rc):
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_warp_kernel_of_a_dense_liquid(precision):
-    s = I.lj_lattice(15, rc=3.4, seed=6, precision=precision)  # 3,375 particles, small enough for the resident engine
-    want = _forces(s * 4)  # 13,500 particles: the row kernel
+    s = I.lj_lattice(14, rc=3.4, seed=6, precision=precision)  # 2,744 particles, small enough for the resident engine
+    want = _forces(s * 5)  # 13,720 particles: the row kernel
     for _ in range(5):
         got = _forces(s)
         assert all(np.array_equal(a, b[:s[0]["n"]]) for a, b in zip(got, want))
