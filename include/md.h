@@ -330,12 +330,12 @@ int md_step(md_handle* h, int64_t nsteps);
  * run, md_step falls back to the separate launches (md_get_option then
  * reads 0). */
 #define MD_OPT_FUSED_REBUILD 10
-/* MD_OPT_LIST_WARP (with the Verlet list, MD_OPT_PAIR_QUEUE = 1): most
- * particles per warp of the list walk, 32 (default), 16 or 8 (small systems
- * take fewer by themselves). The warp walks its particles' lists as one
- * sequence, 32 entries at a time, so long lists (long cutoffs, dense systems)
- * spread over more warps with fewer particles each. The same bits for every
- * setting. */
+/* MD_OPT_LIST_WARP (with the Verlet list, MD_OPT_PAIR_QUEUE = 1): particles
+ * per warp of the list walk, 32, 16 or 8. Until it is set the walk takes 32,
+ * or fewer on small systems (md_get_option then reads 32); a value that is set
+ * holds for every size. The warp walks its particles' lists as one sequence,
+ * 32 entries at a time, so long lists (long cutoffs, dense systems) spread over
+ * more warps with fewer particles each. The same bits for every setting. */
 #define MD_OPT_LIST_WARP 11
 /* MD_OPT_STORE_NOISE: 1 (default) = the integrator stores the unit normals
  * xi^k it draws for step k (16 bytes per particle, 24 in float64) and the next

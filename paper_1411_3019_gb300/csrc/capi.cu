@@ -922,7 +922,7 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
   A.pair_lanes = 1;
   A.rec_stride = 1;
   A.pair_queue = 1;
-  A.list_warp = 32;
+  A.list_warp = 0;  // follows the size until it is set
   A.store_noise = 1;
   // Cell list every step, dense cells: the cell-tiled pair kernel (8 particles
   // per warp) instead of the row kernel, whose lanes diverge over hundreds of
@@ -1449,7 +1449,7 @@ int md_get_option(md_handle* h, int32_t key, int64_t* value) {
     case MD_OPT_SPIN_LIMIT: *value = h->A.spin_limit; return MD_OK;
     case MD_OPT_PAIR_QUEUE: *value = h->A.pair_queue; return MD_OK;
     case MD_OPT_FUSED_REBUILD: *value = h->fused_rebuild; return MD_OK;
-    case MD_OPT_LIST_WARP: *value = h->A.list_warp; return MD_OK;
+    case MD_OPT_LIST_WARP: *value = h->A.list_warp ? h->A.list_warp : 32; return MD_OK;
     case MD_OPT_STORE_NOISE: *value = h->A.store_noise; return MD_OK;
     case MD_OPT_NLIST_BUILDS: {
       unsigned long long b = 0;

@@ -4318,15 +4318,16 @@ static void pair_dispatch_nlq64(const DevArrays& A, int bonds, int walls, cudaSt
   }
 }
 
-// Particles per warp of the list walks (the same bits for any): at most
-// MD_OPT_LIST_WARP, fewer on small systems, whose walk is one wave of long
-// sequences, and up to twice the size where lists are long (max_neighbors >=
-// 128). Mixed path, 32 / 16 / 8 per warp, us: sphere of 1,000 11.4 / 9.2 / 8.6,
+// Particles per warp of the list walks (the same bits for any): what the caller
+// set (MD_OPT_LIST_WARP), else 32, or fewer on small systems, whose walk is one
+// wave of long sequences, and up to twice the size where lists are long
+// (max_neighbors >= 128). Mixed path, 32 / 16 / 8 per warp, us: sphere of 1,000 11.4 / 9.2 / 8.6,
 // 40,000 9.7 / 9.9 / 13.4; bead molecules, 10,000 15.0 / 13.1 / 11.6, 40,000
 // 17.4 / 15.8 / 17.9; liquid of 27,000 187 / 111 / 71.
 static int32_t list_warp_of(const DevArrays& A) {
+  if (A.list_warp) return A.list_warp;
   const int64_t n = A.nl_max >= 128 ? A.n / 2 : A.n;
-  return std::min(A.list_warp, n <= 16384 ? 8 : n <= 32768 ? 16 : 32);
+  return n <= 16384 ? 8 : n <= 32768 ? 16 : 32;
 }
 
 // energy = 0 (a step's forces): the float64 list walk leaves the pair energies out.
