@@ -493,8 +493,7 @@ def main(argv=None):
     elif skin > 0:
         tuned = {"options": {"neighbor_list_skin": skin, "max_neighbors": workload_max_neighbors(args)},
                  "trials": list_tuned["trials"] if list_tuned else None}
-        if precision != "fp64":
-            tuned["options"]["list_warp"] = md.md_get_option(sim.h, md.MD_OPT_LIST_WARP)
+        tuned["options"]["list_warp"] = md.md_get_option(sim.h, md.MD_OPT_LIST_WARP)
     elif args.pair_tile is not None:
         md.md_set_option(sim.h, md.MD_OPT_PAIR_TILE, args.pair_tile)
         tuned = {"options": {**tuned["options"], "pair_tile": args.pair_tile}}

@@ -147,8 +147,8 @@ def autotune_list(systems, max_neighbors: int, skins=LIST_SKINS, list_warps=LIST
     the handles are destroyed (the caller creates its own with the choice).
     Skins whose list overflows max_neighbors are skipped."""
     trials = []
-    if systems and systems[0]["params"].get("precision") in ("fp64", 0):
-        list_warps = list_warps[:1]  # the float64 path walks per lane: no warp width to choose
+    if list_warps is LIST_WARPS:
+        list_warps = (*LIST_WARPS, 8)  # what the unset walk of a small system takes
     for skin in skins:
         sim = md.Simulation(_with_cell_size(systems, skin), stream=stream)
         try:
@@ -157,10 +157,7 @@ def autotune_list(systems, max_neighbors: int, skins=LIST_SKINS, list_warps=LIST
             sim.step(warmup)
             sim.sync()
             for lw in list_warps:
-                try:
-                    md.md_set_option(sim.h, md.MD_OPT_LIST_WARP, lw)
-                except md.MdError:
-                    continue  # the float64 path has no warp-queued walk
+                md.md_set_option(sim.h, md.MD_OPT_LIST_WARP, lw)
                 md.md_profile_step(sim.h, 2)  # capture and warm this setting
                 if flush is not None:
                     flush()
