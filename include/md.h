@@ -287,10 +287,15 @@ int md_step(md_handle* h, int64_t nsteps);
 /* MD_OPT_RESIDENT_STEPS: most steps one resident launch runs (1..100000,
  * default 256); longer md_step calls are split into several launches. */
 #define MD_OPT_RESIDENT_STEPS 5
-/* MD_OPT_PAIR_TILE: 0 (default) = the pair kernel runs one particle per
- * thread, one per warp on small systems (same bits), MD_OPT_PAIR_LANES lanes
- * per particle, or the cell-tiled kernel at 8 where cells are dense and the
- * systems too large for the resident engine; 8, 16 or 32 = cell-tiled:
+/* MD_OPT_PAIR_TILE: 0 = the pair kernel runs one particle per thread, one per
+ * warp on small systems (same bits), or MD_OPT_PAIR_LANES lanes per particle;
+ * 8, 16 or 32 = cell-tiled; until it is set (md_get_option then reads 0) as 0,
+ * or as 8 in a handle of more than 12,288 particles (8,192 in float64) whose
+ * cells are dense on average over all its systems and of which some system is
+ * too large for the resident engine. The cell-tiled kernel adds a particle's
+ * terms in another order, so the last bits of such a system's forces can
+ * differ between the system alone, in a batch and from md_forces_noalloc; with
+ * 0 set they are one order's everywhere (MD_OPT_PAIR_LANES = 1). Cell-tiled:
  * each warp takes that many consecutive sorted particles, split at cell
  * boundaries; for each piece it copies the records of the home cell's
  * 27-cell stencil into shared memory once and the piece's particles share

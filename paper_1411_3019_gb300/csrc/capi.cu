@@ -1429,6 +1429,7 @@ int md_set_option(md_handle* h, int32_t key, int64_t value) {
       if (value != 0 && h->has_pairs && h->A.hashed)
         return fail(h, MD_ERR_INVALID_ARG, "the cell-tiled pair kernel needs a grid of at most max(2^20, 4N) cells");
       h->A.pair_tile = (int32_t)value;
+      h->A.dense_tile = 0;  // a value that is set holds, 0 too
       break;
     default:
       return fail(h, MD_ERR_INVALID_ARG, "unknown option");
