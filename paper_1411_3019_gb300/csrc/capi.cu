@@ -661,7 +661,8 @@ std::string plan_resident(md_handle* h, int threads) {
   return "";
 }
 
-constexpr int64_t kRebuildLaunches = 7;  // bin, scan, scatter, bucket build, visiting order (3)
+// Kernels that rebuild_cells launches: bin, scan, scatter, bucket build, then the neighbour list or the visiting order (3).
+int64_t rebuild_launches(const md_handle* h) { return !h->has_pairs ? 0 : h->A.nl_dirty ? 5 : 7; }
 
 // Enqueue nsteps steps of every system on the resident engine: chunks of at
 // most res_steps_per_launch steps, one launch per size class per chunk, the
@@ -691,7 +692,7 @@ int resident_steps(md_handle* h, int64_t nsteps) {
   CK(h, enqueue_resident(h, nsteps, h->stream(), &launches));
   int rc = rebuild_cells(h);
   if (rc) return rc;
-  h->last_launches = launches + kRebuildLaunches;
+  h->last_launches = launches + rebuild_launches(h);
   return MD_OK;
 }
 
@@ -1237,7 +1238,7 @@ int md_profile_step(md_handle* h, int64_t nsteps, double* kernel_ms, int32_t max
     kernel_ms[0] = ms[0] / (double)nsteps;
     if (max_kernels > 1) kernel_ms[1] = ms[1] / (double)nsteps;
     if (n_kernels) *n_kernels = 2;
-    h->last_launches = launches + kRebuildLaunches;
+    h->last_launches = launches + rebuild_launches(h);
     return check_device_status(h);
   }
   const StepKernel* ks;
