@@ -343,7 +343,8 @@ int md_step(md_handle* h, int64_t nsteps);
  * more warps with fewer particles each. The same bits for every setting. */
 #define MD_OPT_LIST_WARP 11
 /* MD_OPT_STORE_NOISE: 1 (default) = the integrator stores the unit normals
- * xi^k it draws for step k (16 bytes per particle, 24 in float64) and the next
+ * xi^k it draws for step k (16 bytes per particle, 24 in float64, held by every
+ * handle in which some system has kT and gamma > 0) and the next
  * step's force combination, which needs xi^k again beside xi^(k+1), reads them
  * instead of drawing them a second time; 0 = both steps' normals are drawn
  * every step (the resident engine always draws both). The stored values are

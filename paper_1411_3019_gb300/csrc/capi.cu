@@ -974,13 +974,14 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
     h->rec_plain = A.rec;
     h->rec_lo_plain = A.rec_lo;
   }
-  {  // unit normals of the last step
+  if (std::any_of(h->sys.begin(), h->sys.end(), [](const SysDev& S) { return S.noise_unit != 0.0; })) {
+    // unit normals of the last step (without a thermostat none are drawn)
     void* w = nullptr;
     al(h->precision == MD_PREC_FP64 ? dalloc(h, reinterpret_cast<double**>(&w), 3 * n)
                                     : dalloc(h, reinterpret_cast<float4**>(&w), n));
     A.noise = w;
-    al(dalloc(h, &A.noise_k, 1));
   }
+  al(dalloc(h, &A.noise_k, 1));
   al(dalloc(h, &A.meta, n));
   if (h->excl) al(dalloc(h, &A.mol, n));
   al(dalloc(h, &A.cell, n));
