@@ -1341,7 +1341,13 @@ int md_set_neighbor_list(md_handle* h, double skin, int32_t max_neighbors) {
     }
     A.nl_max = max_neighbors;
     A.nl_skin = skin;
-    A.nl_half_skin2 = (float)(0.25 * skin * skin);
+    // a move just beyond skin / 2 must raise the flag whatever float32 rounds: on the mixed path the displacement is a
+    // difference of record parts (half a cell edge and the skin long, each rounded to 2^-24 of that on three axes)
+    double reach = skin;
+    if (h->precision != MD_PREC_FP64)
+      for (const SysDev& S : h->sys) reach = std::max({reach, S.cs[0] + skin, S.cs[1] + skin, S.cs[2] + skin});
+    const double limit = 0.5 * skin - std::ldexp(reach, -22);
+    A.nl_half_skin2 = limit > 0.0 ? (float)(limit * limit) : -1.f;
     A.nl_dirty = h->d_nl_dirty;
     if (h->precision == MD_PREC_FP64) {
       A.rec_lo = h->rec_pair;

@@ -206,7 +206,7 @@ struct DevArrays {
                         // origin of the particle's record (position minus record)
   unsigned long long* nl_builds;  // list builds so far (counter)
   int32_t nl_max;
-  float nl_half_skin2;  // (skin / 2)^2
+  float nl_half_skin2;  // (skin / 2)^2, less what float32 may round
   double nl_skin;
   int32_t rec_cell;     // 1: a record's w word holds type | cell << 3 (no exclusions,
                         // cells < 2^29), so the pair kernel needs no sorted-cell load;
