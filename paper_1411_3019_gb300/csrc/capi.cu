@@ -941,7 +941,7 @@ int md_create_batch(int32_t nsys, const md_surface* surfs, const md_params* prms
     if (mean >= (h->precision == MD_PREC_FP64 ? 48.0 : 96.0) && !resident_fits) A.dense_tile = 8;
   }
   for (const SysDev& S : h->sys)
-    A.composed = std::max(A.composed, S.kind == kThylakoid ? 2 : S.kind == kBump ? 1 : 0);
+    A.composed |= S.kind == kThylakoid ? 2 : S.kind == kBump ? 1 : 0;
   A.ntypes = prms[0].ntypes;
   A.spin_limit = kDefaultSpinLimit;
   A.rec_cell = (!h->excl && cell_total < (uint64_t(1) << 29)) ? 1 : 0;

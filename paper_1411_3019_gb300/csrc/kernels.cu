@@ -3566,13 +3566,14 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
   }
 }
 
-// SURF (mixed path): DevArrays::composed, 1 where some system's surface is a
-// Gaussian bump, 2 where one is a thylakoid composite, else 0; a kernel holds no
-// more surfaces than it needs, and the thylakoid's, the longest, takes 80 registers
-// (128 thylakoids: 66.9 us a step at 64 with spills, 63.8 at 80; a million with a bump
-// 118.2, without the thylakoid compiled in 117.0).
+// SURF (mixed path): DevArrays::composed, bit 0 where some system's surface is a
+// Gaussian bump, bit 1 where one is a thylakoid composite; a kernel holds no more
+// surfaces than it needs, and the thylakoid's, the longest, takes 80 registers
+// (128 thylakoids: 66.9 us a step at 64 with spills, 63.8 at 80, 60.6 without the
+// bump compiled in, which ends the spills; a million with a bump 118.2, without the
+// thylakoid compiled in 117.0).
 template <typename R, int SURF>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 && SURF < 2 ? 4 : 3) k_integrate_nl(DevArrays A) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 && !(SURF & 2) ? 4 : 3) k_integrate_nl(DevArrays A) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
@@ -3587,7 +3588,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && SURF < 2 ? 4 : 3) k_int
 }
 
 template <typename R, bool BIN, int SURF>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 && SURF < 2 ? 4 : 3) k_integrate(DevArrays A) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 && !(SURF & 2) ? 4 : 3) k_integrate(DevArrays A) {
   pdl_enter();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
@@ -3782,7 +3783,7 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 2) k_resident(DevArrays A
       const int mode = j == 0 ? mode0 : 1;
       for (uint32_t li = tid; li < n; li += bd) {
         const Force3<R> f{s_fx[li], s_fy[li], s_fz[li]};
-        if constexpr (sizeof(R) == 4) integrate_particle_mixed<2>(A, first + li, f, k, mode, bin);
+        if constexpr (sizeof(R) == 4) integrate_particle_mixed<3>(A, first + li, f, k, mode, bin);
         else integrate_particle_fp64(A, first + li, f, k, mode, bin);
       }
       __syncthreads();
@@ -4421,19 +4422,22 @@ cudaError_t launch_integrate(const DevArrays& A, int precision, int has_pairs, c
   const unsigned g = grid_for(A.n, b);
   if (A.nl_dirty && has_pairs) {
     if (precision == 0) go(k_integrate_nl<double, 0>, g, b, st, A);
+    else if (A.composed == 3) go(k_integrate_nl<float, 3>, g, b, st, A);
     else if (A.composed == 2) go(k_integrate_nl<float, 2>, g, b, st, A);
-    else if (A.composed) go(k_integrate_nl<float, 1>, g, b, st, A);
+    else if (A.composed == 1) go(k_integrate_nl<float, 1>, g, b, st, A);
     else go(k_integrate_nl<float, 0>, g, b, st, A);
   } else if (precision == 0) {
     if (has_pairs) go(k_integrate<double, true, 0>, g, b, st, A);
     else go(k_integrate<double, false, 0>, g, b, st, A);
   } else if (has_pairs) {
-    if (A.composed == 2) go(k_integrate<float, true, 2>, g, b, st, A);
-    else if (A.composed) go(k_integrate<float, true, 1>, g, b, st, A);
+    if (A.composed == 3) go(k_integrate<float, true, 3>, g, b, st, A);
+    else if (A.composed == 2) go(k_integrate<float, true, 2>, g, b, st, A);
+    else if (A.composed == 1) go(k_integrate<float, true, 1>, g, b, st, A);
     else go(k_integrate<float, true, 0>, g, b, st, A);
   } else {
-    if (A.composed == 2) go(k_integrate<float, false, 2>, g, b, st, A);
-    else if (A.composed) go(k_integrate<float, false, 1>, g, b, st, A);
+    if (A.composed == 3) go(k_integrate<float, false, 3>, g, b, st, A);
+    else if (A.composed == 2) go(k_integrate<float, false, 2>, g, b, st, A);
+    else if (A.composed == 1) go(k_integrate<float, false, 1>, g, b, st, A);
     else go(k_integrate<float, false, 0>, g, b, st, A);
   }
   return cudaGetLastError();

@@ -22,8 +22,8 @@
 //   Gaussian bump  from its value at x^k: with E = A exp(-rho^2 / 2w^2) at
 //     x^k (the one exponential of a step) and the displacement e = x(mu) - x^k,
 //     g = g(x^k) + e_z - E expm1(-(2 rho.e + |e_xy|^2) / 2w^2), a short
-//     argument (a displacement of 0.1 sigma on a width of 25 sigma: 4e-3); where
-//     the step crosses half the box from the bump, from the nearer image of it
+//     argument (a displacement of 0.1 sigma on a width of 25 sigma: 4e-3); a step
+//     over half the box from the bump goes on with the image it comes to
 //   thylakoid composite  its piece, chosen at x^k and held for the solve, is a
 //     plane, a cylinder or a torus in coordinates mirrored into the block's
 //     first quadrant and rotated so that the piece's axis is the third
@@ -63,6 +63,10 @@ struct DFTorusEval {
 struct DFBumpEval {
   DF E, g0;
   float n1x, n1y;
+  __device__ __forceinline__ void at(const SysDev& S, const DF C[3]) {
+    E = df_mul(S.bumpA_df, df_exp_neg(df_neg(df_mul(df_add(df_mul(C[0], C[0]), df_mul(C[1], C[1])), S.half_iw2_df))));
+    g0 = df_sub(C[2], E);
+  }
   __device__ __forceinline__ DF g(const SysDev& S, const DF C[3], const DF T[3], const DF N[3], DF mu) {
     DF e[3];
 #pragma unroll
@@ -70,22 +74,16 @@ struct DFBumpEval {
     // -(2 rho.e + |e_xy|^2) / 2w^2
     const DF sx = df_mul(df_add(df_scale2(C[0], 2.f), e[0]), e[0]), sy = df_mul(df_add(df_scale2(C[1], 2.f), e[1]), e[1]);
     const DF ds = df_neg(df_mul(df_add(sx, sy), S.half_iw2_df));
-    float dx = C[0].h + e[0].h, dy = C[1].h + e[1].h;
     DF dE;  // E(x(mu)) - E
-    if (fabsf(ds.h) <= 0.35f && fabsf(dx) <= 0.5f * S.box_len_df[0].h && fabsf(dy) <= 0.5f * S.box_len_df[1].h) {
+    if (fabsf(ds.h) <= 0.35f) {
       dE = df_mul(E, df_expm1_small(ds));
-    } else {  // a displacement of the order of the bump's width, or into another image of it: the exponential anew
-      const float kx = rintf(dx / S.box_len_df[0].h), ky = rintf(dy / S.box_len_df[1].h);
-      const DF wx = df_sub(df_add(C[0], e[0]), df_mul_f(S.box_len_df[0], kx));
-      const DF wy = df_sub(df_add(C[1], e[1]), df_mul_f(S.box_len_df[1], ky));
-      const DF r2 = df_add(df_mul(wx, wx), df_mul(wy, wy));
+    } else {  // a displacement of the order of the bump's width: the exponential anew
+      const DF r2 = df_add(df_mul(df_add(C[0], e[0]), df_add(C[0], e[0])), df_mul(df_add(C[1], e[1]), df_add(C[1], e[1])));
       dE = df_sub(df_mul(S.bumpA_df, df_exp_neg(df_neg(df_mul(r2, S.half_iw2_df)))), E);
-      dx = wx.h;
-      dy = wy.h;
     }
     const float q = 2.f * S.half_iw2_df.h * (E.h + dE.h);  // E(x(mu)) / w^2
-    n1x = q * dx;
-    n1y = q * dy;
+    n1x = q * (C[0].h + e[0].h);
+    n1y = q * (C[1].h + e[1].h);
     return df_sub(df_add(g0, e[2]), dE);
   }
   __device__ __forceinline__ float n1n0(const DF N[3]) const {  // n1 = (E dx / w^2, E dy / w^2, 1), n0_z = 1
@@ -185,10 +183,9 @@ __device__ __forceinline__ DFPiece df_thyl_piece(const SysDev& S, DF C[3], DF T[
 // differs from the handle's) x^k + (y - x^k - mu n0) in float64;
 // p^{k+1/2} = p + (kick F - (m/dt) mu n0) adds a float32 increment to the
 // float64 momentum.
-// SURF = 0 leaves out the bump and the thylakoid, 1 the thylakoid: a handle without
-// them runs the integrator at fewer registers (with them compiled in, the
-// 250,000-particle ellipsoid + torus step takes 44.0 us, without
-// 39.4).
+// SURF: the composed surfaces compiled in, bit 0 the bump, bit 1 the thylakoid: a
+// handle runs the integrator without the ones it does not have, at fewer
+// registers and spills.
 template <int SURF>
 __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, int mode, const double xv[3],
                                                  const double pv[3], const DF P[3], const float F[3],
@@ -206,7 +203,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
   int32_t shape = S.kind;
   DF gconst = S.gconst_df, R = S.R_df;
   int axis = S.axis;
-  const bool moved = (SURF == 2 && shape == kThylakoid) || (SURF >= 1 && shape == kBump);  // C is not x - c componentwise
+  const bool moved = ((SURF & 2) && shape == kThylakoid) || ((SURF & 1) && shape == kBump);  // C is not x - c componentwise
   DFPiece piece{};
   if (moved) {
 #pragma unroll
@@ -215,7 +212,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
       const float k = rintf(C[d].h / S.box_len_df[d].h);
       if (k != 0.f) C[d] = df_from(fma(-f2d(k), S.box_len[d], xv[d] - S.c[d]));
     }
-    if (SURF == 2 && shape == kThylakoid) {
+    if ((SURF & 2) && shape == kThylakoid) {
       piece = df_thyl_piece(S, C, T);
       shape = piece.shape;
       gconst = piece.gconst;
@@ -261,10 +258,8 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
       N[2] = df_scale2(C[2], 2.f);
       break;
     }
-    case kBump: if constexpr (SURF >= 1) {
-      const DF s = df_neg(df_mul(df_add(df_mul(C[0], C[0]), df_mul(C[1], C[1])), S.half_iw2_df));
-      B.E = df_mul(S.bumpA_df, df_exp_neg(s));
-      B.g0 = df_sub(C[2], B.E);
+    case kBump: if constexpr ((SURF & 1) != 0) {
+      B.at(S, C);
       const DF q = df_scale2(df_mul(B.E, S.half_iw2_df), 2.f);  // E / w^2
       N[0] = df_mul(q, C[0]);
       N[1] = df_mul(q, C[1]);
@@ -299,11 +294,11 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
   const float dmax = fmaxf(fabsf(D[0].h), fmaxf(fabsf(D[1].h), fabsf(D[2].h)));
   const float floor_mu =
       4.f * 0x1p-47f * dmax * rcp_approx(fmaxf(fabsf(N[0].h), fmaxf(fabsf(N[1].h), fabsf(N[2].h))));
-  const bool torus = shape == kTorus, bump = SURF >= 1 && shape == kBump, line = !torus && !bump;
+  const bool torus = shape == kTorus, bump = (SURF & 1) && shape == kBump, line = !torus && !bump;
   int it = 0;
-  const float seed = mu0;
-  bool redo = SURF == 2 && moved && line;  // a thylakoid piece whose updates run out: once more, all in double-float
-  if (line) {  // float32 Newton on the line form g(y) - b mu + c mu^2
+  // float32 Newton on the line form g(y) - b mu + c mu^2, whose updates count towards max_newton too: on a thylakoid
+  // piece only where that leaves ample for the double-float ones (two or three of each; the frozen normal takes more)
+  if (line && !((SURF & 2) && moved && S.max_newton < (S.frozen ? 16 : 8))) {
     for (; it < S.max_newton; ++it) {
       const float gf = fmaf(fmaf(c, mu0, -b.h), mu0, gy.h);
       if (fabsf(gf) < 0.5f * tol_n) break;
@@ -318,21 +313,37 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
   DFTorusEval Q;
   DF mu = {mu0, 0.f};
   bool ok = false;
-  for (;; ++it) {
-    const DF g = torus ? Q.g(R, gconst, D, N, mu)
-                       : (bump ? B.g(S, C, T, N, mu) : df_add_f(df_sub(gy, df_mul(b, mu)), c * mu.h * mu.h));
-    if (fabsf(g.h) < tol_n) { ok = true; break; }
-    if (it >= S.max_newton) {
-      if (!redo) break;
-      redo = false;
-      mu = {seed, 0.f};
-      it = -1;
-      continue;
+  for (bool turned = !bump;;) {
+    for (;; ++it) {
+      const DF g = torus ? Q.g(R, gconst, D, N, mu)
+                         : (bump ? B.g(S, C, T, N, mu) : df_add_f(df_sub(gy, df_mul(b, mu)), c * mu.h * mu.h));
+      if (fabsf(g.h) < tol_n) { ok = true; break; }
+      if (it >= S.max_newton) break;
+      const float den = S.frozen ? nnf : (torus ? Q.n1n0(N) : (bump ? B.n1n0(N) : fmaf(-2.f * mu.h, c, b.h)));
+      const float dmu = g.h * rcp_approx(den);
+      mu = df_add_f(mu, dmu);
+      if (it > 0 && fabsf(dmu) <= floor_mu) { ok = true; break; }
     }
-    const float den = S.frozen ? nnf : (torus ? Q.n1n0(N) : (bump ? B.n1n0(N) : fmaf(-2.f * mu.h, c, b.h)));
-    const float dmu = g.h * rcp_approx(den);
-    mu = df_add_f(mu, dmu);
-    if (it > 0 && fabsf(dmu) <= floor_mu) { ok = true; break; }
+    // a step of the bump's over half the box: on from here with the image of the bump that it has come to
+    if (turned) break;
+    const float px = fmaf(-N[0].h, mu.h, D[0].h), py = fmaf(-N[1].h, mu.h, D[1].h);
+    const float near = 0.5f - 0x1p-18f;  // (screened in float32, decided in double-float)
+    if (!(fabsf(px) > near * S.box_len_df[0].h || fabsf(py) > near * S.box_len_df[1].h)) break;
+    turned = true;
+    bool moves = false;
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      const DF L = S.box_len_df[d], e = df_sub(D[d], df_mul(N[d], mu)), half = df_scale2(L, 0.5f);
+      const float k = df_less(half, e) ? 1.f : (df_less(e, df_neg(half)) ? -1.f : 0.f);
+      if (k != 0.f) {
+        C[d] = df_sub(C[d], df_mul_f(L, k));
+        moves = true;
+      }
+    }
+    if (!moves) break;
+    B.at(S, C);
+    it = 0;
+    ok = false;
   }
   if (!ok) flag(status, kFlagRattle);
   const float kickf = mode ? S.dt_df.h : S.half_dt_df.h;
@@ -342,7 +353,7 @@ __device__ __forceinline__ void position_half_df(const SysDev& S, uint32_t ty, i
     float nf[3] = {N[0].h, N[1].h, N[2].h};
 #pragma unroll
     for (int d = 0; d < 3; ++d) e[d] = df_sub(T[d], df_mul(N[d], mu));  // (y - x) - mu n0
-    if (SURF == 2 && S.kind == kThylakoid) {  // back from the piece's frame
+    if ((SURF & 2) && S.kind == kThylakoid) {  // back from the piece's frame
       const DF r[3] = {e[0], e[1], e[2]};
       const float nr[3] = {nf[0], nf[1], nf[2]};
       const float s[3] = {piece.fx, piece.fy, 1.f};

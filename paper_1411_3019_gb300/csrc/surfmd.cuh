@@ -179,7 +179,7 @@ struct DevArrays {
   int32_t pair_tile;    // 0, or particles per warp (8, 16, 32) of the cell-tiled pair kernel (needs hashed == 0)
   int32_t dense_tile;   // pair_tile of a dense large handle while the caller sets none (0: the row kernel)
   int32_t pair_queue;   // mixed path with the Verlet list: 1 = warp-queued list walk (k_pair_nlq), 0 = per-lane walk
-  int32_t composed;     // 2: some system's surface is a thylakoid composite, else 1: some is a Gaussian bump, else 0
+  int32_t composed;     // bit 0: some system's surface is a Gaussian bump, bit 1: some is a thylakoid composite
   int32_t list_warp;    // particles per warp of the warp-queued list walk (8, 16 or 32; 0 until set: by the size)
   // Verlet neighbour list (nl_dirty == null: off). Built from the cell list
   // with every pair within r_c + skin; between builds the integrator moves
