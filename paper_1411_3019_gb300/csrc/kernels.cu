@@ -4102,11 +4102,15 @@ __global__ void k_observables(DevArrays A, double* obs) {
 // Launch with programmatic dependent launch allowed (see pdl_wait) for grids of
 // up to kPdlThreads threads. Larger ones gain nothing from a hidden launch
 // latency and lose where a kernel's first CTAs start under the shared-memory
-// split of the kernel before. Microseconds a step without and with it (and the
-// blocks of steps of capi.cu): 1,000 particles in float64 27.5 and 24.0, 100,000
-// bead molecules 38.2 and 36.7, 250,000 38.6 and 36.0, but 588,000 85.2 and 86.5,
-// a million 134.5 and 137.6.
-constexpr int64_t kPdlThreads = 400000;
+// split of the kernel before. 1,000 particles in float64 take 27.5 us a step
+// without and 24.0 with it. Around the line, 20 steps and a read-out with the list,
+// us without and with it: ellipsoid + torus of 270,000 786 and 776, 330,000 945 and
+// 952, 390,000 1,043 and 1,050; sphere of 270,000 760 and 763, 330,000 917 and 924,
+// 390,000 1,008 and 1,023; 2D plane of 270,000 678 and 682, 330,000 785 and 802,
+// 390,000 875 and 899; thylakoids of 270,000 1,082 and 1,071, 320,000 1,217 and
+// 1,213; capsids of 246,000 beads 1,380 and 1,371. (A bump with crowders loses by it
+// from 100,000 on, 270,000 731 and 752.)
+constexpr int64_t kPdlThreads = 300000;
 template <class... P, class... Q>
 static cudaError_t go(void (*kernel)(P...), unsigned grid, int block, cudaStream_t st, Q... args) {
   cudaLaunchConfig_t cfg = {};
