@@ -86,11 +86,14 @@ struct md_handle {
 static std::string g_create_err;
 // With the list, a handle of more particles than this keeps a slot's record and
 // low part side by side in one 32-byte sector: one sector to fetch for a neighbour
-// and one whole sector to write, where the two arrays' traffic outgrows the L2.
-// Microseconds a step, apart and side by side: 588,000 particles 76.1 and 75.0, a
-// million 117.0 and 111.9; at 250,000 no gain, and long lists whose neighbours are
-// found in L1 (245,760 beads of capsids) lose 1.5 %: two arrays coalesce better there.
-constexpr int64_t kPairedRecords = 400000;
+// and one whole sector to write, where the two arrays' traffic outgrows the L2. 20
+// steps and a read-out, us apart and side by side: bump with free crowders, whose
+// neighbours are scattered, 480,000 1,119 and 1,139, 640,000 1,478 and 1,488, 800,000
+// 1,815 and 1,821, a million 2,287 and 2,230 (a step at 900,000: 95.2 and 94.2).
+// Particles on surfaces find their neighbours in L1 and lose by it: spheres of 480,000
+// 1,237 and 1,249, a million 112.3 and 114.6 a step; replicas of 588,000 1,506 and
+// 1,516; capsids of 480,000 beads 2,436 and 2,460.
+constexpr int64_t kPairedRecords = 850000;
 // Steps of the longer graph: consecutive graph launches are ordered end to
 // start, while the kernels inside one graph overlap their launches. It is built
 // when a handle has run kBlockAfter steps, so that a short run does not pay for
