@@ -928,9 +928,14 @@ struct PairAcc {
   float c24[kMaxTypes * kMaxTypes], c4[kMaxTypes * kMaxTypes], s6[kMaxTypes * kMaxTypes];
 };
 
-template <typename R> struct PairTab {
-  R c24[kMaxTypes * kMaxTypes], c48[kMaxTypes * kMaxTypes], c4[kMaxTypes * kMaxTypes], c4b[kMaxTypes * kMaxTypes], rc2[kMaxTypes * kMaxTypes],
-      shift[kMaxTypes * kMaxTypes], lin[kMaxTypes * kMaxTypes], rc[kMaxTypes * kMaxTypes];
+// The float64 path's coefficients (lj_factor); the mixed path's are PairAcc's.
+template <typename R> struct PairCoef {};
+template <> struct PairCoef<double> {
+  double c24[kMaxTypes * kMaxTypes], c48[kMaxTypes * kMaxTypes], c4[kMaxTypes * kMaxTypes], c4b[kMaxTypes * kMaxTypes];
+};
+
+template <typename R> struct PairTab : PairCoef<R> {
+  R rc2[kMaxTypes * kMaxTypes], shift[kMaxTypes * kMaxTypes], lin[kMaxTypes * kMaxTypes], rc[kMaxTypes * kMaxTypes];
   PairAcc acc;
 };
 
@@ -965,10 +970,6 @@ template <> __device__ __forceinline__ void load_tab<double>(PairTab<double>& t,
   }
 }
 
-template <typename R> __device__ __forceinline__ R rsq(R v);
-template <> __device__ __forceinline__ float rsq<float>(float v) { return rsqrtf(v); }
-template <> __device__ __forceinline__ double rsq<double>(double v) { return nr_rsqrt(v); }
-
 // Lennard-Jones pair term inside the cutoff (r2 < r_c^2), phi(r) = 4 eps
 // [(s/r)^12 - (s/r)^6]: the truncated-shifted V = phi(r) - phi(r_c) of Eq. S1
 // and, where the table holds phi'(r_c) != 0, the linearly smoothed form of the
@@ -986,7 +987,7 @@ __device__ __forceinline__ void lj_factor(const PairTab<R>& tab, uint32_t qt, R 
   v = fma(q, fma(tab.c4b[qt], q, -tab.c4[qt]), -tab.shift[qt]);
   const R lin = tab.lin[qt];
   if (lin != (R)0) {
-    const R inv_r = rsq<R>(r2);
+    const R inv_r = nr_rsqrt(r2);
     fr += lin * inv_r;
     v -= (r2 * inv_r - tab.rc[qt]) * lin;
   }
