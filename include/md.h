@@ -316,8 +316,8 @@ int md_step(md_handle* h, int64_t nsteps);
  * 2^22). When the limit runs out the kernel latches MD_FLAG_TIMEOUT, gives its
  * tile a zero prefix (the cell list of that step is then wrong, every access
  * stays in bounds) and returns; the next synchronising call reports
- * MD_ERR_TIMEOUT and the next md_step rebuilds the cell list from the
- * positions before it steps. With 0 the wait gives up without reading, so a
+ * MD_ERR_TIMEOUT (md_status the flag), and the next md_step or read-out that
+ * needs forces rebuilds the cell list from the positions first. With 0 the wait gives up without reading, so a
  * scan of more than one tile (more than 8192 buckets) always times out. */
 #define MD_OPT_SPIN_LIMIT 8
 /* MD_OPT_PAIR_QUEUE (with the Verlet list): 1 (default) = a warp walks its

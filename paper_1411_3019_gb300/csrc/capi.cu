@@ -464,6 +464,7 @@ int rebuild_cells(md_handle* h, bool flagged = false) {
   CK(h, launch_bin(h->A, h->precision, h->stream()));
   CK(h, launch_cells_after_bin(h->A, 0, h->stream()));
   CK(h, launch_bucket_build(h->A, h->precision, h->stream()));
+  h->cells_stale = false;
   if (h->A.nl_dirty) CK(h, launch_nl_build(h->A, h->precision, h->excl, h->stream()));
   if (h->A.nl_dirty) return MD_OK;  // (the list walk takes the slots in order; switching the list off comes back here)
   CK(h, launch_order(h->A, h->O, h->order_coord_shift, h->order_morton_drop, h->order_sys_shift, h->d_order,
@@ -699,7 +700,12 @@ int resident_steps(md_handle* h, int64_t nsteps) {
   return MD_OK;
 }
 
+// Rebuilds a cell list that a reported timeout left incomplete.
+int complete_cells(md_handle* h) { return h->cells_stale ? rebuild_cells(h) : MD_OK; }
+
 int forces_now(md_handle* h) {
+  int rc = complete_cells(h);
+  if (rc) return rc;
   CK(h, launch_pair(h->A, h->precision, h->has_pairs, h->bonds, h->walls, h->excl, 1, h->stream()));
   if (h->bends) CK(h, launch_bend(h->A, h->precision, h->stream()));
   return MD_OK;
@@ -1173,11 +1179,8 @@ int md_step(md_handle* h, int64_t nsteps) {
   if (nsteps < 0) return fail(h, MD_ERR_INVALID_ARG, "nsteps must be >= 0");
   h->last_launches = 0;
   if (nsteps == 0) return MD_OK;
-  if (h->cells_stale) {  // the previous step's cell list did not complete
-    rc = rebuild_cells(h);
-    if (rc) return rc;
-    h->cells_stale = false;
-  }
+  rc = complete_cells(h);
+  if (rc) return rc;
   if (h->engine == 1) return resident_steps(h, nsteps);
   rc = build_graph(h);
   if (rc) return rc;
@@ -1216,6 +1219,8 @@ int md_profile_step(md_handle* h, int64_t nsteps, double* kernel_ms, int32_t max
   int rc = require_state(h);
   if (rc) return rc;
   if (nsteps < 1 || !kernel_ms || max_kernels < 1) return fail(h, MD_ERR_INVALID_ARG, "bad profile arguments");
+  rc = complete_cells(h);
+  if (rc) return rc;
   if (h->engine == 1) {  // resident engine: its launches per step, then the global cell-list rebuild per call
     cudaEvent_t ev[3];
     for (auto& e : ev) CK(h, cudaEventCreate(&e));
@@ -1488,6 +1493,7 @@ int md_status(md_handle* h, uint32_t* flags) {
   CK(h, cudaMemcpyAsync(h->h_status, h->A.status, sizeof(uint32_t), cudaMemcpyDeviceToHost, h->stream()));
   CK(h, cudaStreamSynchronize(h->stream()));
   *flags = *h->h_status & 0xffu;
+  if (*flags & kFlagTimeout) h->cells_stale = true;  // as where a call reports it: the next step rebuilds the cell list
   CK(h, cudaMemsetAsync(h->A.status, 0, sizeof(uint32_t), h->stream()));
   CK(h, cudaStreamSynchronize(h->stream()));
   return MD_OK;

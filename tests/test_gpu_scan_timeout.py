@@ -67,3 +67,21 @@ def test_first_list_timed_out(skin):
             sim.sync()
             got.append(sim.state()["x"])
     assert np.array_equal(got[0], got[1])
+
+
+def test_what_is_read_after_a_timeout_has_a_rebuilt_list():
+    """md_status reports and clears the timeout as md_sync does; forces read then, and the next md_step, have the cell
+    list rebuilt first."""
+    got = []
+    for limit in (1 << 22, 0):
+        with md.Simulation(_systems("surfaces", "mixed")) as sim:
+            sim.set_state()
+            md.md_set_option(sim.h, md.MD_OPT_SPIN_LIMIT, limit)
+            sim.step(1)
+            assert md.md_status(sim.h) == (0 if limit else md.MD_FLAG_TIMEOUT)
+            md.md_set_option(sim.h, md.MD_OPT_SPIN_LIMIT, 1 << 22)
+            f, u = sim.forces()
+            sim.step(3)
+            sim.sync()
+            got.append([f, u, *(sim.state()[k] for k in ("x", "v", "p_half"))])
+    assert all(np.array_equal(a, b) for a, b in zip(*got))
