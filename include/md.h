@@ -121,8 +121,17 @@ typedef struct md_surface {
 
 /* ---- parameters of one system ------------------------------------------ */
 #define MD_PREC_FP64  0  /* every step in float64                              */
-#define MD_PREC_MIXED 1  /* float32 pair forces and noise; float64 state,
-                            Newton solve, projection and position update      */
+#define MD_PREC_MIXED 1 /* float32 pair forces, noise and force combination;
+                            state held in float64. The Newton solve and the
+                            position update of constrained particles, and
+                            what cancels in pair, bond, bend-angle and wall
+                            terms, are double-float arithmetic (two float32
+                            numbers, about 46 bits): the constraint is met to
+                            rattle_tol, or to about 2^-46 of the coordinates
+                            about the surface's centre where that is more
+                            (2e-13 sigma at a size of 10). Free particles'
+                            position update and the projection of the
+                            velocities that are read out are float64.         */
 
 /* Pair potential forms, phi(r) = 4 eps [(sigma/r)^12 - (sigma/r)^6], both 0
  * for r >= rcut:
@@ -261,9 +270,11 @@ int md_step(md_handle* h, int64_t nsteps);
  * partial forces combined by shuffles). A change takes effect at the next
  * md_step (the captured step is rebuilt). */
 #define MD_OPT_PAIR_LANES 1
-/* MD_OPT_PAIR_ORDER: 1 (default) = the pair kernel visits particles in a
- * spatial (Morton) order refreshed every 16 steps, so neighbouring threads
- * share cache lines; 0 = bucket order. */
+/* MD_OPT_PAIR_ORDER: 1 (default) = the pair kernel of one particle per thread
+ * visits particles in a spatial (Morton) order refreshed every 16 steps, so
+ * neighbouring threads share cache lines; 0 = bucket order. The other pair
+ * kernels (a warp or several lanes per particle, cell-tiled, the neighbour
+ * list's) take the slots in order. */
 #define MD_OPT_PAIR_ORDER 2
 /* MD_OPT_ENGINE: 0 (default) = every step is one graph of five kernels over
  * the whole batch with the cell list in global memory; 1 = resident engine:

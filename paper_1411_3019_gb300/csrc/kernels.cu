@@ -3570,7 +3570,7 @@ __device__ __forceinline__ void integrate_particle_mixed(const DevArrays& A, int
 // SURF (mixed path): DevArrays::composed, bit 0 where some system's surface is a
 // Gaussian bump, bit 1 where one is a thylakoid composite; a kernel holds no more
 // surfaces than it needs, and the thylakoid's, the longest, takes 80 registers
-// (128 thylakoids: 66.9 us a step at 64 with spills, 63.8 at 80, 60.6 without the
+// (128 thylakoids: 66.9 us a step at 64 with spills, 63.8 at 80, 61 without the
 // bump compiled in, which ends the spills; a million with a bump 118.2, without the
 // thylakoid compiled in 117.0).
 template <typename R, int SURF>
@@ -4229,12 +4229,15 @@ static void pair_dispatch_row(const DevArrays& A, int bonds, int walls, int excl
   }
 }
 
-// A system of at most this many particles takes k_pair_warp instead of
+// A handle of at most this many particles takes k_pair_warp instead of
 // k_pair_row (same bits). Above, a warp per particle is more work than the row
-// kernel's latency hides: on the sparsest workload (a 2D plane, 9 cells of one
-// particle each) the two cross near 12,000 particles on the mixed path (20,000:
-// row 15.7, warp 21.1 us) and 8,000 in float64 (20,000: 29.3 and 47.3 us); on
-// the others later (sphere, 16,000: 29.3 and 19.1 us; float64 57.6 and 42.2).
+// kernel's latency hides. Where the two cross depends on the candidates per
+// particle; the line is the sparsest workload's (a 2D plane, 9 cells of one
+// particle each), which crosses first: near 12,000 particles on the mixed path
+// (20,000: row 15.7, warp 21.1 us) and 8,000 in float64 (20,000: 29.3 and 47.3 us).
+// Denser ones cross later (sphere, 16,000: 29.3 and 19.1 us; float64 57.6 and 42.2)
+// and take the row kernel from the line on, as every size did before the warp
+// kernel was there, or the tiled one.
 template <typename R> constexpr int64_t warp_pair_max() { return sizeof(R) == 4 ? 12288 : 8192; }
 
 template <typename R>
