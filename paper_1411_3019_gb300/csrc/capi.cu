@@ -631,7 +631,7 @@ std::string plan_resident(md_handle* h, int threads) {
   if (threads > 0) cands.push_back(threads);
   else cands.assign(std::begin(cands_auto), std::end(cands_auto));
   auto ctas = [&](int64_t n, uint32_t t_b, int thr) {
-    return resident_blocks_per_sm(h->precision, h->bonds, h->walls, h->excl, (uint32_t)n, t_b, thr);
+    return resident_blocks_per_sm(h->precision, h->bonds, h->walls, h->excl, h->A.composed, (uint32_t)n, t_b, thr);
   };
   const int nsys = (int)h->res_n_sorted.size();
   for (int i = 0; i < nsys;) {

@@ -84,7 +84,8 @@ cudaError_t launch_resident(const DevArrays& A, int precision, const ResidentJob
                             int threads, int grid_cap, cudaStream_t st);
 cudaError_t launch_advance_n(const DevArrays& A, int32_t nsteps, cudaStream_t st);
 // CTAs of the resident kernel that fit on one SM (0: none).
-int resident_blocks_per_sm(int precision, int bonds, int walls, int excl, uint32_t nmax, uint32_t tmax, int threads);
+int resident_blocks_per_sm(int precision, int bonds, int walls, int excl, int composed, uint32_t nmax, uint32_t tmax,
+                           int threads);
 
 // out_f[i] = in[i] rounded to float32, out_d[i] = out_f[i] widened to float64,
 // by the integer-pipe conversions of the mixed path.

@@ -3701,7 +3701,10 @@ __device__ __forceinline__ void resident_cells(const DevArrays& A, const SysDev&
   __syncthreads();
 }
 
-template <typename R, bool BONDS, bool WALLS, bool EXCL>
+// SURF as in k_integrate: with every composed surface compiled in, the 64
+// registers spill 140 bytes, with none 32 (1,024 capsids 236 and 219 us a step,
+// 4,096 replicas 1,208 and 1,147).
+template <typename R, bool BONDS, bool WALLS, bool EXCL, int SURF>
 __global__ void __launch_bounds__(kResidentMaxThreads, 2) k_resident(DevArrays A, ResidentJob J) {
   using Rec = typename RecT<R>::T;
   __shared__ PairTab<R> tab;
@@ -3784,7 +3787,7 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 2) k_resident(DevArrays A
       const int mode = j == 0 ? mode0 : 1;
       for (uint32_t li = tid; li < n; li += bd) {
         const Force3<R> f{s_fx[li], s_fy[li], s_fz[li]};
-        if constexpr (sizeof(R) == 4) integrate_particle_mixed<3>(A, first + li, f, k, mode, bin);
+        if constexpr (sizeof(R) == 4) integrate_particle_mixed<SURF>(A, first + li, f, k, mode, bin);
         else integrate_particle_fp64(A, first + li, f, k, mode, bin);
       }
       __syncthreads();
@@ -3808,10 +3811,10 @@ size_t resident_smem_bytes(int precision, uint32_t nmax, uint32_t tmax) {
          sizeof(uint32_t) * ((size_t)tmax + 1) + 32;
 }
 
-template <typename R, bool BONDS, bool WALLS, bool EXCL>
+template <typename R, bool BONDS, bool WALLS, bool EXCL, int SURF>
 cudaError_t resident_one(const DevArrays& A, const ResidentJob& J, int threads, int grid_cap, cudaStream_t st) {
   const size_t smem = resident_smem_bytes(sizeof(R) == 4 ? 1 : 0, J.nmax, J.tmax);
-  auto kern = k_resident<R, BONDS, WALLS, EXCL>;
+  auto kern = k_resident<R, BONDS, WALLS, EXCL, SURF>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
@@ -3832,19 +3835,24 @@ cudaError_t launch_advance_n(const DevArrays& A, int32_t nsteps, cudaStream_t st
   return cudaGetLastError();
 }
 
-template <typename R>
+template <typename R, int SURF>
 cudaError_t resident_dispatch(const DevArrays& A, const ResidentJob& J, int bonds, int walls, int excl, int threads,
                               int grid_cap, cudaStream_t st) {
-  const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
-  switch (key) {
-    case 0: return resident_one<R, false, false, false>(A, J, threads, grid_cap, st);
-    case 1: return resident_one<R, false, false, true>(A, J, threads, grid_cap, st);
-    case 2: return resident_one<R, false, true, false>(A, J, threads, grid_cap, st);
-    case 3: return resident_one<R, false, true, true>(A, J, threads, grid_cap, st);
-    case 4: return resident_one<R, true, false, false>(A, J, threads, grid_cap, st);
-    case 5: return resident_one<R, true, false, true>(A, J, threads, grid_cap, st);
-    case 6: return resident_one<R, true, true, false>(A, J, threads, grid_cap, st);
-    default: return resident_one<R, true, true, true>(A, J, threads, grid_cap, st);
+  if constexpr (SURF != 0) {  // (composed surfaces: bonds and walls by each system's own switches, fewer kernels to build)
+    return excl ? resident_one<R, true, true, true, SURF>(A, J, threads, grid_cap, st)
+                : resident_one<R, true, true, false, SURF>(A, J, threads, grid_cap, st);
+  } else {
+    const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
+    switch (key) {
+      case 0: return resident_one<R, false, false, false, SURF>(A, J, threads, grid_cap, st);
+      case 1: return resident_one<R, false, false, true, SURF>(A, J, threads, grid_cap, st);
+      case 2: return resident_one<R, false, true, false, SURF>(A, J, threads, grid_cap, st);
+      case 3: return resident_one<R, false, true, true, SURF>(A, J, threads, grid_cap, st);
+      case 4: return resident_one<R, true, false, false, SURF>(A, J, threads, grid_cap, st);
+      case 5: return resident_one<R, true, false, true, SURF>(A, J, threads, grid_cap, st);
+      case 6: return resident_one<R, true, true, false, SURF>(A, J, threads, grid_cap, st);
+      default: return resident_one<R, true, true, true, SURF>(A, J, threads, grid_cap, st);
+    }
   }
 }
 
@@ -3853,42 +3861,43 @@ cudaError_t launch_resident(const DevArrays& A, int precision, const ResidentJob
   if (J.nsys <= 0 || J.nsteps <= 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(J.next, 0, sizeof(uint32_t), st);
   if (e != cudaSuccess) return e;
-  return precision == 0 ? resident_dispatch<double>(A, J, bonds, walls, excl, threads, grid_cap, st)
-                        : resident_dispatch<float>(A, J, bonds, walls, excl, threads, grid_cap, st);
+  if (precision == 0) return resident_dispatch<double, 0>(A, J, bonds, walls, excl, threads, grid_cap, st);
+  if (A.composed & 1) return resident_dispatch<float, 3>(A, J, bonds, walls, excl, threads, grid_cap, st);
+  return A.composed ? resident_dispatch<float, 2>(A, J, bonds, walls, excl, threads, grid_cap, st)
+                    : resident_dispatch<float, 0>(A, J, bonds, walls, excl, threads, grid_cap, st);
 }
 
-int resident_blocks_per_sm(int precision, int bonds, int walls, int excl, uint32_t nmax, uint32_t tmax, int threads) {
-  const size_t smem = resident_smem_bytes(precision, nmax, tmax);
-  int per_sm = 0;
-  cudaError_t e;
-  const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
+template <typename R, int SURF>
+static cudaError_t resident_occupancy(int key, size_t smem, int threads, int* per_sm) {
   auto q = [&](auto kern) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, threads, smem);
   };
-  if (precision == 0) {
-    switch (key) {
-      case 0: e = q(k_resident<double, false, false, false>); break;
-      case 1: e = q(k_resident<double, false, false, true>); break;
-      case 2: e = q(k_resident<double, false, true, false>); break;
-      case 3: e = q(k_resident<double, false, true, true>); break;
-      case 4: e = q(k_resident<double, true, false, false>); break;
-      case 5: e = q(k_resident<double, true, false, true>); break;
-      case 6: e = q(k_resident<double, true, true, false>); break;
-      default: e = q(k_resident<double, true, true, true>); break;
-    }
+  if constexpr (SURF != 0) {
+    return key & 1 ? q(k_resident<R, true, true, true, SURF>) : q(k_resident<R, true, true, false, SURF>);
   } else {
     switch (key) {
-      case 0: e = q(k_resident<float, false, false, false>); break;
-      case 1: e = q(k_resident<float, false, false, true>); break;
-      case 2: e = q(k_resident<float, false, true, false>); break;
-      case 3: e = q(k_resident<float, false, true, true>); break;
-      case 4: e = q(k_resident<float, true, false, false>); break;
-      case 5: e = q(k_resident<float, true, false, true>); break;
-      case 6: e = q(k_resident<float, true, true, false>); break;
-      default: e = q(k_resident<float, true, true, true>); break;
+      case 0: return q(k_resident<R, false, false, false, SURF>);
+      case 1: return q(k_resident<R, false, false, true, SURF>);
+      case 2: return q(k_resident<R, false, true, false, SURF>);
+      case 3: return q(k_resident<R, false, true, true, SURF>);
+      case 4: return q(k_resident<R, true, false, false, SURF>);
+      case 5: return q(k_resident<R, true, false, true, SURF>);
+      case 6: return q(k_resident<R, true, true, false, SURF>);
+      default: return q(k_resident<R, true, true, true, SURF>);
     }
   }
+}
+
+int resident_blocks_per_sm(int precision, int bonds, int walls, int excl, int composed, uint32_t nmax, uint32_t tmax,
+                           int threads) {
+  const size_t smem = resident_smem_bytes(precision, nmax, tmax);
+  const int key = (bonds ? 4 : 0) | (walls ? 2 : 0) | (excl ? 1 : 0);
+  int per_sm = 0;
+  const cudaError_t e = precision == 0 ? resident_occupancy<double, 0>(key, smem, threads, &per_sm)
+                        : composed & 1 ? resident_occupancy<float, 3>(key, smem, threads, &per_sm)
+                        : composed     ? resident_occupancy<float, 2>(key, smem, threads, &per_sm)
+                                       : resident_occupancy<float, 0>(key, smem, threads, &per_sm);
   return e == cudaSuccess ? per_sm : 0;
 }
 

@@ -167,9 +167,9 @@ __device__ __forceinline__ DFPiece df_thyl_piece(const SysDev& S, DF C[3], DF T[
 }
 
 // What bounds it: instruction issue. The bump and the thylakoid went through
-// float64 before (two operations per SM and clock): 128 thylakoids of 2,500
-// particles 179 us per integrator launch (CUDA events), now 36; 100,000
-// particles on a bump and 900,000 free ones 74.5 us, now 62.7.
+// float64 before (two operations per SM and clock): the integrator launch of 128
+// thylakoids of 2,500 particles took 179 us (CUDA events) and takes 35, that of
+// 100,000 particles on a bump and 900,000 free ones 74.5 us and takes 51.
 //
 // Position half of a constrained particle: reads x^k, p^{k-1/2} (or p^k on the
 // first step) and the combined force F, returns x^{k+1} and p^{k+1/2}. y - c,
